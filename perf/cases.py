@@ -265,3 +265,84 @@ def tolerance(case):
     if case["weights"] == "f32":
         return {"rel": 7e-7, "max": 4e-6}
     return {"rel": 7e-3, "max": 4e-2}
+
+
+# ------------------------------------------------------------------------------------------------------------------
+def _exact_select(p, taken, alpha, params, k, resident):
+    """The eligible set of one block in 64 bits: Eq. 4 to 7 on probabilities `p` [n, E] and natural membership `taken`."""
+    E = p.shape[1]
+    u = (alpha[:, None] * p * taken).sum(0)
+    votes, anchor = taken.sum(0), taken[0]
+    rest = torch.where(anchor, 0.0, u)
+    positive = int((rest > 0).sum())
+    keep = max(0, k - int(anchor.sum()))
+    if positive:
+        q = rest[rest > 0] / rest.sum()
+        keep = max(keep, min(max(math.ceil(math.exp(float(-(q * q.log()).sum())) - params.ceil_guard), 1), positive))
+    order = sorted((e for e in range(E) if not anchor[e]), key=lambda e: (-float(u[e]), e))
+    S = anchor.clone()
+    S[order[:keep]] = True
+    if params.residency == 2:
+        S = (S & resident) | anchor
+    elif params.residency == 1:
+        budget, moved, size, removed = int(votes[~S].sum()), 0, int(S.sum()), []
+        for e in sorted((e for e in range(E) if S[e] and not resident[e]), key=lambda e: (float(u[e]), e)):
+            moved += int(votes[e])
+            if moved > budget or size - len(removed) - 1 < k or len(removed) == params.max_remove:
+                break
+            removed.append(e)
+        S[removed] = False
+    return S, u
+
+
+def _exact_weights(w, experts):
+    """expert -> (gate_up [2I, H], down [H, I]) in 64 bits"""
+    def mxfp4(codes, scales):
+        grid = torch.tensor(wl.E2M1_VALUES, dtype=torch.float64, device=codes.device)
+        value = grid[(codes & 7).long()] * torch.where(codes >= 8, -1.0, 1.0)
+        return value * torch.exp2(scales.double() - 127).repeat_interleave(32, -1)
+    if w["gate_up"] is None:
+        return lambda e: (mxfp4(w["gate_up_codes"][e], w["gate_up_scales"][e]), mxfp4(w["down_codes"][e], w["down_scales"][e]))
+    return lambda e: (w["gate_up"][e].double(), w["down"][e].double()) if e < experts else \
+        (w["shared_gate_up"][e - experts].double(), w["shared_down"][e - experts].double())
+
+
+def exact(case, seed):
+    """What `run` returns, in 64 bits throughout: routes are ranked on 64-bit logits, and the activation between the two
+    products is not rounded."""
+    cfg, dev, sizes = _config(case, seed), torch.device(DEVICE), _blocks(case)
+    E, k, T, params = cfg.n_experts, cfg.top_k, cfg.n_nodes, acm.SelectParams(residency=case["residency"])
+    table, alpha = wl.commitment_table(cfg).double(), []
+    for i, n in enumerate(sizes):
+        depth = wl.tree_depths(replace(cfg, n_nodes=n, index=cfg.index + 7919 * i)).long()
+        alpha.append((table[depth].sqrt() / torch.bincount(depth)[depth].double().sqrt()).float().double().to(dev))
+    results = []
+    for layer in range(cfg.n_layers):
+        w = wl.layer_weights_mxfp4(cfg, layer, dev) if case["weights"] == "mxfp4" else wl.layer_weights(cfg, layer, dev)
+        mask = wl.resident_mask(cfg, layer).tolist()
+        resident = torch.tensor([bool((mask[e // 32] >> (e % 32)) & 1) for e in range(E)])
+        x = wl.hidden_states(cfg, layer, dev).double()
+        z = x @ w["w_router"].double().T + (0 if w["router_bias"] is None else w["router_bias"].double())
+        p, natural = torch.softmax(z, 1), z.sort(dim=1, descending=True, stable=True).indices[:, :k]
+        taken = torch.zeros(T, E, dtype=torch.bool, device=dev).scatter_(1, natural, True)
+        eligible, demand, row = torch.ones(T, E, dtype=torch.bool, device=dev), None, 0
+        for n, a in zip(sizes, alpha) if case["call"] != "natural" else ():
+            S, demand = _exact_select(p[row:row + n].cpu(), taken[row:row + n].cpu(), a.cpu(), params, k, resident)
+            eligible[row:row + n] = S.to(dev)
+            row += n
+        zr = z.masked_fill(~eligible, float("-inf"))
+        top = zr.sort(dim=1, descending=True, stable=True)
+        zk, idx = top.values[:, :k], top.indices[:, :k]
+        wk = torch.softmax(zk, 1) if cfg.weighting == 0 else p.gather(1, idx) if cfg.weighting == 1 else torch.softmax(zr, 1).gather(1, idx)
+        wk = wk.masked_fill(zk == float("-inf"), 0.0)
+        weight = torch.zeros(T, E + cfg.n_shared, dtype=torch.float64, device=dev).scatter_(1, idx, wk)
+        weight[:, E:] = 1.0
+        out, expert = torch.zeros(T, cfg.hidden, dtype=torch.float64, device=dev), _exact_weights(w, E)
+        for e in weight.any(0).nonzero().flatten().tolist():
+            rows = weight[:, e].nonzero().flatten()
+            gate_up, down = expert(e)
+            g, up = (x[rows] @ gate_up.T).chunk(2, 1)
+            out[rows] += weight[rows, e, None] * ((torch.nn.functional.silu(g) * up) @ down.T)
+        results.append(out if case["call"] != "stages" else
+                       {"logits": z, "natural": None, "mask": None, "demand": demand.to(dev), "idx": None, "w": wk, "out": out})
+    return results
