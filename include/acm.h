@@ -370,6 +370,10 @@ acm_status acm_expert_ffn_f32_noalloc(const float* x, int T, int hidden, int int
 acm_status acm_ffn_plan(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,
                         int32_t* pieces /*host*/, int capacity, int32_t* n_pieces /*host*/, int32_t* n_segments /*host*/);
 
+/* The same for an MXFP4 layer (inter a multiple of 128): its kernel deals every tile whole. */
+acm_status acm_ffn_plan_mxfp4(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,
+                              int32_t* pieces /*host*/, int capacity, int32_t* n_pieces /*host*/, int32_t* n_segments /*host*/);
+
 /* How far the kernels of a fused call (acm_moe_verify, acm_moe_verify_batch, acm_moe_verify_host) overlap.
  * The stages of Section 3.1-3.4 form a chain, and the expert FFN needs only part of its result to start:
  *   ACM_OVERLAP_NONE       plain stream order.  The FFN kernel is a cooperative launch, so the driver itself
@@ -403,7 +407,7 @@ acm_status acm_set_wait_limit(acm_ctx* ctx, uint64_t nanoseconds);
  * Synchronises the device.  site_out [capacity] (host): 0 = that CTA saw no wait run out, -1 = that CTA never
  * started (it found no SM), else a wait-site number (1, 2: words published by the router / selection kernel;
  * 3-5: the CTA's own pipeline; 6-10: data from other CTAs; 11-16: hand-overs inside the CTA; 17: the rest of
- * the plan; 18: a packed MXFP4 stage).  *n_ctas = CTAs of that launch.  Call it before acm_device_status
+ * the plan; 18-22: MXFP4 layers: packed weights, activation pieces).  *n_ctas = CTAs of that launch.  Call it before acm_device_status
  * clears the state, or after: the words are kept until the next launch. */
 acm_status acm_wait_report(acm_ctx* ctx, int32_t* site_out /*host*/, int capacity, int32_t* n_ctas /*host*/);
 

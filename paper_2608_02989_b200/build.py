@@ -20,7 +20,7 @@ def _nvcc() -> str:
 
 
 def sources_mtime() -> float:
-    files = [CSRC / s for s in SOURCES] + [CSRC / "acm_internal.h", PKG.parent / "include" / "acm.h"]
+    files = [CSRC / s for s in SOURCES] + [CSRC / h for h in ("acm_internal.h", "ffn_plan.h", "mx_act.cuh")] + [PKG.parent / "include" / "acm.h"]
     return max(f.stat().st_mtime for f in files)
 
 

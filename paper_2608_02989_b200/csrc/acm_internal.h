@@ -52,6 +52,8 @@ struct Workspace {
   int32_t* ticket;      // [4] spare words (the MXFP4 scale check keeps its maximum in one)
   uint32_t* sel_words;  // [kMaxEarlyBlocks][8] the eligible masks as tagged 16-bit pieces (early start of the FFN kernel)
   unsigned long long* root_words;   // [kMaxEarlyBlocks][kMaxExperts] the roots' logits under the call's 32-bit tag (router kernel, see RootArgs)
+  unsigned char* xq;    // MXFP4 layers: the hidden states' pieces and scales (mx_act.cuh)
+  int32_t* xq_count;    // CTAs that have stored their part of them, over all calls (never cleared)
   uint32_t* anc_words;  // [kMaxEarlyBlocks][8] the anchor experts (each root's natural top-k) as tagged 16-bit pieces, published by the router kernel's root CTAs
 };
 
@@ -91,6 +93,15 @@ struct RootArgs {
   unsigned long long wait_limit_ns;
 };
 
+// MXFP4 layers: the hidden states as e4m3 pieces for the FFN kernel (mx_act.cuh), stored by CTAs of the router kernel (or
+// by launch_split_x); each of them adds one to *count when its part is stored.
+struct XqArgs {
+  unsigned char* xq;      // null: not wanted
+  int32_t* count;
+  int n_pad;
+  int rows;               // router kernel: rows of CTAs that do it
+};
+
 struct RouteArgs {
   const float* logits;
   const uint32_t* mask;
@@ -126,7 +137,13 @@ cudaError_t launch_router_logits(int dtype, const void* x, const void* w_router,
                                  float* logits, int T, int H, int E, float* zero_buf,
                                  size_t zero_floats, float* zero_buf2, size_t zero_floats2, int32_t* status,
                                  float* probs, int32_t* nat_idx, uint32_t* nat_mask, int k, int32_t* tile_done,
-                                 bool pdl, cudaStream_t s, long long* dbg = nullptr, const RootArgs* root = nullptr);
+                                 bool pdl, cudaStream_t s, long long* dbg = nullptr, const RootArgs* root = nullptr,
+                                 const XqArgs* xq = nullptr);
+// CTAs that add to XqArgs::count: split_x_rows rows of split_x_row_ctas in the router kernel, split_x_ctas in launch_split_x
+int split_x_rows(int T, int H, int E);
+int split_x_row_ctas(int E);
+int split_x_ctas(int T, int H);
+cudaError_t launch_split_x(const void* x, int T, int H, const XqArgs& xq, cudaStream_t s);
 cudaError_t launch_select(const SelectArgs& a, int T, int E, int k, cudaStream_t s);
 cudaError_t launch_route(const RouteArgs& a, int T, int E, int k, cudaStream_t s);
 // The fused calls' stages 1b-3 in ONE launch, a cluster of select_ctas_per_block(widest block) CTAs per block of `bd`
@@ -181,6 +198,9 @@ struct FfnLaunch {
   int32_t launch_tag = 0;         // launch number << 8
   const void* mx_gate_up = nullptr;   // MXFP4 layers (launch_ffn_mxfp4): the tiled code + scale tensors
   const void* mx_down = nullptr;
+  const void* xq = nullptr;             // MXFP4 layers: the hidden states' pieces (XqArgs), complete once
+  const int32_t* xq_count = nullptr;    // *xq_count has reached xq_target
+  int32_t xq_target = 0;
   unsigned long long* trace; // optional [grid][32] device time stamps (acm_stage_timing) or null
 };
 cudaError_t ffn_configure();   // one-time function attributes

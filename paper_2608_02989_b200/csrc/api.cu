@@ -9,6 +9,7 @@
 
 #include "acm_internal.h"
 #include "ffn_plan.h"
+#include "mx_act.cuh"
 
 using namespace acm;
 
@@ -98,8 +99,8 @@ bool plan_pool_block(int E, int n_slots, std::vector<int32_t>& slot_expert, std:
   return true;
 }
 
-// MXFP4 tile records: 128 x 64 code bytes, then 128 x 4 E8M0 scale bytes.  The FFN kernel applies a scale with one
-// bf16 multiply, which covers block scales up to 2 (scale byte 128); larger ones are refused at registration.
+// MXFP4 tile records: 128 x 64 code bytes, then 128 x 4 E8M0 scale bytes.  Block scales up to 2 (scale byte 128) are
+// taken; larger ones are refused at registration.
 constexpr size_t kMxRecordBytes = 128 * 64 + 128 * 4;
 constexpr int kMxMaxScaleByte = 128;
 __global__ void k_mx_max_scale(const unsigned char* tiles, size_t n_records, int* max_out) {
@@ -136,6 +137,7 @@ struct acm_ctx {
   std::vector<Layer> layers;
   EncodeTiledFn encode = nullptr;
   int32_t epoch = 0;
+  int32_t xq_target = 0;                 // what ws.xq_count reads once the latest call's hidden-state pieces are stored
   size_t frag_bytes = 0, flag_bytes = 0;   // fragment buffers and arrival counters (zero between launches)
   CUtensorMap h_map[2];
   CUtensorMap h_store_map[2];            // same buffers, one 64-feature tile per TMA store
@@ -393,6 +395,7 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
   if (pdl_ok && c->sm_count > 2 * routing_ctas) p.grid = c->sm_count - routing_ctas;
   c->last_ffn_grid = p.grid;
   if (L.mx) {
+    p.xq = c->ws.xq; p.xq_count = c->ws.xq_count; p.xq_target = c->xq_target;
     p.mx_gate_up = L.has_pool ? L.pool_gate_up : L.mx_gate_up;      // a pool: slot s of the pool tensors
     p.mx_down = L.has_pool ? L.pool_down : L.mx_down;
     ACM_CUDA(launch_ffn_mxfp4(p, maps, x_map, c->h_map[li], c->h_store_map[li], s));
@@ -402,6 +405,19 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
   c->launches += 1;
   if (e1) ACM_CUDA(cudaEventRecord(e1, s));
   return ACM_OK;
+}
+
+// MXFP4 layers: where the call's first kernel stores the hidden states' pieces (run_ffn_list uses the same padding).
+XqArgs xq_args(acm_ctx* c, int T) {
+  XqArgs xa;
+  xa.xq = c->ws.xq;
+  xa.count = c->ws.xq_count;
+  xa.n_pad = (T + 15) / 16 * 16;
+  xa.rows = split_x_rows(T, c->desc.hidden, c->desc.n_experts);
+  return xa;
+}
+void xq_expect(acm_ctx* c, int n_ctas) {
+  c->xq_target = static_cast<int32_t>(static_cast<uint32_t>(c->xq_target) + static_cast<uint32_t>(n_ctas));
 }
 
 // The sequence number of a fused call: its low 16 bits tag the words its kernels publish for one another (0 is
@@ -454,6 +470,51 @@ acm_status ensure_staging(acm_ctx* c) {
   return ACM_OK;
 }
 
+}  // namespace
+
+namespace {
+template <bool kUncut>
+acm_status list_plan(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid, int32_t* pieces,
+                     int capacity, int32_t* n_pieces, int32_t* n_segments) {
+  if (!pieces || !n_pieces || !n_segments || capacity < 0) return ACM_ERR_INVALID;
+  if (n_experts_streamed < 1 || n_experts_streamed > kMaxSlots || n_anchor_first < 0 || n_anchor_first > n_experts_streamed ||
+      hidden < 128 || hidden % 128 != 0 || inter < 64 || inter % 64 != 0 || grid < 1 || grid > 1024)
+    return ACM_ERR_INVALID;
+  using namespace acm::plan;
+  const int tpe = inter / 64, kc1 = hidden / 128, kpe = (tpe + 1) / 2, h_tiles = hidden / 128;
+  if (n_anchor_first * tpe > grid) return ACM_ERR_INVALID;      // the pre-segment gives a CTA at most one tile
+  const FastDiv d_grid = make_fastdiv(grid), d_kc1 = make_fastdiv(kc1), d_tpe = make_fastdiv(tpe);
+  int n = 0, n_seg = 0;
+  for (int cta = 0; cta < grid; ++cta) {
+    Plan pl = {};
+    int base = 0;
+    if (n_anchor_first > 0) {
+      const Segment sg0 = Segment{1, 1, 0, n_anchor_first * tpe, 0, 0, 0, d_kc1, 0};
+      pl.seg[0] = sg0;
+      pl.range[0] = make_range(sg0, cta, d_grid, h_tiles);
+      base = 1;
+    }
+    for (int lane = 3; lane >= 0; --lane)
+      plan_lane<kUncut>(pl, lane, cta, n_experts_streamed, tpe, grid, d_kc1, kpe, d_grid, d_tpe, h_tiles, n_anchor_first, base);
+    n_seg = pl.n_seg;
+    for (int si = 0; si < pl.n_seg; ++si) {
+      const Segment& sg = pl.seg[si];
+      Sched sc(pl.range[si]);
+      int t, k0, k1;
+      while (sc.next(t, k0, k1)) {
+        if (n < capacity) {
+          int32_t* q = pieces + static_cast<size_t>(8) * n;
+          q[0] = cta; q[1] = si; q[2] = sg.phase; q[3] = sg.phase == 1 ? sg.whole : 0;
+          q[4] = sg.phase == 1 ? sg.t0 + t : t; q[5] = k0; q[6] = k1; q[7] = sg.phase == 1 ? sg.p1_index : sg.a0;
+        }
+        ++n;
+      }
+    }
+  }
+  *n_pieces = n;
+  *n_segments = n_seg;
+  return n <= capacity ? ACM_OK : ACM_ERR_NOMEM;
+}
 }  // namespace
 
 extern "C" {
@@ -537,6 +598,8 @@ acm_status acm_create(const acm_model_desc* desc, acm_ctx** out) {
   const size_t o_selw = carve(32 * kMaxEarlyBlocks);
   const size_t o_ancw = carve(32 * kMaxEarlyBlocks);
   const size_t o_rootw = carve(sizeof(unsigned long long) * kMaxExperts * kMaxEarlyBlocks);
+  const size_t o_xq = carve(desc->dtype == ACM_BF16 ? mx_act_bytes(desc->hidden) : 0);
+  const size_t o_xqc = carve(16);
   const size_t o_res = carve(sizeof(uint32_t) * 4 * desc->n_layers);
   const size_t o_diag = carve(sizeof(int32_t) * c->sm_count);
   if (cudaMalloc(&c->ws_base, off) != cudaSuccess) return fail(ACM_ERR_NOMEM);
@@ -566,6 +629,8 @@ acm_status acm_create(const acm_model_desc* desc, acm_ctx** out) {
   c->ws.sel_words = reinterpret_cast<uint32_t*>(b + o_selw);
   c->ws.anc_words = reinterpret_cast<uint32_t*>(b + o_ancw);
   c->ws.root_words = reinterpret_cast<unsigned long long*>(b + o_rootw);
+  c->ws.xq = reinterpret_cast<unsigned char*>(b + o_xq);
+  c->ws.xq_count = reinterpret_cast<int32_t*>(b + o_xqc);
   c->resident_dev = reinterpret_cast<uint32_t*>(b + o_res);
   c->wait_diag = reinterpret_cast<int32_t*>(b + o_diag);
   *out = c;
@@ -760,6 +825,11 @@ acm_status acm_expert_ffn(acm_ctx* c, int layer, const void* x, int T, const int
   ACM_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * static_cast<size_t>(T) * d.hidden, s));
   ACM_CUDA(launch_routes_to_table(idx, w, c->ws.act_mask, c->ws.wtab, c->ws.ready, T, d.n_experts, d.top_k, s));
   c->launches += 1;
+  if (L.mx) {
+    ACM_CUDA(launch_split_x(x, T, d.hidden, xq_args(c, T), s));
+    xq_expect(c, split_x_ctas(T, d.hidden));
+    c->launches += 1;
+  }
   return run_ffn_list(c, L, x, T, 0, out, s);
 }
 
@@ -817,11 +887,13 @@ acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const flo
   root.anc_words = c->ws.anc_words;
   root.anc_tag = static_cast<uint32_t>(early_epoch) & 0xffffu;
   root.wait_limit_ns = c->wait_limit_ns;
+  const XqArgs xa = xq_args(c, T);
   ACM_CUDA(launch_router_logits(d.dtype, x, L.w_router, L.bias, c->ws.logits, T, d.hidden, E, f32 ? nullptr : out,
                                 f32 ? 0 : static_cast<size_t>(T) * d.hidden, c->ws.wtab, c->ffn_in_floats,
                                 c->ws.status, nullptr, nullptr, nullptr, k, nullptr, c->pdl, s,
                                 c->trace ? reinterpret_cast<long long*>(c->trace) + 32 * c->sm_count : nullptr,
-                                early ? &root : nullptr));
+                                early ? &root : nullptr, L.mx ? &xa : nullptr));
+  if (L.mx) xq_expect(c, xa.rows * split_x_row_ctas(E));
   // stages 1b-3: one cluster of CTAs, which also fills the FFN kernel's routing inputs
   SelectArgs sa;
   sa.probs = nullptr; sa.nat_idx = nullptr; sa.alpha = alpha; sa.anchor_nodes = nullptr;   // (the fused kernel keeps both on chip)
@@ -1025,9 +1097,12 @@ acm_status acm_moe_verify_batch(acm_ctx* c, int layer, const void* x, int n_bloc
   root.anc_words = c->ws.anc_words;
   root.anc_tag = static_cast<uint32_t>(early_epoch) & 0xffffu;
   root.wait_limit_ns = c->wait_limit_ns;
+  const XqArgs xa = xq_args(c, T);
   ACM_CUDA(launch_router_logits(d.dtype, x, L.w_router, L.bias, c->ws.logits, T, d.hidden, E, out,
                                 static_cast<size_t>(T) * d.hidden, c->ws.wtab, c->ffn_in_floats, c->ws.status,
-                                nullptr, nullptr, nullptr, k, nullptr, c->pdl, s, nullptr, early ? &root : nullptr));
+                                nullptr, nullptr, nullptr, k, nullptr, c->pdl, s, nullptr, early ? &root : nullptr,
+                                L.mx ? &xa : nullptr));
+  if (L.mx) xq_expect(c, xa.rows * split_x_row_ctas(E));
   // stages 1b-3: one cluster of CTAs per block
   SelectArgs sa;
   sa.probs = nullptr; sa.nat_idx = nullptr; sa.alpha = alpha; sa.anchor_nodes = nullptr;   // (the fused kernel keeps both on chip)
@@ -1406,44 +1481,13 @@ acm_status acm_launch_count(acm_ctx* c, uint64_t* launches_out) {
 
 acm_status acm_ffn_plan(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid, int32_t* pieces,
                         int capacity, int32_t* n_pieces, int32_t* n_segments) {
-  if (!pieces || !n_pieces || !n_segments || capacity < 0) return ACM_ERR_INVALID;
-  if (n_experts_streamed < 1 || n_experts_streamed > kMaxSlots || n_anchor_first < 0 || n_anchor_first > n_experts_streamed ||
-      hidden < 128 || hidden % 128 != 0 || inter < 64 || inter % 64 != 0 || grid < 1 || grid > 1024)
-    return ACM_ERR_INVALID;
-  using namespace acm::plan;
-  const int tpe = inter / 64, kc1 = hidden / 128, kpe = (tpe + 1) / 2, h_tiles = hidden / 128;
-  if (n_anchor_first * tpe > grid) return ACM_ERR_INVALID;      // the pre-segment gives a CTA at most one tile
-  const FastDiv d_grid = make_fastdiv(grid), d_kc1 = make_fastdiv(kc1), d_tpe = make_fastdiv(tpe);
-  int n = 0, n_seg = 0;
-  for (int cta = 0; cta < grid; ++cta) {
-    Plan pl = {};
-    int base = 0;
-    if (n_anchor_first > 0) {
-      const Segment sg0 = Segment{1, 1, 0, n_anchor_first * tpe, 0, 0, 0, d_kc1, 0};
-      pl.seg[0] = sg0;
-      pl.range[0] = make_range(sg0, cta, d_grid, h_tiles);
-      base = 1;
-    }
-    for (int lane = 3; lane >= 0; --lane)
-      plan_lane(pl, lane, cta, n_experts_streamed, tpe, grid, d_kc1, kpe, d_grid, d_tpe, h_tiles, n_anchor_first, base);
-    n_seg = pl.n_seg;
-    for (int si = 0; si < pl.n_seg; ++si) {
-      const Segment& sg = pl.seg[si];
-      Sched sc(pl.range[si]);
-      int t, k0, k1;
-      while (sc.next(t, k0, k1)) {
-        if (n < capacity) {
-          int32_t* q = pieces + static_cast<size_t>(8) * n;
-          q[0] = cta; q[1] = si; q[2] = sg.phase; q[3] = sg.phase == 1 ? sg.whole : 0;
-          q[4] = sg.phase == 1 ? sg.t0 + t : t; q[5] = k0; q[6] = k1; q[7] = sg.phase == 1 ? sg.p1_index : sg.a0;
-        }
-        ++n;
-      }
-    }
-  }
-  *n_pieces = n;
-  *n_segments = n_seg;
-  return n <= capacity ? ACM_OK : ACM_ERR_NOMEM;
+  return list_plan<false>(n_experts_streamed, n_anchor_first, hidden, inter, grid, pieces, capacity, n_pieces, n_segments);
+}
+
+acm_status acm_ffn_plan_mxfp4(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid, int32_t* pieces,
+                              int capacity, int32_t* n_pieces, int32_t* n_segments) {
+  if (inter % 128 != 0) return ACM_ERR_INVALID;
+  return list_plan<true>(n_experts_streamed, n_anchor_first, hidden, inter, grid, pieces, capacity, n_pieces, n_segments);
 }
 
 acm_status acm_set_overlap(acm_ctx* c, int level) {

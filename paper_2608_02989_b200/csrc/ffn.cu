@@ -32,6 +32,7 @@
 
 #include "acm_internal.h"
 #include "ffn_plan.h"
+#include "mx_act.cuh"
 
 namespace acm {
 namespace {
@@ -40,7 +41,7 @@ namespace {
 #define ACM_FFN_MX 0
 #endif
 constexpr int kMaxStages = 3;                            // pipeline stages of the weight ring (see Geo)
-constexpr int kAcc = 4;                                  // TMEM accumulators in flight (power of two)
+constexpr int kAcc = ACM_FFN_MX ? 3 : 4;                 // TMEM accumulators in flight
 constexpr int kBK = 64;                                  // K elements of one 128-byte swizzle atom
 constexpr int kAtoms = 2;                                // atoms per pipeline stage: a stage covers 128 K
 constexpr int kTileM = 128;
@@ -49,18 +50,39 @@ constexpr int kABytes = kAtoms * kAtomABytes;            // 32 KB weight tile, o
 // The epilogue handles node columns kMaxNodes = 64 at a time: one fragment, one activation tile.  A wide tile (a
 // batch of blocks with more than 64 nodes in all, up to kWideNodes = 128 accumulator columns) goes in two halves.
 constexpr int kOutStageBytes = kTileM * kMaxNodes * 4;   // 32 KB: outgoing fragment (also the gate/up exchange buffer)
-constexpr int kHStageBytes = kMaxNodes * 64 * 2;         // 8 KB: one finished activation tile (64 features x 64 nodes)
-constexpr int kMxACols = 64;                             // MXFP4: one expanded weight stage in tensor memory = 128 K bf16 per row
-static_assert(kAcc * kMaxNodes + kMaxStages * kMxACols <= 512, "tensor memory: accumulators + expanded weight stages");
-// ACM_FFN_MX = 1 (set by ffn_mx.cu, which includes this file) builds the same kernel for MXFP4 expert
-// weights: a pipeline stage of a weight tile arrives as 128 rows x 64 bytes of E2M1 codes + 128 x 4 E8M0
-// scale bytes (one contiguous 8704-byte copy into the stage's weight area), and four more warps expand it
-// there to the 32 KB bf16 tile the MMAs read -- every MXFP4 value is a bf16, so the arithmetic is the
-// bf16 path's.
-constexpr int kThreads = ACM_FFN_MX ? 384 : 256;         // producer, MMA, 4 epilogue warps, helper, publisher (+ 4 expanding warps)
-constexpr int kMxCodeBytes = kTileM * 64;                // 128 rows x 128 four-bit codes
+// One finished activation tile (64 features x 64 nodes): 8 KB of bf16, or -- the same 8 KB -- two e4m3 pieces per
+// element plus their 512 bytes of scales (MXFP4, see below).
+constexpr int kHStages = ACM_FFN_MX ? 1 : 2;             // of them in shared memory
+constexpr int kHStageBytes = kMaxNodes * 64 * 2 + (ACM_FFN_MX ? kMxActScaleBytes : 0);
+// ACM_FFN_MX = 1 (set by ffn_mx.cu, which includes this file) builds the same kernel for MXFP4 expert weights on the
+// block-scaled tensor-core instruction (tcgen05.mma kind::mxf8f6f4: 8-bit operands, an E8M0 scale per row and 32 K).
+//   Weights.  A pipeline stage of a tile is one contiguous 8704-byte record (128 rows x 64 bytes of E2M1 codes, 128 x 4
+//   scale bytes).  Eight unpacking warps give every code a byte of its own -- two bits up, it is the same value as an
+//   e2m3: sign | 2 exponent bits | 3 mantissa bits, of which the lower two are zero -- four instructions for eight codes
+//   (an e4m3 would take seven), and store them in tensor memory, from where the MMAs take their A operand.  (4-bit
+//   operands as they are would do without the moves, but have to lie in shared memory, 16 bytes for 16 codes: written
+//   there and read again by the MMAs they made shared-memory bandwidth the bound, 670 of 720 clocks a stage.)
+//   Activations.  A bf16 has 8 significand bits, an e4m3 four: x = a + b, a = e4m3(x / s), b = e4m3 of the rest, with
+//   s a power of two per node and 32 K that puts the largest |x| into [128, 256) and b scaled by 2^-4 s.  The split is
+//   exact for every |x| >= 2^-14 of that maximum, and off by at most 2^-22 of the maximum below (an fp32 accumulator
+//   of such products rounds at 2^-24).  The pieces are node columns of their own -- a in columns [0, n_pad), b in
+//   [n_pad, 2 n_pad) of ONE accumulator, added when it is read -- because an instruction costs little more for them
+//   (64 clocks at 128 columns, 44 at 32; K = 32 each, so four a stage where bf16 took eight of 75).  What the two-piece
+//   product loses against 64 bits: 6.4e-8 (2-norm) over K = 4096, a serial fp32 sum of the unsplit one: 1.2e-7.
+//   The features are stored in the order the moves leave the weights in (mx_act.cuh).
+constexpr int kThreads = ACM_FFN_MX ? 512 : 256;         // producer, MMA, 4 epilogue warps, helper, publisher (+ 2 x 4 unpacking warps)
+[[maybe_unused]] constexpr int kMxCodeBytes = kTileM * 64;                // 128 rows x 128 four-bit codes
 [[maybe_unused]] constexpr int kMxStageBytes = kMxCodeBytes + kTileM * 4; // + one scale byte per row and 32 K
-constexpr int kFragBytes = kTileM * kMaxNodes * 4;       // contributor fragments pre-summed in shared memory
+[[maybe_unused]] constexpr int kMxACols = 32;                             // an unpacked stage in tensor memory: 4 weights a column
+[[maybe_unused]] constexpr int kMxScaleCols = 8;                          // its scales: 4 columns the weights', 4 the activations'
+[[maybe_unused]] constexpr int kMxA = 3;                                  // such stages in flight
+static_assert(!ACM_FFN_MX || kAcc * 2 * kMaxNodes + kMxA * (kMxACols + kMxScaleCols) <= 512, "tensor memory: accumulators + unpacked stages");
+// Shared-memory rings of the MXFP4 kernel: activation pieces and packed records.  Both are 1.5 us from request to arrival
+// under load, from L2 and from HBM; they share the space, an activation stage being 256 n_pad bytes: 7 of either beside
+// 64 node columns, 10 and 12 beside 16 (mx_rings).
+[[maybe_unused]] constexpr int kMaxRaw = 12, kMaxAct = 10;
+[[maybe_unused]] constexpr int kMxRingBytes = 181 * 1024;
+constexpr int kFragBytes = ACM_FFN_MX ? 0 : kTileM * kMaxNodes * 4;   // contributor fragments pre-summed in shared memory (MXFP4: no cut tiles)
 constexpr int kFragFloats = kTileM * kMaxNodes;
 
 using plan::FastDiv;
@@ -96,7 +118,11 @@ enum WaitSite : int {
   kSiteFragFull = 15,       // epilogue: the summed fragments of a cut tile
   kSiteActFree = 16,        // epilogue: an activation staging buffer
   kSitePlanReady = 17,      // any role: the rest of the plan (anchor start)
-  kSitePackedStage = 18     // MXFP4 expanding warps: the packed weight stage
+  kSitePackedStage = 18,    // MXFP4 unpacking warps: the packed weight stage
+  kSitePackedFree = 19,     // MXFP4 weight producer: a record slot the unpacking warps have not read
+  kSiteActStage = 20,       // MXFP4 unpacking warps: the stage's activations
+  kSiteActSlot = 21,        // MXFP4 activation producer: a stage the MMAs have not released
+  kSiteXPieces = 22         // MXFP4 activation producer: the hidden states' pieces
 };
 struct GiveUp {
   volatile int flag;             // set once this CTA has given up: every role then leaves at its next slow path
@@ -119,7 +145,8 @@ struct __align__(8) BarriersT {
   unsigned long long ost_full, ost_free;   // epilogue <-> publisher: outgoing fragment staged / copied out
   unsigned long long hst_full[2], hst_free[2];   // epilogue <-> publisher: activation tile staged / stored
 #if ACM_FFN_MX
-  unsigned long long raw[kMaxStages];   // the packed weight stage has landed (producer's copy -> expanding warps)
+  unsigned long long raw[kMaxRaw], raw_empty[kMaxRaw];   // packed records: landed (-> unpacking warps) / read (-> producer)
+  unsigned long long act[kMaxAct], act_empty[kMaxAct];   // activation stages: landed / multiplied (-> activation producer)
 #endif
   volatile uint32_t armed;           // stages whose barrier the weight producer has armed so far
   volatile int32_t n_routed_slots;   // routed experts in this launch's work list (known with the complete list)
@@ -141,9 +168,10 @@ struct Geo {
   static constexpr int kStages = kN > kMaxNodes ? 2 : 3;
   static constexpr int kBBytes = kAtoms * kN * kBK * 2;          // activation chunk of a stage, one TMA copy
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kTmemCols = ACM_FFN_MX ? 512 : kAcc * kN;    // MXFP4: accumulators, then the expanded weight stages
+  static constexpr int kTmemCols = ACM_FFN_MX ? 512 : kAcc * kN;    // MXFP4: two-piece accumulators, then the scales
+  static constexpr int kRingBytes = ACM_FFN_MX ? kMxRingBytes : kStages * kStageBytes;
   static constexpr size_t kSmemBytes =
-      1024 + static_cast<size_t>(kStages) * kStageBytes + kOutStageBytes + kFragBytes + 2 * kHStageBytes + sizeof(BarriersT<kN>);
+      1024 + static_cast<size_t>(kRingBytes) + kOutStageBytes + kFragBytes + kHStages * kHStageBytes + sizeof(BarriersT<kN>);
   static_assert(kSmemBytes <= 232448, "shared memory: ring + staging buffers + control block exceed 227 KB");
   static_assert(kStages <= kMaxStages, "barrier arrays");
 };
@@ -235,6 +263,22 @@ __device__ bool flag_wait_ge(const int32_t* p, int target, GiveUp* g, int site) 
     }
   }
 }
+#if ACM_FFN_MX
+// Bounded wait until a running count (it never goes back; it may wrap) has reached `target`.
+__device__ bool count_wait(const int32_t* p, int32_t target, GiveUp* g, int site) {
+  auto reached = [&]() { return static_cast<int32_t>(static_cast<uint32_t>(ld_acquire(p)) - static_cast<uint32_t>(target)) >= 0; };
+  if (reached()) return true;
+  const unsigned long long t0 = global_timer();
+  for (;;) {
+    if (reached()) return true;
+    if (g->flag) return false;
+    if (limit_passed(t0, g->limit_ns)) {
+      give_up(g, site);
+      return false;
+    }
+  }
+}
+#endif
 // Bounded poll of one self-validating word (16 payload bits under a 16-bit tag) written by an earlier kernel
 // of the same stream: returns the payload, or sets `seen` to false when the limit ran out.
 __device__ __forceinline__ uint32_t poll_tagged_word(const uint32_t* word, uint32_t tag, unsigned long long limit_ns, bool& seen) {
@@ -254,6 +298,11 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 __device__ __forceinline__ void bulk_load_hint(uint32_t smem_dst, const void* gmem_src, uint32_t bytes, uint32_t bar, uint64_t policy) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
                ::"r"(smem_dst), "l"(gmem_src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
+}
+#endif
+#if ACM_FFN_MX
+__device__ __forceinline__ void bulk_store(void* gmem_dst, uint32_t smem_src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gmem_dst), "r"(smem_src), "r"(bytes) : "memory");
 }
 #endif
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
@@ -349,20 +398,44 @@ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t smem_addr) {
   return d;
 }
 #if ACM_FFN_MX
-// The same MMA with the A operand (128 rows x 16 K bf16) in tensor memory: row = lane, two K elements per column.
-__device__ __forceinline__ void umma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc,
-                                             uint32_t accumulate) {
+// Block-scaled MMA over 32 K: unpacked weights (128 rows, e2m3, in tensor memory: row = lane, four K a column) x e4m3
+// activation pieces (K-major in shared memory), with their E8M0 scales in tensor memory (row or column j: lane j % 32 of
+// every quarter, column j / 32).
+__device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate,
+                                        uint32_t tmem_sfa, uint32_t tmem_sfb) {
   asm volatile(
       "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}\n"
-      ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate) : "memory");
+      "tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], [%1], %2, %3, [%5], [%6], p;\n\t}\n"
+      ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(tmem_sfa), "r"(tmem_sfb) : "memory");
 }
-// 16 consecutive columns of this thread's lane
-__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t* v) {
+// Its instruction descriptor: A = E2M3, B = E4M3, E8M0 scales, fp32 accumulator, M = 128, N = n (bits 29, 30 and 4, 5: which
+// byte of the scales' words).
+__device__ __forceinline__ uint32_t umma_mx_idesc(int n) {
+  return (3u << 7) | (static_cast<uint32_t>(n >> 3) << 17) | (1u << 23) | (static_cast<uint32_t>(kTileM >> 7) << 27);
+}
+// One lane of a converged warp (always the same one).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+  return r != 0;
+}
+// Descriptor of an activation half-stage: rows of 64 bytes (64 K e4m3), 64-byte swizzle, groups of 8 rows 512 bytes apart.
+__device__ __forceinline__ uint64_t umma_smem_desc_64(uint32_t smem_addr) {
+  return static_cast<uint64_t>((smem_addr & 0x3ffffu) >> 4) | (static_cast<uint64_t>(1) << 16) |
+         (static_cast<uint64_t>(512 >> 4) << 32) | (static_cast<uint64_t>(1) << 46) | (static_cast<uint64_t>(4) << 61);
+}
+// 4 consecutive columns of this thread's lane
+__device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
   asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};"
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};"
       ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(v[8]),
-        "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+        "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(v[16]), "r"(v[17]),
+        "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]), "r"(v[24]), "r"(v[25]), "r"(v[26]),
+        "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 #endif
@@ -401,6 +474,13 @@ struct FfnArgs {
 #if ACM_FFN_MX
   const unsigned char* mx_gate_up;   // [E][I/64][H/128][8704]
   const unsigned char* mx_down;      // [E][H/128][I/128][8704]
+  const unsigned char* xq;           // hidden states in pieces: [H/64][2 n_pad][64], 64-byte swizzled
+  const unsigned char* xq_scale;     // [H/64][512] (mx_scale_at)
+  unsigned char* hq;                 // activations alike: [slot][I/64][2 n_pad][64]
+  unsigned char* hq_scale;           // [slot][I/64][512]
+  const int32_t* xq_count;           // CTAs that have stored their part of the pieces, over all calls of the context
+  int32_t xq_target;                 // ... and what it reads once this call's are complete
+  int n_raw, n_act;                  // depths of the rings of packed records and activation stages
 #endif
 };
 
@@ -424,17 +504,31 @@ __global__ void __launch_bounds__(kThreads, 1)
 ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUtensorMap x_map,
            const __grid_constant__ CUtensorMap h_map, const __grid_constant__ CUtensorMap hs_map,
            const FfnArgs p) {
-  constexpr int kStages = Geo<kN>::kStages, kStageBytes = Geo<kN>::kStageBytes, kAccCols = kN, kTmemCols = Geo<kN>::kTmemCols;
+  constexpr int kStages = Geo<kN>::kStages, kAccCols = ACM_FFN_MX ? 2 * kN : kN, kTmemCols = Geo<kN>::kTmemCols;
+#if !ACM_FFN_MX
+  constexpr int kStageBytes = Geo<kN>::kStageBytes;
+#endif
   using Barriers = BarriersT<kN>;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+#if !ACM_FFN_MX
   unsigned char* stage_base = smem;
-  unsigned char* after_ring = smem + static_cast<size_t>(kStages) * kStageBytes;
+#endif
+  unsigned char* after_ring = smem + static_cast<size_t>(Geo<kN>::kRingBytes);
+#if ACM_FFN_MX
+  // the ring area: activation pieces, their scales, packed records
+  const int act_bytes = p.n_pad * 256;
+  unsigned char* act_base = smem;
+  unsigned char* act_scale_base = act_base + p.n_act * act_bytes;
+  unsigned char* raw_base = act_scale_base + p.n_act * 2 * kMxActScaleBytes;
+#endif
   float* ostage = reinterpret_cast<float*>(after_ring);           // outgoing fragment [node][128 rows]
+#if !ACM_FFN_MX
   float* ex = ostage;                                             // gate/up exchange aliases it (never used at once)
   float* sfrag = reinterpret_cast<float*>(after_ring + kOutStageBytes);
+#endif
   unsigned char* hstage = after_ring + kOutStageBytes + kFragBytes;   // 2 x [node][64 features] bf16, swizzled
-  Barriers* bars = reinterpret_cast<Barriers*>(after_ring + kOutStageBytes + kFragBytes + 2 * kHStageBytes);
+  Barriers* bars = reinterpret_cast<Barriers*>(after_ring + kOutStageBytes + kFragBytes + kHStages * kHStageBytes);
   GiveUp* const quit = &bars->give_up;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -442,12 +536,19 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   griddep_launch_dependents();
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(smem_u32(&bars->full[s]), ACM_FFN_MX ? 5 : 1);   // MXFP4: + one arrival per expanding warp
+      mbar_init(smem_u32(&bars->full[s]), ACM_FFN_MX ? 4 : 1);   // MXFP4: one arrival per unpacking warp
       mbar_init(smem_u32(&bars->empty[s]), 1);
-#if ACM_FFN_MX
-      mbar_init(smem_u32(&bars->raw[s]), 1);
-#endif
     }
+#if ACM_FFN_MX
+    for (int s = 0; s < p.n_raw; ++s) {
+      mbar_init(smem_u32(&bars->raw[s]), 1);
+      mbar_init(smem_u32(&bars->raw_empty[s]), 4);
+    }
+    for (int s = 0; s < p.n_act; ++s) {
+      mbar_init(smem_u32(&bars->act[s]), 1);
+      mbar_init(smem_u32(&bars->act_empty[s]), 1);
+    }
+#endif
     for (int b = 0; b < kAcc; ++b) {
       mbar_init(smem_u32(&bars->tfull[b]), 1);
       mbar_init(smem_u32(&bars->tempty[b]), 128);
@@ -476,9 +577,9 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #if !ACM_FFN_MX
     prefetch_tensormap(&maps.gate_up);
     prefetch_tensormap(&maps.down);
-#endif
     prefetch_tensormap(&x_map);
     prefetch_tensormap(&h_map);
+#endif
   }
   if (warp == 1) {
     tmem_alloc(smem_u32(&bars->tmem_base), kTmemCols);
@@ -561,19 +662,21 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   const int kc1 = p.H / (kBK * kAtoms);   // K-chunks (stages) of a gate/up tile
   const int kpe = (tpe + kAtoms - 1) / kAtoms;   // K-chunks (stages) per expert in the down phase
   const int h_tiles = p.H / kTileM;  // output tiles of the down phase
+#if !ACM_FFN_MX
   const uint32_t b_atom_bytes = static_cast<uint32_t>(p.n_pad) * kBK * 2;   // one atom of the activation chunk
   const uint32_t b_bytes = kAtoms * b_atom_bytes;
+#endif
   if (pre) {
-    if (threadIdx.x == kThreads - 32) {            // segment 0: the pre-streamed experts' tiles, one whole tile per CTA
+    if (threadIdx.x == 7 * 32) {            // segment 0: the pre-streamed experts' tiles, one whole tile per CTA
       Segment sg0 = Segment{1, 1, 0, n_pre * tpe, 0, 0, 0, p.d_kc1, 0};
       bars->plan.seg[0] = sg0;
       bars->plan.range[0] = make_range(sg0, cta, p.d_grid, h_tiles);
       bars->plan.n_pre = n_pre;
       bars->plan.n_seg = 1;
     }
-  } else if (warp == kThreads / 32 - 1 && lane < 4) {      // (the publisher warp has nothing else to do yet)
+  } else if (warp == 7 && lane < 4) {      // (the publisher warp has nothing else to do yet)
     if (lane == 0) bars->n_routed_slots = n_routed;
-    plan_lane(bars->plan, lane, cta, n_act, tpe, G, p.d_kc1, kpe, p.d_grid, p.d_tpe, h_tiles);
+    plan_lane<ACM_FFN_MX>(bars->plan, lane, cta, n_act, tpe, G, p.d_kc1, kpe, p.d_grid, p.d_tpe, h_tiles);
   }
   int32_t* s_entry = bars->entry;
   if (threadIdx.x < kMaxExperts) {
@@ -612,6 +715,75 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     }
   };
 
+  // The rest of the plan behind the anchors' pre-segment, by a warp that has nothing to do before it is there: the bf16
+  // helper, the MXFP4 publisher (no tile is finalised before the routing kernel has completed).
+  auto complete_plan = [&]() -> bool {
+    // While the others run the anchors' pre-segment: wait for the eligible set, give the other experts the
+    // slots behind the pre-streamed ones (ascending id), append the shared experts, work out the rest of the
+    // plan, and let everyone on.
+    // eight words per block; lane l takes words l and l + 32 (blocks 0-3 and 4-7), the union goes to lanes 0..7
+    bool seen = true;
+    uint32_t half = 0u;
+    {
+      const uint32_t tag = static_cast<uint32_t>(p.sel_epoch) & 0xffffu;
+      const int n_words = 2 * kMaskWords * p.sel_blocks;
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        const int j = lane + 32 * part;
+        if (j < n_words) {
+          bool got = true;
+          half |= poll_tagged_word(p.sel_flag + j, tag, p.wait_limit_ns, got);
+          seen = seen && got;
+        }
+      }
+      half |= __shfl_xor_sync(0xffffffffu, half, 8);
+      half |= __shfl_xor_sync(0xffffffffu, half, 16);
+    }
+    const bool good = __all_sync(0xffffffffu, seen);
+    uint32_t rest[kMaskWords];
+    int n_rest = 0;
+#pragma unroll
+    for (int wd = 0; wd < kMaskWords; ++wd) {
+      const uint32_t lo = __shfl_sync(0xffffffffu, half, 2 * wd), hi = __shfl_sync(0xffffffffu, half, 2 * wd + 1);
+      rest[wd] = ((lo | (hi << 16)) & p.only[wd]) & ~am[wd];
+      n_rest += __popc(rest[wd]);
+    }
+    if (good) {
+      for (int e = lane; e < kMaxExperts; e += 32) {
+        const int wd = e >> 5;
+        const uint32_t mine = wd == 0 ? rest[0] : wd == 1 ? rest[1] : wd == 2 ? rest[2] : rest[3];
+        if ((mine >> (e & 31)) & 1u) {
+          int slot = n_pre + __popc(mine & ((1u << (e & 31)) - 1u));
+#pragma unroll
+          for (int w2 = 0; w2 < kMaskWords; ++w2) slot += w2 < wd ? __popc(rest[w2]) : 0;
+          s_entry[slot] = make_entry(kSrcRouted, e);
+          bars->expert[slot] = e;
+        }
+      }
+      if (lane < p.n_shared) {
+        s_entry[n_pre + n_rest + lane] = make_entry(kSrcShared, lane);
+        bars->expert[n_pre + n_rest + lane] = -1;
+      }
+      if (lane == 0) bars->n_routed_slots = n_pre + n_rest;
+      if (lane < 4)
+        plan_lane<ACM_FFN_MX>(bars->plan, lane, cta, n_pre + n_rest + p.n_shared, tpe, G, p.d_kc1, kpe, p.d_grid, p.d_tpe, h_tiles,
+                  n_pre, 1);
+    } else if (lane == 0) {
+      give_up(quit, kSiteEligibleWords);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      mbar_arrive(smem_u32(&bars->plan_ready));
+    }
+    return good;
+  };
+#if ACM_FFN_MX
+  // The CTAs walk the K-chunks of their (whole) tiles from different ones on: in step, all of them would fetch the same
+  // chunk of the hidden states at the same time, from the same few slices of L2.
+  const int k_first = cta % kc1;
+  auto k_rot = [&](int kc) { return kc + k_first < kc1 ? kc + k_first : kc + k_first - kc1; };
+#endif
+
   if (warp == 0) {
     // ------------------------------------------------------------------ weight producer
     // Streams every weight tile of this CTA (and the x chunk of gate/up stages).  It arms each
@@ -619,8 +791,12 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     // added by the helper warp once that expert group is complete, so this stream never stalls on
     // it.  The loop is kept to a few instructions per stage: one thread pays every one of them.
     if (lane == 0) {
-      const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
-      uint32_t s = 0, par = 0, n_armed = 0;
+      const uint64_t pol_w = policy_evict_first();
+      uint32_t s = 0, par = 0;
+#if !ACM_FFN_MX
+      const uint64_t pol_x = policy_evict_last();
+      uint32_t n_armed = 0;
+#endif
       bool ok = true;
       for (int si = 0; ok && have_seg(si, true); ++si) {
         const Segment sg = seg[si];
@@ -631,26 +807,28 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
             const int a_of = static_cast<int>(fdiv(static_cast<unsigned>(sg.t0 + tile), p.d_tpe));
             const int32_t ent = s_entry[a_of];
             const int r0 = (sg.t0 + tile - a_of * tpe) * 64, eidx = entry_idx(ent);
+#if !ACM_FFN_MX
             const CUtensorMap* gu = pick_map(entry_src(ent), &maps.gate_up, &maps.shared_gate_up, &maps.staged_gate_up);
+#endif
             for (int kc = k0; kc < k1; ++kc) {
+#if ACM_FFN_MX
+              if (!(ok = mbar_wait(smem_u32(&bars->raw_empty[s]), par ^ 1u, quit, kSitePackedFree))) break;
+              const uint32_t rawb = smem_u32(&bars->raw[s]);
+              mbar_expect_tx(rawb, kMxStageBytes);
+              bulk_load_hint(smem_u32(raw_base) + s * kMxStageBytes,
+                             p.mx_gate_up + (static_cast<size_t>(eidx * tpe + (r0 >> 6)) * kc1 + k_rot(kc)) * kMxStageBytes,
+                             kMxStageBytes, rawb, pol_w);
+              if (++s == static_cast<uint32_t>(p.n_raw)) { s = 0; par ^= 1u; }
+#else
               if (!(ok = mbar_wait(smem_u32(&bars->empty[s]), par ^ 1u, quit, kSiteStageEmpty))) break;
               const uint32_t full = smem_u32(&bars->full[s]);
               const uint32_t sa = smem_u32(stage_base) + s * kStageBytes;
-#if ACM_FFN_MX
-              mbar_expect_tx(full, b_bytes);
-              {
-                const uint32_t rawb = smem_u32(&bars->raw[s]);
-                mbar_expect_tx(rawb, kMxStageBytes);
-                bulk_load_hint(sa, p.mx_gate_up + (static_cast<size_t>(eidx * tpe + (r0 >> 6)) * kc1 + kc) * kMxStageBytes,
-                               kMxStageBytes, rawb, pol_w);
-              }
-#else
               mbar_expect_tx(full, kABytes + b_bytes);
               tma_load_5d(sa, gu, full, 0, r0, 0, kc * kAtoms, eidx, pol_w);   // 64 gate + 64 up rows, 2 atoms
-#endif
               tma_load_3d(sa + kABytes, &x_map, full, 0, 0, kc * kAtoms, pol_x);
               ++n_armed;
               if (++s == kStages) { s = 0; par ^= 1u; }
+#endif
             }
           }
         } else {
@@ -660,24 +838,30 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
             const int q0 = static_cast<int>(fdiv(static_cast<unsigned>(k0), p.d_kpe));
             int a = sg.a0 + q0, ic = k0 - q0 * kpe;
             int32_t ent = s_entry[a];
+#if !ACM_FFN_MX
             const CUtensorMap* dn = pick_map(entry_src(ent), &maps.down, &maps.shared_down, &maps.staged_down);
+#endif
             int eidx = entry_idx(ent);
             for (int kc = k0; kc < k1; ++kc) {
+#if ACM_FFN_MX
+              if (!(ok = mbar_wait(smem_u32(&bars->raw_empty[s]), par ^ 1u, quit, kSitePackedFree))) break;
+              const uint32_t rawb = smem_u32(&bars->raw[s]);
+              mbar_expect_tx(rawb, kMxStageBytes);
+              bulk_load_hint(smem_u32(raw_base) + s * kMxStageBytes,
+                             p.mx_down + (static_cast<size_t>(eidx * h_tiles + ht) * kpe + ic) * kMxStageBytes,
+                             kMxStageBytes, rawb, pol_w);
+              if (++s == static_cast<uint32_t>(p.n_raw)) { s = 0; par ^= 1u; }
+              if (++ic == kpe && kc + 1 < k1) {
+                ic = 0;
+                ent = s_entry[++a];
+                eidx = entry_idx(ent);
+              }
+#else
               if (!(ok = mbar_wait(smem_u32(&bars->empty[s]), par ^ 1u, quit, kSiteStageEmpty))) break;
               const uint32_t full = smem_u32(&bars->full[s]);
               const uint32_t sa = smem_u32(stage_base) + s * kStageBytes;
-#if ACM_FFN_MX
-              mbar_expect_tx(full, b_bytes);
-              {
-                const uint32_t rawb = smem_u32(&bars->raw[s]);
-                mbar_expect_tx(rawb, kMxStageBytes);
-                bulk_load_hint(sa, p.mx_down + (static_cast<size_t>(eidx * h_tiles + ht) * kpe + ic) * kMxStageBytes,
-                               kMxStageBytes, rawb, pol_w);
-              }
-#else
               mbar_expect_tx(full, kABytes + b_bytes);
               tma_load_4d(sa, dn, full, 0, ht * kTileM, ic * kAtoms, eidx, pol_w);
-#endif
               bars->armed = ++n_armed;      // the helper warp may now add this stage's activation chunk
               if (++s == kStages) { s = 0; par ^= 1u; }
               if (++ic == kpe && kc + 1 < k1) {
@@ -686,6 +870,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
                 dn = pick_map(entry_src(ent), &maps.down, &maps.shared_down, &maps.staged_down);
                 eidx = entry_idx(ent);
               }
+#endif
             }
           }
         }
@@ -711,6 +896,57 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         while (global_timer() - t0 < 200000ull) {}
       }
     }
+#if ACM_FFN_MX
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer
+    // The whole warp walks the stages and one elected lane issues: the operands of an MMA are uniform registers, and
+    // in code that only lane 0 runs every one of them is moved there from a vector register first.
+    const uint32_t idesc = umma_mx_idesc(2 * p.n_pad);
+    const uint64_t act_hi = umma_smem_desc_64(0);
+    const uint32_t half_step = static_cast<uint32_t>(act_bytes) >> 5;      // (in 16-byte units) from one half-stage to the other
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint32_t act0 = (smem_u32(act_base) & 0x3ffffu) >> 4;
+    uint32_t s = 0, par = 0, act_slot = 0, b = 0, bpar = 1;
+    bool ok = true;
+    for (int si = 0; ok && __all_sync(0xffffffffu, have_seg(si, true)); ++si) {
+      Sched sc(bars->plan.range[si]);
+      int tile, k0 = 0, k1 = 0;
+      while (ok && __any_sync(0xffffffffu, sc.next(tile, k0, k1))) {
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->tempty[b]), bpar, quit, kSiteAccEmpty));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d_tmem = tm + b * kAccCols;
+        const int nk = __shfl_sync(0xffffffffu, k1 - k0, 0);
+        for (int kc = 0; kc < nk; ++kc) {
+          ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->full[s]), par, quit, kSiteStageFull));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t ta = tm + kAcc * kAccCols + s * kMxACols;
+          const uint32_t sf = tm + kAcc * kAccCols + kMxA * kMxACols + s * kMxScaleCols;
+          const uint64_t db = act_hi | (act0 + act_slot * (static_cast<uint32_t>(act_bytes) >> 4));
+          if (elect_one()) {
+            // 32 K = one scale each (byte kb of the scales' words); two half-stages of 64 K of activations
+            umma_mx(d_tmem, ta, db, idesc, kc > 0 ? 1u : 0u, sf, sf + 4);
+            umma_mx(d_tmem, ta + 8, db + 2, idesc | (1u << 29) | (1u << 4), 1u, sf, sf + 4);
+            umma_mx(d_tmem, ta + 16, db + half_step, idesc | (2u << 29) | (2u << 4), 1u, sf, sf + 4);
+            umma_mx(d_tmem, ta + 24, db + half_step + 2, idesc | (3u << 29) | (3u << 4), 1u, sf, sf + 4);
+            umma_commit(smem_u32(&bars->empty[s]));
+            if (kc + 1 == nk) umma_commit(smem_u32(&bars->tfull[b]));
+          }
+          __syncwarp();
+          if (++act_slot == static_cast<uint32_t>(p.n_act)) act_slot = 0;
+          if (++s == kMxA) { s = 0; par ^= 1u; }
+        }
+        if (++b == kAcc) { b = 0; bpar ^= 1u; }
+      }
+    }
+    if (!ok) {
+      // giving up: wait (bounded) for the MMAs already issued before TMEM is released
+      if (lane == 0) umma_commit(smem_u32(&bars->drained));
+      const unsigned long long t0 = global_timer();
+      while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
+    }
+#else
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     if (lane == 0) {
@@ -732,22 +968,14 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
             tc_fence_after();
             // descriptors: only the address field changes from stage to stage and atom to atom
             const uint32_t sa = smem_u32(stage_base) + s * kStageBytes;
-#if !ACM_FFN_MX
             const uint64_t da0 = desc_hi | ((sa & 0x3ffffu) >> 4);
-#endif
             const uint64_t db0 = desc_hi | (((sa + kABytes) & 0x3ffffu) >> 4);
 #pragma unroll
             for (int at = 0; at < kAtoms; ++at) {
 #pragma unroll
               for (int kk = 0; kk < kBK / 16; ++kk) {
-#if ACM_FFN_MX
-                // the expanded weights are in tensor memory: stage s, 8 columns per 16 K
-                umma_bf16_ts(d_tmem, tmem_base + kAcc * kAccCols + s * kMxACols + (at * (kBK / 16) + kk) * 8,
-                             db0 + (at * (b_atom_bytes >> 4) + 2 * kk), idesc, (kc > k0 || at > 0 || kk > 0) ? 1u : 0u);
-#else
                 umma_bf16(d_tmem, da0 + (at * (kAtomABytes >> 4) + 2 * kk), db0 + (at * (b_atom_bytes >> 4) + 2 * kk), idesc,
                           (kc > k0 || at > 0 || kk > 0) ? 1u : 0u);
-#endif
               }
             }
             umma_commit(smem_u32(&bars->empty[s]));
@@ -764,6 +992,73 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
       }
     }
+#endif
+#if ACM_FFN_MX
+  } else if (warp == 6) {
+    // ------------------------------------------------------------------ activation producer
+    // Fetches the activation pieces of every stage, a stage of 128 K = two half-stages of 64: the hidden states' once
+    // the router kernel's CTAs have stored them all, an expert's activations once all its tiles have been stored.
+    bool ok = true, x_seen = false;
+    const uint64_t pol_x = policy_evict_last();
+    uint32_t ai = 0, apar = 0;
+    auto fetch = [&](const unsigned char* pieces, const unsigned char* scales) -> bool {
+      if (!mbar_wait(smem_u32(&bars->act_empty[ai]), apar ^ 1u, quit, kSiteActSlot)) return false;
+      const uint32_t full = smem_u32(&bars->act[ai]);
+      mbar_expect_tx(full, static_cast<uint32_t>(act_bytes) + 2 * kMxActScaleBytes);
+      bulk_load_hint(smem_u32(act_base) + ai * act_bytes, pieces, act_bytes, full, pol_x);
+      bulk_load_hint(smem_u32(act_scale_base) + ai * 2 * kMxActScaleBytes, scales, 2 * kMxActScaleBytes, full, pol_x);
+      if (++ai == static_cast<uint32_t>(p.n_act)) { ai = 0; apar ^= 1u; }
+      return true;
+    };
+    for (int si = 0; ok && have_seg(si, true); ++si) {
+      const Segment sg = seg[si];
+      const SegRange& rg = bars->plan.range[si];
+      if (sg.phase == 1) {
+        if (lane == 0) {
+          if (!x_seen) {
+            ok = count_wait(p.xq_count, p.xq_target, quit, kSiteXPieces);
+            fence_proxy_async();
+            x_seen = true;
+          }
+          Sched sc(rg);
+          int tile, k0, k1;
+          while (ok && sc.next(tile, k0, k1))
+            for (int kc = k0; ok && kc < k1; ++kc)
+              ok = fetch(p.xq + static_cast<size_t>(k_rot(kc)) * act_bytes, p.xq_scale + static_cast<size_t>(k_rot(kc)) * 2 * kMxActScaleBytes);
+        }
+      } else {
+        bool good = true;
+        const unsigned n_units = rg.u_end - rg.u;
+        if (n_units > 0) {      // the experts this CTA's share reads (as in the bf16 build's helper warp)
+          int q_lo = 0, q_hi = sg.a1 - sg.a0 - 1;
+          if (static_cast<unsigned>(rg.k00) + n_units <= static_cast<unsigned>(rg.kc)) {
+            q_lo = static_cast<int>(fdiv(static_cast<unsigned>(rg.k00), p.d_kpe));
+            q_hi = static_cast<int>(fdiv(static_cast<unsigned>(rg.k00) + n_units - 1u, p.d_kpe));
+          }
+          for (int q = q_lo + lane; q <= q_hi && good; q += 32)
+            good = flag_wait_ge(&p.ready[sg.a0 + q], tpe, quit, kSiteExpertReady);
+        }
+        ok = __all_sync(0xffffffffu, good);
+        if (ok && lane == 0) {
+          Sched sc(rg);
+          int ht, k0, k1;
+          fence_proxy_async();
+          while (ok && sc.next(ht, k0, k1)) {
+            const int q0 = static_cast<int>(fdiv(static_cast<unsigned>(k0), p.d_kpe));
+            // (an expert's K-chunks lie one after the other, and so do the experts of a segment)
+            size_t at = static_cast<size_t>(sg.a0 + q0) * kpe + (k0 - q0 * kpe);
+            for (int kc = k0; ok && kc < k1; ++kc, ++at) ok = fetch(p.hq + at * act_bytes, p.hq_scale + at * 2 * kMxActScaleBytes);
+          }
+        }
+      }
+      ok = __all_sync(0xffffffffu, ok);
+    }
+    if (!ok) {
+      // giving up: let copies already in flight land before the CTA exits
+      const unsigned long long t0 = global_timer();
+      while (global_timer() - t0 < 200000ull) {}
+    }
+#else
   } else if (warp == 6) {
     // ------------------------------------------------------------------ helper warp
     // Keeps slow global round trips off the other roles' paths: (a) for each gate/up segment whose
@@ -773,66 +1068,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     bool ok = true;
     int frag_uses = 0;
     uint32_t hs = 0, hidx = 0;   // ring slot and running index of the next stage, tracked through the gate/up stages too
-    if (pre) {
-      // While the others run the anchors' pre-segment: wait for the eligible set, give the other experts the
-      // slots behind the pre-streamed ones (ascending id), append the shared experts, work out the rest of the
-      // plan, and let everyone on.
-      // eight words per block; lane l takes words l and l + 32 (blocks 0-3 and 4-7), the union goes to lanes 0..7
-      bool seen = true;
-      uint32_t half = 0u;
-      {
-        const uint32_t tag = static_cast<uint32_t>(p.sel_epoch) & 0xffffu;
-        const int n_words = 2 * kMaskWords * p.sel_blocks;
-#pragma unroll
-        for (int part = 0; part < 2; ++part) {
-          const int j = lane + 32 * part;
-          if (j < n_words) {
-            bool got = true;
-            half |= poll_tagged_word(p.sel_flag + j, tag, p.wait_limit_ns, got);
-            seen = seen && got;
-          }
-        }
-        half |= __shfl_xor_sync(0xffffffffu, half, 8);
-        half |= __shfl_xor_sync(0xffffffffu, half, 16);
-      }
-      const bool good = __all_sync(0xffffffffu, seen);
-      uint32_t rest[kMaskWords];
-      int n_rest = 0;
-#pragma unroll
-      for (int wd = 0; wd < kMaskWords; ++wd) {
-        const uint32_t lo = __shfl_sync(0xffffffffu, half, 2 * wd), hi = __shfl_sync(0xffffffffu, half, 2 * wd + 1);
-        rest[wd] = ((lo | (hi << 16)) & p.only[wd]) & ~am[wd];
-        n_rest += __popc(rest[wd]);
-      }
-      if (good) {
-        for (int e = lane; e < kMaxExperts; e += 32) {
-          const int wd = e >> 5;
-          const uint32_t mine = wd == 0 ? rest[0] : wd == 1 ? rest[1] : wd == 2 ? rest[2] : rest[3];
-          if ((mine >> (e & 31)) & 1u) {
-            int slot = n_pre + __popc(mine & ((1u << (e & 31)) - 1u));
-#pragma unroll
-            for (int w2 = 0; w2 < kMaskWords; ++w2) slot += w2 < wd ? __popc(rest[w2]) : 0;
-            s_entry[slot] = make_entry(kSrcRouted, e);
-            bars->expert[slot] = e;
-          }
-        }
-        if (lane < p.n_shared) {
-          s_entry[n_pre + n_rest + lane] = make_entry(kSrcShared, lane);
-          bars->expert[n_pre + n_rest + lane] = -1;
-        }
-        if (lane == 0) bars->n_routed_slots = n_pre + n_rest;
-        if (lane < 4)
-          plan_lane(bars->plan, lane, cta, n_pre + n_rest + p.n_shared, tpe, G, p.d_kc1, kpe, p.d_grid, p.d_tpe, h_tiles,
-                    n_pre, 1);
-      } else if (lane == 0) {
-        give_up(quit, kSiteEligibleWords);
-      }
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(smem_u32(&bars->plan_ready));
-      }
-      ok = good;
-    }
+    if (pre) ok = complete_plan();
     for (int si = 0; ok && have_seg(si, false); ++si) {
       const Segment sg = seg[si];
       const int n_exp = sg.a1 - sg.a0;
@@ -937,22 +1173,34 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         ok = __all_sync(0xffffffffu, good);
       }
     }
+#endif
   } else if (warp == 7) {
     // ------------------------------------------------------------------ publisher
     // Moves what the epilogue staged in shared memory to global memory with bulk copies, waits for
     // them to complete and only then announces them (fragment flag / finished-tile counter).
+#if ACM_FFN_MX
+    const bool planned = !pre || complete_plan();
+#else
+    constexpr bool planned = true;
+#endif
     if (lane == 0) {
-      uint32_t ost_n = 0, fin_n = 0;
-      bool ok = true;
+      uint32_t fin_n = 0;
+#if !ACM_FFN_MX
+      uint32_t ost_n = 0;
+#endif
+      bool ok = planned;
       for (int si = 0; ok && have_seg(si, true); ++si) {
         const Segment sg = seg[si];
         if (sg.phase != 1) continue;
+#if !ACM_FFN_MX
         float* frag = p.frag + static_cast<size_t>(sg.p1_index) * G * 2 * kFragFloats;
         int32_t* frag_flag = p.frag_flag + sg.p1_index * G * 2;
+#endif
         Sched sc(bars->plan.range[si]);
         int tile, k0, k1;
         while (ok && sc.next(tile, k0, k1)) {
          for (int h = 0; h < n_halves && ok; ++h) {          // a wide tile comes in two column halves
+#if !ACM_FFN_MX
           if (k0 > 0) {
             if (!(ok = mbar_wait(smem_u32(&bars->ost_full), ost_n & 1u, quit, kSiteOutStaged))) break;
             const uint32_t bytes = static_cast<uint32_t>(min(p.n_pad - h * kMaxNodes, kMaxNodes)) * kTileM * 4u;
@@ -969,12 +1217,21 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
             red_release_add(&frag_flag[c_head * 2 + h], 1);
             mbar_arrive(smem_u32(&bars->ost_free));
             ++ost_n;
-          } else {
-            const uint32_t hb = fin_n & 1u;
-            if (!(ok = mbar_wait(smem_u32(&bars->hst_full[hb]), (fin_n >> 1) & 1u, quit, kSiteActStaged))) break;
+          } else
+#endif
+          {
+            const uint32_t hb = fin_n % kHStages;
+            if (!(ok = mbar_wait(smem_u32(&bars->hst_full[hb]), (fin_n / kHStages) & 1u, quit, kSiteActStaged))) break;
             const int a = static_cast<int>(fdiv(static_cast<unsigned>(sg.t0 + tile), p.d_tpe)), ti = sg.t0 + tile - a * tpe;
+#if ACM_FFN_MX
+            const size_t tile_at = static_cast<size_t>(a) * tpe + ti;
+            bulk_store(p.hq + tile_at * (act_bytes / 2), smem_u32(hstage + hb * kHStageBytes), act_bytes / 2);
+            bulk_store(p.hq_scale + tile_at * kMxActScaleBytes, smem_u32(hstage + hb * kHStageBytes) + kMaxNodes * 128,
+                       kMxActScaleBytes);
+#else
             asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
                          ::"l"(&hs_map), "r"(0), "r"(h * kMaxNodes), "r"(ti), "r"(a), "r"(smem_u32(hstage + hb * kHStageBytes)) : "memory");
+#endif
             bulk_commit();
             bulk_wait_all();
             red_release_add(&p.ready[a], 1);
@@ -987,67 +1244,89 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     }
 #if ACM_FFN_MX
   } else if (warp >= 8) {
-    // ------------------------------------------------------------------ expanding warps (MXFP4 -> bf16)
-    // Thread r owns weight-tile row r = lane r of tensor memory.  Per stage: wait for the packed copy, take
-    // the row's 64 code bytes and 4 scale bytes from shared memory, expand them to 128 bf16 in registers and
-    // store those into the stage's 64 columns of tensor memory, from where the MMAs take their A operand --
-    // the expanded tile never passes through shared memory.
-    // A code is sign | 2 exponent bits | 1 mantissa bit with subnormals: put at bits 15 | 8:7 | 6 of a bf16 it
-    // is the value times 2^-126 exactly, so one bf16 multiply by 2^(scale byte - 1) finishes the job.
-    const int r = threadIdx.x - 256;
-    const uint32_t my_lane = static_cast<uint32_t>(r & ~31) << 16;          // this warp's quarter of the lanes
+    // ------------------------------------------------------------------ unpacking warps
+    // Two groups of four warps take the stages in turn.  Thread r of a group unpacks row r = lane r of tensor memory;
+    // every warp stores the stage's scales, both operands', into its quarter (rows i, i + 32, i + 64, i + 96 in lane i;
+    // copies by tcgen05.cp instead took 260 clocks a stage out of the MMAs' pipe).  A group's next
+    // record is loaded while the stage at hand is being stored, and given back behind it.
+    const int r = threadIdx.x & 127, group = (warp - 8) >> 2;
+    const uint32_t my_lane = static_cast<uint32_t>((warp & 3) * 32) << 16;
     bool ok = true;
-    // the row's packed data of the stage at hand
+    unsigned it = static_cast<unsigned>(group), total = 0;
+    uint32_t ri = static_cast<uint32_t>(group), rpar = 0, ai = static_cast<uint32_t>(group), apar = 0;
+    uint32_t ai_done = static_cast<uint32_t>(group ^ 1);      // of the stage kMxA before the group's next one from stage kMxA on
     uint4 q[4];
-    uint32_t sc = 0;
-    auto fetch = [&](unsigned it) -> bool {
-      const uint32_t s = it % kStages, par = (it / kStages) & 1u;
-      if (!mbar_wait(smem_u32(&bars->raw[s]), par, quit, kSitePackedStage)) return false;
-      const unsigned char* A = stage_base + static_cast<size_t>(s) * kStageBytes;
+    uint32_t sa[4];
+    auto wait_raw = [&]() -> bool {
+      return __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->raw[ri]), rpar, quit, kSitePackedStage));
+    };
+    auto load_raw = [&]() {
+      const unsigned char* R = raw_base + static_cast<size_t>(ri) * kMxStageBytes;
       // (the record keeps the row's four 16-byte pieces rotated by the row number, so that a warp's loads
       // spread over all banks)
 #pragma unroll
-      for (int b = 0; b < 4; ++b) q[b] = *reinterpret_cast<const uint4*>(A + r * 64 + 16 * (b ^ ((r >> 1) & 3)));
-      sc = *reinterpret_cast<const uint32_t*>(A + kMxCodeBytes + r * 4);
-      return true;
+      for (int b = 0; b < 4; ++b) q[b] = *reinterpret_cast<const uint4*>(R + r * 64 + 16 * (b ^ ((r >> 1) & 3)));
+#pragma unroll
+      for (int g = 0; g < 4; ++g) sa[g] = *reinterpret_cast<const uint32_t*>(R + kMxCodeBytes + (lane + 32 * g) * 4);
     };
-    // stage by stage through the segments (with the anchors' pre-segment the later ones arrive behind plan_ready)
-    unsigned it = 0, total = 0;
+    auto release_raw = [&]() {        // (once the loads above have arrived)
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->raw_empty[ri]));
+      ri += 2u;
+      if (ri >= static_cast<uint32_t>(p.n_raw)) { ri -= static_cast<uint32_t>(p.n_raw); rpar ^= 1u; }
+    };
     bool fetched = false;
     for (int si = 0; ok && have_seg(si, true); ++si) {
      total += bars->plan.range[si].n_stages;
-     if (!fetched && it < total) { ok = fetch(it); fetched = true; }
-     for (; it < total && ok; ++it) {
-      const uint32_t s = it % kStages;
-      const uint32_t a_tmem = tmem_base + my_lane + kAcc * kAccCols + s * kMxACols;
-      tc_fence_after();
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {                     // 32 K = one scale = 16 columns
-        const uint32_t field = min(((sc >> (8 * b)) & 0xffu) + 126u, 254u) << 7;
-        const uint32_t c2 = field | (field << 16);
-        const uint32_t words[4] = {q[b].x, q[b].y, q[b].z, q[b].w};
-        uint32_t o[16];
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          // a word holds elements 2j (nibble j) and 2j+1 (nibble 4+j): pairs 0 and 1 are masked out where they
-          // sit -- the multiplier that moves magnitude and sign into place differs -- pairs 2 and 3 after one shift
-          const uint32_t w2 = words[w] >> 8;
-          const uint32_t e0 = ((words[w] & 0x000f000fu) * 0x1040u) & 0x81c081c0u;
-          const uint32_t e1 = ((words[w] & 0x00f000f0u) * 0x0104u) & 0x81c081c0u;
-          const uint32_t e2 = ((w2 & 0x000f000fu) * 0x1040u) & 0x81c081c0u;
-          const uint32_t e3 = ((w2 & 0x00f000f0u) * 0x0104u) & 0x81c081c0u;
-          asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(o[4 * w + 0]) : "r"(e0), "r"(c2));
-          asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(o[4 * w + 1]) : "r"(e1), "r"(c2));
-          asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(o[4 * w + 2]) : "r"(e2), "r"(c2));
-          asm("mul.rn.bf16x2 %0, %1, %2;" : "=r"(o[4 * w + 3]) : "r"(e3), "r"(c2));
-        }
-        tmem_st16(a_tmem + 16 * b, o);
+     for (; it < total; it += 2) {
+      if (!fetched) {
+        if (!(ok = wait_raw())) break;
+        load_raw();
+        release_raw();
       }
+      uint32_t o[32], so[4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const uint32_t words[4] = {q[b].x, q[b].y, q[b].z, q[b].w};
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {      // the low nibbles of a word's bytes, then the high ones
+          o[8 * b + 2 * w] = (words[w] << 2) & 0x3c3c3c3cu;
+          o[8 * b + 2 * w + 1] = (words[w] >> 2) & 0x3c3c3c3cu;
+        }
+      }
+      // (scale bytes above the limit, which no registered tensor holds, count as the limit)
+#pragma unroll
+      for (int g = 0; g < 4; ++g) so[g] = __vminu4(sa[g], 0x80808080u);
+      const uint32_t s = it % kMxA, par = (it / kMxA) & 1u;
+      if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->empty[s]), par ^ 1u, quit, kSiteStageEmpty)))) break;
+      tc_fence_after();
+      if (it >= static_cast<unsigned>(kMxA)) {
+        // the stage before in this slot has been multiplied: so have its activations (a commit of their own would cost
+        // the MMAs' pipe 60 clocks a stage)
+        if (r == 0) mbar_arrive(smem_u32(&bars->act_empty[ai_done]));
+        ai_done += 2u;
+        if (ai_done >= static_cast<uint32_t>(p.n_act)) ai_done -= static_cast<uint32_t>(p.n_act);
+      }
+      tmem_st32(tmem_base + my_lane + kAcc * kAccCols + s * kMxACols, o);
+      const uint32_t sf = tmem_base + my_lane + kAcc * kAccCols + kMxA * kMxACols + s * kMxScaleCols;
+      tmem_st4(sf, so[0], so[1], so[2], so[3]);
+      fetched = it + 2 < total;
+      if (fetched) {
+        if (!(ok = wait_raw())) break;
+        load_raw();
+      }
+      if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->act[ai]), apar, quit, kSiteActStage)))) break;
+      const uint4* S = reinterpret_cast<const uint4*>(act_scale_base + ai * 2 * kMxActScaleBytes) + lane;
+      const uint4 lo = S[0], hi = S[kMxActScaleBytes / 16];      // two half-stages, two bytes of a word each
+      tmem_st4(sf + 4, __byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.z, hi.z, 0x5410),
+               __byte_perm(lo.w, hi.w, 0x5410));
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->full[s]));
-      if (it + 1 < total) ok = fetch(it + 1); else fetched = false;
+      ai += 2u;
+      if (ai >= static_cast<uint32_t>(p.n_act)) { ai -= static_cast<uint32_t>(p.n_act); apar ^= 1u; }
+      if (fetched) release_raw();
      }
     }
 #endif
@@ -1059,8 +1338,31 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     const int quarter = warp & 3;               // TMEM lanes this warp may read
     const int row = quarter * 32 + lane;        // accumulator row = weight-tile row
     const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
-    uint32_t f = 0, ost_uses = 0, fin_count = 0, frag_reads = 0;
+    uint32_t f = 0, fin_count = 0;
+#if !ACM_FFN_MX
+    uint32_t ost_uses = 0, frag_reads = 0;
+#endif
     bool ok = true, waited = !early;
+#if ACM_FFN_MX
+    // 32 node columns from column c on (the last 16 only if there are that many): both pieces' sums
+    auto load_32 = [&](uint32_t b, int c, int np, float (&v)[32]) {
+      float v2[32];
+      const uint32_t at = tmem_base + lane_addr + b * kAccCols + c;
+      tmem_ld16(at, v);
+      tmem_ld16(at + np, v2);
+      if (c + 16 < np) {
+        tmem_ld16(at + 16, v + 16);
+        tmem_ld16(at + np + 16, v2 + 16);
+      }
+      tmem_ld_wait();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] += v2[j];
+    };
+    auto release_acc = [&](uint32_t b) {
+      tc_fence_before();
+      mbar_arrive(smem_u32(&bars->tempty[b]));
+    };
+#else
     float v[kMaxNodes];
     // one half (up to 64 columns from column `cb` on) of accumulator b; the accumulator is released with its last half
     auto load_half = [&](uint32_t b, int cb, int np, bool release) {
@@ -1073,12 +1375,15 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         mbar_arrive(smem_u32(&bars->tempty[b]));
       }
     };
+#endif
+#if !ACM_FFN_MX
     // the outgoing-fragment buffer (and the exchange buffer aliasing it) is free once the publisher
     // has copied the previous fragment out
     auto wait_ostage = [&]() -> bool {
       if (ost_uses == 0) return true;
       return epi_vote_all(mbar_wait(smem_u32(&bars->ost_free), (ost_uses - 1) & 1u, quit, kSiteOutFree));
     };
+#endif
     for (int si = 0; ok && have_seg(si, true); ++si) {
       const Segment sg = seg[si];
       if (sg.phase == 1) {
@@ -1108,6 +1413,63 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
           for (int h = 0; h < n_halves && ok; ++h) {
             const int cb = h * kMaxNodes;                              // first node column of this half
             const int np = min(p.n_pad - cb, kMaxNodes);               // its columns (a multiple of 16)
+#if ACM_FFN_MX
+            // The tile goes through the exchange buffer, [node][64 gate rows, 64 up rows] with the rows rotated by the
+            // node, and a thread then takes up the 32 features of one node, i.e. one scale block, so that the block's
+            // maximum and its packed pieces never leave the thread.  (A thread per feature, which needs a warp reduction
+            // per node, took 2.7-4.6 us a tile in a rolled loop and 5-8 us unrolled -- 40 KB of instructions, fetched
+            // anew through the busy L2.)
+#pragma unroll 1
+            for (int c = 0; c < np; c += 32) {
+              float v[32];
+              load_32(b, c, np, v);
+              float* dst = ostage + c * kTileM;
+#pragma unroll
+              for (int j = 0; j < 32; ++j)
+                if (j < 16 || c + 16 < np) dst[j * kTileM + (row ^ j)] = v[j];
+            }
+            release_acc(b);
+            bool hst_ok = true;
+            if (fin_count >= 1) hst_ok = mbar_wait(smem_u32(&bars->hst_free[0]), (fin_count - 1) & 1u, quit, kSiteActFree);
+            ok = epi_vote_all(hst_ok);      // also orders the writes above before the reads below
+            if (!ok) break;
+            {
+              unsigned char* hs = hstage;
+              const int t = row & 63, half = row >> 6;        // this thread's node and 32 features
+              if (t < np) {
+                const float wgt = bars->wd[t];
+                const float* gate = ostage + t * kTileM;
+                uint32_t h2[16];
+#pragma unroll
+                for (int i = 0; i < 32; i += 2) {
+                  float hval[2];
+#pragma unroll
+                  for (int j = 0; j < 2; ++j) {
+                    // w * u * silu(g), silu(g) = g/2 * (1 + tanh(g/2))
+                    const int at = 32 * half + ((i + j) ^ (t & 31));
+                    const float g = gate[at], u = gate[64 + at];
+                    const float hg = 0.5f * g;
+                    float th;
+                    asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(hg));
+                    const float q = wgt * u * hg;
+                    hval[j] = fmaf(q, th, q);
+                  }
+                  const __nv_bfloat162 pair = __floats2bfloat162_rn(hval[0], hval[1]);
+                  h2[i / 2] = *reinterpret_cast<const uint32_t*>(&pair);
+                }
+                MxBlock blk;
+                mx_split_block(h2, blk);
+                const int tb = p.n_pad + t;
+                mx_store_rows(hs, blk, t, tb, half);
+                unsigned char* scales = hs + kMaxNodes * 128 + half;
+                scales[mx_scale_at(t)] = blk.scale_a;
+                scales[mx_scale_at(tb)] = blk.scale_b;
+              }
+              fence_proxy_async_smem();
+              mbar_arrive(smem_u32(&bars->hst_full[0]));
+              ++fin_count;
+            }
+#else
             load_half(b, cb, np, h == n_halves - 1);
             if (k0 > 0) {
               // tail part of a tile whose first chunks belong to an earlier CTA: stage the fragment
@@ -1187,6 +1549,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
               mbar_arrive(smem_u32(&bars->hst_full[hb]));
               ++fin_count;
             }
+#endif
           }
         }
         if (row == 0) ACM_STAMP(10);
@@ -1199,6 +1562,18 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
           if (!ok) break;
           tc_fence_after();
           ++f;
+#if ACM_FFN_MX
+#pragma unroll 1
+          for (int c = 0; c < p.n_pad; c += 32) {
+            float v[32];
+            load_32(b, c, p.n_pad, v);
+            float* dst = p.out + static_cast<size_t>(c) * p.H + static_cast<size_t>(ht) * kTileM + row;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (c + j < p.T) atomicAdd(dst + static_cast<size_t>(j) * p.H, v[j]);
+          }
+          release_acc(b);
+#else
           for (int h = 0; h < n_halves; ++h) {
             const int cb = h * kMaxNodes;
             load_half(b, cb, min(p.n_pad - cb, kMaxNodes), h == n_halves - 1);
@@ -1207,6 +1582,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
             for (int c = 0; c < kMaxNodes; ++c)
               if (cb + c < p.T) atomicAdd(dst + static_cast<size_t>(c) * p.H, v[c]);
           }
+#endif
         }
         if (row == 0) ACM_STAMP(11);
       }
@@ -1280,6 +1656,15 @@ __global__ void k_ffn_f32_down(const float* __restrict__ down, const float* __re
 }  // namespace
 
 #if ACM_FFN_MX
+namespace {
+// Ring depths for a launch of n_pad node columns: as many activation stages as there is room for with a packed record
+// each, then records with what is left (at least 7 of either).
+void mx_rings(int n_pad, int* n_act, int* n_raw) {
+  const int left = kMxRingBytes, act = n_pad * 256 + 2 * kMxActScaleBytes;
+  *n_act = min(kMaxAct, left / (act + kMxStageBytes));
+  *n_raw = min(kMaxRaw, (left - *n_act * act) / kMxStageBytes);
+}
+}  // namespace
 cudaError_t ffn_mx_configure() {
   return cudaFuncSetAttribute(ACM_FFN_KERNEL<kMaxNodes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(Geo<kMaxNodes>::kSmemBytes));
@@ -1326,6 +1711,14 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
   if (!L.mx_gate_up || !L.mx_down || L.I % 128 != 0 || L.n_shared != 0) return cudaErrorInvalidValue;
   a.mx_gate_up = static_cast<const unsigned char*>(L.mx_gate_up);
   a.mx_down = static_cast<const unsigned char*>(L.mx_down);
+  if (!L.xq || L.n_pad > kMaxNodes) return cudaErrorInvalidValue;
+  a.xq = static_cast<const unsigned char*>(L.xq);
+  a.xq_scale = a.xq + mx_act_scale_offset(L.H);
+  a.xq_count = L.xq_count; a.xq_target = L.xq_target;
+  // (a slot's share of the activation buffer is 256 I bytes: up to 128 I of pieces; the scales lie behind all pieces)
+  a.hq = static_cast<unsigned char*>(L.hbuf);
+  a.hq_scale = a.hq + static_cast<size_t>(kMaxSlots) * 128 * L.I;
+  mx_rings(L.n_pad, &a.n_act, &a.n_raw);
 #endif
   void* args[] = {const_cast<FfnMaps*>(&maps), const_cast<CUtensorMap*>(&x_map), const_cast<CUtensorMap*>(&h_map),
                   const_cast<CUtensorMap*>(&hs_map), &a};

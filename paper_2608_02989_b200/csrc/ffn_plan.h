@@ -24,7 +24,10 @@
 // others are still in their anchor tile:
 //   fewer rest tiles than CTAs: they are dealt whole, one per CTA, to the idle CTAs first (no exchange at all);
 //   else as above.  The anchors' experts are complete early: their down projection comes first.
-// (Measured and dropped: every tile whole with the CTAs that get one tile less taking down work early -- the last
+// A launch of the MXFP4 kernel (kUncut) deals every tile whole, behind the anchors to the idle CTAs first: its tiles take
+// a third of the bf16 ones' time, less than the exchange of a cut tile's partial sums (7-9 us, during which the CTA that
+// waits for them finalises nothing else).
+// (Measured and dropped, bf16: every tile whole with the CTAs that get one tile less taking down work early -- the last
 // round's experts then start their down projection too late; the leftover tiles after the whole rounds instead of
 // before them; the leftover tiles cut over the idle CTAs only.)
 #pragma once
@@ -152,6 +155,8 @@ ACM_PLAN_FN SegRange make_range(const Segment& sg, int cta, const FastDiv& d_gri
 // (the candidates in order, each present or not), so nothing waits for a serial pass; lane 0 publishes the count
 // last.  n_act counts every slot of the work list (the n_pre pre-streamed experts first); base = 1 when segment 0
 // is the pre-segment.
+// (kUncut: the MXFP4 kernel's plan, see above.)
+template <bool kUncut = false>
 ACM_PLAN_FN void plan_lane(Plan& pl, int lane, int cta, int n_act, int tpe, int grid, const FastDiv& d_kc1, int kpe,
                            const FastDiv& d_grid, const FastDiv& d_tpe, int h_tiles, int n_pre = 0, int base = 0) {
   const int t_pre = n_pre * tpe;                   // tiles (= CTAs) of the pre-segment
@@ -161,7 +166,11 @@ ACM_PLAN_FN void plan_lane(Plan& pl, int lane, int cta, int n_act, int tpe, int 
   Segment c0 = {}, c1 = {}, c2 = {}, c3 = {};
   bool h0 = false, h1 = false, h2 = false, h3 = false;
   int a_split;
-  if (rounds == 0 && n_pre > 0) {
+  if (kUncut) {
+    const int early_tiles = rem > 0 || rounds == 0 ? rounds * grid : (rounds - 1) * grid;      // dealt before the last round
+    a_split = n_pre + static_cast<int>(fdiv(static_cast<unsigned>(early_tiles), d_tpe));
+    c0 = Segment{1, 1, t_pre, n_t, 0, 0, 0, d_kc1, t_pre < grid ? t_pre : 0};             h0 = n_t > 0;
+  } else if (rounds == 0 && n_pre > 0) {
     // behind the anchors, fewer tiles than CTAs: dealt whole, the idle CTAs [t_pre, G) first
     a_split = n_pre;
     c0 = Segment{1, 1, t_pre, n_t, 0, 0, 0, d_kc1, t_pre < grid ? t_pre : 0};             h0 = n_t > 0;

@@ -11,6 +11,7 @@
 #include <cuda_bf16.h>
 
 #include "acm_internal.h"
+#include "mx_act.cuh"
 
 namespace acm {
 namespace {
@@ -220,12 +221,37 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   return false;
 }
 
-template <typename Elem>
+// Blocks of 32 hidden states into the FFN kernel's pieces, a thread per block of a node: thread i of n.
+__device__ __forceinline__ void split_x(const XqArgs& xa, const __nv_bfloat16* x, int T, int H, int i, int n) {
+  const int per_node = H / 32;
+  for (; i < T * per_node; i += n) {
+    const int t = i / per_node, block = i - t * per_node, half = block >> 1, tb = xa.n_pad + t;
+    uint32_t w[16];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint4 v = *reinterpret_cast<const uint4*>(x + static_cast<size_t>(t) * H + 32 * block + 8 * j);
+      w[4 * j] = v.x; w[4 * j + 1] = v.y; w[4 * j + 2] = v.z; w[4 * j + 3] = v.w;
+    }
+    MxBlock k;
+    mx_split_block(w, k);
+    mx_store_rows(xa.xq + static_cast<size_t>(half) * (2 * xa.n_pad * 64), k, t, tb, block & 1);
+    unsigned char* sc = xa.xq + mx_act_scale_offset(H) + static_cast<size_t>(half) * kMxActScaleBytes + (block & 1);
+    sc[mx_scale_at(t)] = k.scale_a;
+    sc[mx_scale_at(tb)] = k.scale_b;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(xa.count) : "memory");
+}
+
+// kPieces: xa.rows further rows of CTAs, behind the roots', store the hidden states' pieces for an MXFP4 layer's FFN kernel
+// (which polls xa.count: it starts before this kernel has completed).  Work of its own CTAs: done by the tile CTAs ahead of
+// their dot products it put 1.5 us on the logits.  (A template parameter: the bf16 layers' kernel keeps its code size.)
+template <typename Elem, bool kPieces = false>
 __global__ void __launch_bounds__(kRT * kRE * (32 / ElemTraits<Elem>::EPT))
 k_router_logits(const Elem* __restrict__ x, const Elem* __restrict__ wr, const float* __restrict__ bias,
                 float* logits, int T, int H, int E, int n_chunks, float* zero_buf,
                 size_t zero_floats, float* zero_buf2, size_t zero_floats2, int32_t* status, float* probs, int32_t* nat_idx, uint32_t* nat_mask, int k,
-                int32_t* tile_done, long long* dbg, RootArgs ro) {
+                int32_t* tile_done, long long* dbg, RootArgs ro, XqArgs xa) {
   constexpr int EPT = ElemTraits<Elem>::EPT;
   constexpr int Q = 32 / EPT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -234,13 +260,23 @@ k_router_logits(const Elem* __restrict__ x, const Elem* __restrict__ wr, const f
   unsigned char* ws = smem_raw + static_cast<size_t>(kRT) * row_bytes;
 
   const int tid = threadIdx.x;
-  // The first ro.rows rows of CTAs in the grid work on one block's root each (see below); the node tiles follow.
+  // The first ro.rows rows of CTAs in the grid work on one block's root each (see below); the node tiles follow (kPieces:
+  // behind xa.rows rows that store the hidden states' pieces).
   const bool for_root = static_cast<int>(blockIdx.y) < ro.rows;
   int root_row = 0;
 #pragma unroll
   for (int b = 0; b < kMaxEarlyBlocks; ++b) root_row = static_cast<int>(blockIdx.y) == b ? ro.row[b] : root_row;
-  const int e0 = blockIdx.x * kRE, t0 = for_root ? root_row : (static_cast<int>(blockIdx.y) - ro.rows) * kRT;
+  const int e0 = blockIdx.x * kRE, t0 = for_root ? root_row : (static_cast<int>(blockIdx.y) - ro.rows - (kPieces ? xa.rows : 0)) * kRT;
   griddep_launch_dependents();
+  if constexpr (kPieces) {
+    const int row = static_cast<int>(blockIdx.y) - ro.rows;
+    if (row >= 0 && row < xa.rows) {
+      griddep_wait();
+      split_x(xa, x, T, H, static_cast<int>((row * gridDim.x + blockIdx.x) * blockDim.x + threadIdx.x),
+              static_cast<int>(xa.rows * gridDim.x * blockDim.x));
+      return;
+    }
+  }
 
   // Staging: the 4 x-rows and 8 router rows of this tile, in n_chunks pieces along h.  One thread
   // per row issues its pieces as bulk copies; piece c of all rows completes on barrier c.  The
@@ -278,8 +314,10 @@ k_router_logits(const Elem* __restrict__ x, const Elem* __restrict__ wr, const f
   // zero the FFN output buffer (accumulated into by the FFN kernel) and the FFN kernel's routing
   // inputs (activated mask, weight table, finished-tile counters), spread over the grid
   {
-    const size_t nb = static_cast<size_t>(gridDim.x) * gridDim.y;
-    const size_t b = static_cast<size_t>(blockIdx.y) * gridDim.x + blockIdx.x;
+    const int skip = kPieces ? xa.rows : 0;      // (the splitting CTAs take no part)
+    const int row = static_cast<int>(blockIdx.y) - (static_cast<int>(blockIdx.y) >= ro.rows ? skip : 0);
+    const size_t nb = static_cast<size_t>(gridDim.x) * (gridDim.y - skip);
+    const size_t b = static_cast<size_t>(row) * gridDim.x + blockIdx.x;
     if (zero_buf) {
       float4* z4 = reinterpret_cast<float4*>(zero_buf);
       for (size_t i = b * blockDim.x + tid; i < zero_floats / 4; i += nb * blockDim.x) z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -998,16 +1036,37 @@ __global__ void __launch_bounds__(512) k_routes_to_table(const int32_t* idx, con
   }
 }
 
+// The hidden states' pieces for routes given by the caller (acm_expert_ffn).
+__global__ void __launch_bounds__(256) k_split_x(const __nv_bfloat16* x, int T, int H, XqArgs xa) {
+  split_x(xa, x, T, H, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
 }  // namespace
+
+// Two blocks of 32 a thread: few enough CTAs that they, the roots' and the tiles' are resident at once (64 nodes of 2048
+// with 128 experts: 16 + 16 + 256 on 296 places).
+int split_x_rows(int T, int H, int E) {
+  const int gx = (E + kRE - 1) / kRE, per_row = gx * 256 * 2, blocks = T * (H / 32);
+  return (blocks + per_row - 1) / per_row;
+}
+int split_x_row_ctas(int E) { return (E + kRE - 1) / kRE; }
+int split_x_ctas(int T, int H) { return (T * (H / 32) + 255) / 256; }
+cudaError_t launch_split_x(const void* x, int T, int H, const XqArgs& xq, cudaStream_t s) {
+  k_split_x<<<split_x_ctas(T, H), 256, 0, s>>>(static_cast<const __nv_bfloat16*>(x), T, H, xq);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_router_logits(int dtype, const void* x, const void* w_router, const float* bias,
                                  float* logits, int T, int H, int E, float* zero_buf,
                                  size_t zero_floats, float* zero_buf2, size_t zero_floats2, int32_t* status,
                                  float* probs, int32_t* nat_idx, uint32_t* nat_mask, int k, int32_t* tile_done,
-                                 bool pdl, cudaStream_t s, long long* dbg, const RootArgs* root) {
+                                 bool pdl, cudaStream_t s, long long* dbg, const RootArgs* root, const XqArgs* xq) {
   if (!probs && !nat_idx) tile_done = nullptr;
   RootArgs ro = {};
   if (root) ro = *root;
+  XqArgs xa = {};
+  if (xq) xa = *xq;
+  if (xa.xq && dtype != ACM_BF16) return cudaErrorInvalidValue;
   if (ro.rows != 0 && (!ro.words || !ro.anc_words || ro.rows < 0 || ro.rows > kMaxEarlyBlocks)) return cudaErrorInvalidValue;
   cudaLaunchAttribute attr[1];
   set_pdl_attr(attr);
@@ -1015,7 +1074,7 @@ cudaError_t launch_router_logits(int dtype, const void* x, const void* w_router,
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
-  const dim3 grid((E + kRE - 1) / kRE, (T + kRT - 1) / kRT + ro.rows);
+  const dim3 grid((E + kRE - 1) / kRE, (T + kRT - 1) / kRT + ro.rows + (xa.xq ? xa.rows : 0));
   const int elt = dtype == ACM_F32 ? 4 : 2;
   size_t smem = static_cast<size_t>(kRT + kRE) * (static_cast<size_t>(H) * elt + 64);
   // At most two CTAs per SM (by asking for more shared memory than the tile needs): the grid then
@@ -1032,15 +1091,15 @@ cudaError_t launch_router_logits(int dtype, const void* x, const void* w_router,
     cfg.gridDim = grid; cfg.blockDim = dim3(kRT * kRE * 8); cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<const float*>(x), static_cast<const float*>(w_router), bias,
                               logits, T, H, E, n_chunks, zero_buf, zero_floats, zero_buf2, zero_floats2, status, probs, nat_idx, nat_mask, k,
-                              tile_done, dbg, ro);
+                              tile_done, dbg, ro, xa);
   } else {
-    auto kern = k_router_logits<__nv_bfloat16>;
+    auto kern = xa.xq ? k_router_logits<__nv_bfloat16, true> : k_router_logits<__nv_bfloat16, false>;
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (err != cudaSuccess) return err;
     cfg.gridDim = grid; cfg.blockDim = dim3(kRT * kRE * (32 / ElemTraits<__nv_bfloat16>::EPT)); cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<const __nv_bfloat16*>(x),
                               static_cast<const __nv_bfloat16*>(w_router), bias, logits, T, H, E, n_chunks, zero_buf,
-                              zero_floats, zero_buf2, zero_floats2, status, probs, nat_idx, nat_mask, k, tile_done, dbg, ro);
+                              zero_floats, zero_buf2, zero_floats2, status, probs, nat_idx, nat_mask, k, tile_done, dbg, ro, xa);
   }
 }
 

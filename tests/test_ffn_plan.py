@@ -9,10 +9,10 @@ from paper_2608_02989_b200 import acm
 SHAPES = [(2048, 768), (2048, 1024), (2048, 1408), (4096, 1536), (512, 256), (256, 64), (1024, 320)]
 
 
-def _check(n_act, H, I, G, n_pre=0):
+def _check(n_act, H, I, G, n_pre=0, mxfp4=False):
     tpe, kc1, h_tiles = I // 64, H // 128, H // 128
     kpe = (tpe + 1) // 2
-    pieces, n_seg = acm.ffn_plan(n_act, H, I, G, n_pre)
+    pieces, n_seg = acm.ffn_plan(n_act, H, I, G, n_pre, mxfp4)
     assert 1 <= n_seg <= 5
     gu = np.zeros((n_act * tpe, kc1), dtype=np.int32)           # gate/up stage (tile, chunk) -> times streamed
     dn = np.zeros((h_tiles, n_act * kpe), dtype=np.int32)       # down stage (output tile, expert slot * kpe + chunk)
@@ -110,3 +110,24 @@ def test_full_rounds_and_large_launches():
         tpe, kc1 = I // 64, H // 128
         ideal = (n_act * tpe * kc1 + n_act * (H // 128) * ((tpe + 1) // 2)) / 148
         assert load.max() <= ideal + kc1            # never more than a tile above the balanced load
+
+
+@pytest.mark.parametrize("H,I", [(H, I) for H, I in SHAPES if I % 128 == 0] + [(128, 128)])
+def test_mxfp4_plan_streams_every_stage_once_and_cuts_no_tile(H, I):
+    tpe = I // 64
+    for G in (148, 144, 141, 7):
+        for n_act in list(range(1, 34)) + [45, 64, 100, 128]:
+            for n_pre in sorted({0, 1, min(n_act, G // tpe), min(n_act, 8)}):
+                if n_pre <= n_act and n_pre * tpe <= G:
+                    load, pieces = _check(n_act, H, I, G, n_pre, mxfp4=True)
+                    gu = pieces[pieces[:, 2] == 1]
+                    assert (gu[:, 3] == 1).all()
+                    # no CTA has more than one tile above any other behind the anchors
+                    per_cta = np.bincount(gu[gu[:, 1] >= (1 if n_pre else 0)][:, 0], minlength=G)
+                    assert per_cta.max() - per_cta.min() <= 1
+                    # the first down group's experts are complete before the last round of tiles is dealt
+                    dn = pieces[pieces[:, 2] == 2]
+                    rest = gu[gu[:, 1] >= (1 if n_pre else 0)]
+                    if len(set(dn[:, 7].tolist())) == 2 and len(rest):
+                        rounds = -(-len(rest) // G)
+                        assert dn[:, 7].max() * tpe <= n_pre * tpe + (rounds - 1) * G

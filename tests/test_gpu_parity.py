@@ -1000,3 +1000,46 @@ def test_wide_batch_shares_one_pass_over_the_experts(c, sizes):
     with pytest.raises(acm.AcmError):
         ctx.moe_verify_batch(0, x[:70].contiguous(), [0, 70], torch.ones(70, device=DEV))
     ctx.close()
+
+
+@pytest.mark.parametrize("T,H,I", [(1, 128, 128), (16, 256, 384), (17, 2048, 128), (48, 1152, 640), (64, 4096, 256)])
+def test_mxfp4_activation_pieces(T, H, I):
+    """The MXFP4 kernel multiplies bf16 activations as two 8-bit pieces each: for ordinary rows, rows of any magnitude and
+    rows with outliers (features 2^11 times the others in the same block of 32 keep all their bits) the output is as close
+    to 64 bits as the bf16 kernel's on the dequantised weights -- in the fused call, whose router kernel stores the pieces,
+    and in acm_expert_ffn, which has a kernel for it.  A row that is not finite stays so, the others do not notice."""
+    cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, n_nodes=T, hidden=H, inter=I, n_experts=24, zipf_bias=False)
+    ctx = _ctx(cfg, n_layers=2)
+    w = _mx_layer(cfg)
+    x = wl.hidden_states(cfg, 0, DEV)
+    g = torch.Generator().manual_seed(7)
+    if T > 1:
+        x[1] *= 2.0 ** -30
+        x[T // 2] *= 2.0 ** 12
+        x[T - 1, torch.randint(0, H, (H // 64,), generator=g).to(DEV)] *= 2.0 ** 11
+    alpha = torch.ones(T, device=DEV)
+    ctx.set_layer_weights_mxfp4(0, w["w_router"], None, w["gate_up_tiles"], w["down_tiles"])
+    ctx.set_layer_weights(1, w["w_router"], None, w["gate_up_deq"], w["down_deq"])
+    out, idx, wt, _, _ = ctx.moe_verify(0, x, alpha, want=True)
+    bf16 = ctx.moe_verify(1, x, alpha)
+    alone = ctx.expert_ffn(0, x, idx, wt)
+    assert ctx.device_status() == acm.OK
+    ref = oracle.expert_ffn(x, idx.cpu().numpy(), wt.cpu().numpy(), w["gate_up_deq"], w["down_deq"])
+    rms = np.sqrt(np.mean(ref ** 2, axis=1, keepdims=True))
+
+    def off(o):                       # row by row: 2-norm of the error over that of the row
+        return np.sqrt(np.mean((o.double().cpu().numpy() - ref) ** 2, axis=1, keepdims=True)) / rms
+
+    # both round the activations between the two products to bf16, from sums that differ in the last bits only: a value on
+    # the edge rounds the other way now and then (2^-8 of one of I terms), which moves a row's error by a few per cent
+    for o in (out, alone):
+        assert (np.abs(o.double().cpu().numpy() - ref) <= FFN_TOL * rms).all()
+        assert (off(o) <= 1.1 * off(bf16) + 1e-4).all()
+    if T > 1:
+        x[T // 2, 5] = float("inf")
+        bad = ctx.expert_ffn(0, x, idx, wt)
+        assert not torch.isfinite(bad[T // 2]).any()
+        rest = [t for t in range(T) if t != T // 2]
+        assert torch.isfinite(bad[rest]).all()
+        assert float((bad[rest] - alone[rest]).abs().max()) <= 1e-3 * float(alone[rest].double().pow(2).mean().sqrt())
+    ctx.close()
