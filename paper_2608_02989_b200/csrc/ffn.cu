@@ -374,6 +374,12 @@ __device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t desc_a, uint
 __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
+// One lane of a converged warp (always the same one).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
+  return r != 0;
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
@@ -412,12 +418,6 @@ __device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint32_t tmem_a, uint64
 // byte of the scales' words).
 __device__ __forceinline__ uint32_t umma_mx_idesc(int n) {
   return (3u << 7) | (static_cast<uint32_t>(n >> 3) << 17) | (1u << 23) | (static_cast<uint32_t>(kTileM >> 7) << 27);
-}
-// One lane of a converged warp (always the same one).
-__device__ __forceinline__ bool elect_one() {
-  uint32_t r;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
-  return r != 0;
 }
 // Descriptor of an activation half-stage: rows of 64 bytes (64 K e4m3), 64-byte swizzle, groups of 8 rows 512 bytes apart.
 __device__ __forceinline__ uint64_t umma_smem_desc_64(uint32_t smem_addr) {
@@ -896,17 +896,26 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         while (global_timer() - t0 < 200000ull) {}
       }
     }
-#if ACM_FFN_MX
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
     // The whole warp walks the stages and one elected lane issues: the operands of an MMA are uniform registers, and
-    // in code that only lane 0 runs every one of them is moved there from a vector register first.
+    // in code that only lane 0 runs every one of them is moved there from a vector register first (four MMAs of an
+    // MXFP4 stage: 370 clocks to issue, 110 this way).
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+#if ACM_FFN_MX
     const uint32_t idesc = umma_mx_idesc(2 * p.n_pad);
     const uint64_t act_hi = umma_smem_desc_64(0);
     const uint32_t half_step = static_cast<uint32_t>(act_bytes) >> 5;      // (in 16-byte units) from one half-stage to the other
-    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
     const uint32_t act0 = (smem_u32(act_base) & 0x3ffffu) >> 4;
-    uint32_t s = 0, par = 0, act_slot = 0, b = 0, bpar = 1;
+    uint32_t act_slot = 0;
+    constexpr uint32_t kRing = kMxA;
+#else
+    const uint32_t idesc = umma_idesc(p.n_pad);
+    const uint64_t desc_hi = umma_smem_desc(0);
+    const uint32_t stage0 = (smem_u32(stage_base) & 0x3ffffu) >> 4;
+    constexpr uint32_t kRing = kStages;
+#endif
+    uint32_t s = 0, par = 0, b = 0, bpar = 1;
     bool ok = true;
     for (int si = 0; ok && __all_sync(0xffffffffu, have_seg(si, true)); ++si) {
       Sched sc(bars->plan.range[si]);
@@ -921,6 +930,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
           ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->full[s]), par, quit, kSiteStageFull));
           if (!ok) break;
           tc_fence_after();
+#if ACM_FFN_MX
           const uint32_t ta = tm + kAcc * kAccCols + s * kMxACols;
           const uint32_t sf = tm + kAcc * kAccCols + kMxA * kMxACols + s * kMxScaleCols;
           const uint64_t db = act_hi | (act0 + act_slot * (static_cast<uint32_t>(act_bytes) >> 4));
@@ -933,9 +943,25 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
             umma_commit(smem_u32(&bars->empty[s]));
             if (kc + 1 == nk) umma_commit(smem_u32(&bars->tfull[b]));
           }
-          __syncwarp();
           if (++act_slot == static_cast<uint32_t>(p.n_act)) act_slot = 0;
-          if (++s == kMxA) { s = 0; par ^= 1u; }
+#else
+          // descriptors: only the address field changes from stage to stage and atom to atom
+          const uint64_t da0 = desc_hi | (stage0 + s * (kStageBytes >> 4));
+          const uint64_t db0 = desc_hi | (stage0 + s * (kStageBytes >> 4) + (kABytes >> 4));
+          if (elect_one()) {
+#pragma unroll
+            for (int at = 0; at < kAtoms; ++at) {
+#pragma unroll
+              for (int kk = 0; kk < kBK / 16; ++kk)
+                umma_bf16(d_tmem, da0 + (at * (kAtomABytes >> 4) + 2 * kk), db0 + (at * (b_atom_bytes >> 4) + 2 * kk), idesc,
+                          (kc > 0 || at > 0 || kk > 0) ? 1u : 0u);
+            }
+            umma_commit(smem_u32(&bars->empty[s]));
+            if (kc + 1 == nk) umma_commit(smem_u32(&bars->tfull[b]));
+          }
+#endif
+          __syncwarp();
+          if (++s == kRing) { s = 0; par ^= 1u; }
         }
         if (++b == kAcc) { b = 0; bpar ^= 1u; }
       }
@@ -946,53 +972,6 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       const unsigned long long t0 = global_timer();
       while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
     }
-#else
-  } else if (warp == 1) {
-    // ------------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = umma_idesc(p.n_pad);
-      const uint64_t desc_hi = umma_smem_desc(0);
-      uint32_t it = 0, f = 0;
-      bool ok = true;
-      for (int si = 0; ok && have_seg(si, true); ++si) {
-        Sched sc(bars->plan.range[si]);
-        int tile, k0, k1;
-        while (ok && sc.next(tile, k0, k1)) {
-          const uint32_t b = f % kAcc;
-          if (!(ok = mbar_wait(smem_u32(&bars->tempty[b]), ((f / kAcc) & 1u) ^ 1u, quit, kSiteAccEmpty))) break;
-          tc_fence_after();
-          const uint32_t d_tmem = tmem_base + b * kAccCols;
-          for (int kc = k0; kc < k1; ++kc, ++it) {
-            const uint32_t s = it % kStages, par = (it / kStages) & 1u;
-            if (!(ok = mbar_wait(smem_u32(&bars->full[s]), par, quit, kSiteStageFull))) break;
-            tc_fence_after();
-            // descriptors: only the address field changes from stage to stage and atom to atom
-            const uint32_t sa = smem_u32(stage_base) + s * kStageBytes;
-            const uint64_t da0 = desc_hi | ((sa & 0x3ffffu) >> 4);
-            const uint64_t db0 = desc_hi | (((sa + kABytes) & 0x3ffffu) >> 4);
-#pragma unroll
-            for (int at = 0; at < kAtoms; ++at) {
-#pragma unroll
-              for (int kk = 0; kk < kBK / 16; ++kk) {
-                umma_bf16(d_tmem, da0 + (at * (kAtomABytes >> 4) + 2 * kk), db0 + (at * (b_atom_bytes >> 4) + 2 * kk), idesc,
-                          (kc > k0 || at > 0 || kk > 0) ? 1u : 0u);
-              }
-            }
-            umma_commit(smem_u32(&bars->empty[s]));
-          }
-          if (!ok) break;
-          umma_commit(smem_u32(&bars->tfull[b]));
-          ++f;
-        }
-      }
-      if (!ok) {
-        // giving up: wait (bounded) for the MMAs already issued before TMEM is released
-        umma_commit(smem_u32(&bars->drained));
-        const unsigned long long t0 = global_timer();
-        while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
-      }
-    }
-#endif
 #if ACM_FFN_MX
   } else if (warp == 6) {
     // ------------------------------------------------------------------ activation producer
