@@ -212,6 +212,6 @@ cudaError_t launch_ffn_mxfp4(const FfnLaunch& p, const FfnMaps& maps, const CUte
 cudaError_t launch_ffn_f32(const float* x, const float* gate_up, const float* down,
                            const float* shared_gate_up, const float* shared_down, int n_shared,
                            const int32_t* idx, const float* w, float* hbuf, float* out, int T, int H,
-                           int I, int E, int k, cudaStream_t s);
+                           int I, int E, int k, bool pdl, cudaStream_t s);
 
 }  // namespace acm

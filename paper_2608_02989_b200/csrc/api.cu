@@ -818,7 +818,7 @@ acm_status acm_expert_ffn(acm_ctx* c, int layer, const void* x, int T, const int
     ACM_CUDA(launch_ffn_f32(static_cast<const float*>(x), static_cast<const float*>(L.gate_up),
                             static_cast<const float*>(L.down), static_cast<const float*>(L.shared_gate_up),
                             static_cast<const float*>(L.shared_down), d.n_shared, idx, w,
-                            static_cast<float*>(c->ws.hbuf), out, T, d.hidden, d.inter, d.n_experts, d.top_k, s));
+                            static_cast<float*>(c->ws.hbuf), out, T, d.hidden, d.inter, d.n_experts, d.top_k, false, s));
     c->launches += 2;
     return ACM_OK;
   }
@@ -923,7 +923,7 @@ acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const flo
     ACM_CUDA(launch_ffn_f32(static_cast<const float*>(x), static_cast<const float*>(L.gate_up),
                             static_cast<const float*>(L.down), static_cast<const float*>(L.shared_gate_up),
                             static_cast<const float*>(L.shared_down), d.n_shared, c->ws.idx, c->ws.w,
-                            static_cast<float*>(c->ws.hbuf), out, T, d.hidden, d.inter, E, k, s));
+                            static_cast<float*>(c->ws.hbuf), out, T, d.hidden, d.inter, E, k, c->pdl, s));
     c->launches += 2;
   } else if (!L.has_resident) {
     st = run_ffn_list(c, L, x, T, 0, out, s, nullptr, stats_dev, true, early_epoch, nullptr, 0, anchors_first);

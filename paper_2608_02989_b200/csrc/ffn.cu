@@ -1578,56 +1578,121 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 
 #if !ACM_FFN_MX
 // ---------------------------------------------------------------------------------- f32 path
-// h[t][j][i] = silu(g) * u for routed slot j < k (expert idx[t][j]) and shared slot j >= k.
-__global__ void k_ffn_f32_gate_up(const float* __restrict__ x, const float* __restrict__ gate_up,
-                                  const float* __restrict__ shared_gate_up, const int32_t* __restrict__ idx,
-                                  float* __restrict__ hbuf, int T, int H, int I, int E, int k, int n_shared) {
-  const int slots = k + n_shared;
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= T * slots * I) return;
-  const int i = warp % I, j = (warp / I) % slots, t = warp / (I * slots);
-  int e = j < k ? idx[t * k + j] : j - k;
-  if (j < k && e >= E) e = -1;                 // an id outside the layer is an empty slot, like -1
-  const float* base = j < k ? gate_up : shared_gate_up;
-  float h = 0.0f;
-  if (e >= 0) {
-    const float* g_row = base + (static_cast<size_t>(e) * 2 * I + i) * H;
-    const float* u_row = g_row + static_cast<size_t>(I) * H;
-    const float* xr = x + static_cast<size_t>(t) * H;
-    float g = 0.f, u = 0.f;
-    for (int hh = lane; hh < H; hh += 32) {
-      g = fmaf(g_row[hh], xr[hh], g);
-      u = fmaf(u_row[hh], xr[hh], u);
-    }
-    for (int s = 16; s >= 1; s >>= 1) {
-      g += __shfl_xor_sync(0xffffffffu, g, s);
-      u += __shfl_xor_sync(0xffffffffu, u, s);
-    }
-    h = (g / (1.0f + expf(-g))) * u;
-  }
-  if (lane == 0) hbuf[(static_cast<size_t>(t) * slots + j) * I + i] = h;
+// A few MFLOP in L2: what counts is the chain of latencies, so both kernels are dependent launches in the fused call (the
+// second one's CTAs are resident before the first is done), a warp has the loads of four rows in flight, and rows are
+// read 16 bytes a lane where shapes and pointers allow (kVec).  8 nodes, 256 x 512, top-2 of 16, the whole layer:
+// 24.9 -> 23.5 us (by then as long as its launches take on the host).
+constexpr int kF32Rows = 4;      // weight rows (of gate and of up; of down) a warp works on at a time
+
+// Four sums, one per row, over the warp's lanes: lane r < 4 returns that of row r (exchanges of two rows' halves instead of
+// a full reduction per row).
+__device__ __forceinline__ float reduce_rows(const float (&a)[kF32Rows], int lane) {
+  const bool up2 = lane & 2, up1 = lane & 1;
+  const float s0 = (up2 ? a[2] : a[0]) + __shfl_xor_sync(0xffffffffu, up2 ? a[0] : a[2], 2);
+  const float s1 = (up2 ? a[3] : a[1]) + __shfl_xor_sync(0xffffffffu, up2 ? a[1] : a[3], 2);
+  float v = (up1 ? s1 : s0) + __shfl_xor_sync(0xffffffffu, up1 ? s0 : s1, 1);
+#pragma unroll
+  for (int s = 16; s >= 4; s >>= 1) v += __shfl_xor_sync(0xffffffffu, v, s);
+  return v;
 }
 
-__global__ void k_ffn_f32_down(const float* __restrict__ down, const float* __restrict__ shared_down,
-                               const int32_t* __restrict__ idx, const float* __restrict__ w,
-                               const float* __restrict__ hbuf, float* __restrict__ out, int T, int H, int I,
-                               int E, int k, int n_shared) {
-  const int slots = k + n_shared;
+// h[t][j][i] = silu(g) * u for routed slot j < k (expert idx[t][j]) and shared slot j >= k.
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+k_ffn_f32_gate_up(const float* x, const float* __restrict__ gate_up,
+                  const float* __restrict__ shared_gate_up, const int32_t* idx,
+                  float* __restrict__ hbuf, int T, int H, int I, int E, int k, int n_shared) {
+  const int slots = k + n_shared, groups = (I + kF32Rows - 1) / kF32Rows;
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= T * H) return;
-  const int hh = warp % H, t = warp / H;
-  float y = 0.f;
-  for (int j = 0; j < slots; ++j) {
-    const int e = j < k ? idx[t * k + j] : j - k;
-    if (e < 0 || (j < k && e >= E)) continue;
-    const float* d_row = (j < k ? down : shared_down) + (static_cast<size_t>(e) * H + hh) * I;
-    const float* hr = hbuf + (static_cast<size_t>(t) * slots + j) * I;
-    float acc = 0.f;
-    for (int i = lane; i < I; i += 32) acc = fmaf(d_row[i], hr[i], acc);
-    for (int s = 16; s >= 1; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-    y += (j < k ? w[t * k + j] : 1.0f) * acc;
+  griddep_wait();
+  griddep_launch_dependents();      // (behind the wait: what the next kernel waits for then includes the routes)
+  if (warp >= T * slots * groups) return;
+  const int i0 = (warp % groups) * kF32Rows, j = (warp / groups) % slots, t = warp / (groups * slots);
+  int e = j < k ? idx[t * k + j] : j - k;
+  if (j < k && e >= E) e = -1;                 // an id outside the layer is an empty slot, like -1
+  float g[kF32Rows] = {}, u[kF32Rows] = {};
+  if (e >= 0) {
+    const float* base = (j < k ? gate_up : shared_gate_up) + static_cast<size_t>(e) * 2 * I * H;
+    const float* xr = x + static_cast<size_t>(t) * H;
+    const float* g_row[kF32Rows];
+#pragma unroll
+    for (int r = 0; r < kF32Rows; ++r) g_row[r] = base + static_cast<size_t>(min(i0 + r, I - 1)) * H;
+    const size_t to_up = static_cast<size_t>(I) * H;
+    if constexpr (kVec) {
+#pragma unroll 2
+      for (int hh = 4 * lane; hh < H; hh += 128) {
+        const float4 xv = *reinterpret_cast<const float4*>(xr + hh);
+#pragma unroll
+        for (int r = 0; r < kF32Rows; ++r) {
+          const float4 gv = *reinterpret_cast<const float4*>(g_row[r] + hh), uv = *reinterpret_cast<const float4*>(g_row[r] + to_up + hh);
+          g[r] = fmaf(gv.x, xv.x, fmaf(gv.y, xv.y, fmaf(gv.z, xv.z, fmaf(gv.w, xv.w, g[r]))));
+          u[r] = fmaf(uv.x, xv.x, fmaf(uv.y, xv.y, fmaf(uv.z, xv.z, fmaf(uv.w, xv.w, u[r]))));
+        }
+      }
+    } else {
+      for (int hh = lane; hh < H; hh += 32) {
+        const float xv = xr[hh];
+#pragma unroll
+        for (int r = 0; r < kF32Rows; ++r) {
+          g[r] = fmaf(g_row[r][hh], xv, g[r]);
+          u[r] = fmaf(g_row[r][to_up + hh], xv, u[r]);
+        }
+      }
+    }
   }
-  if (lane == 0) out[static_cast<size_t>(t) * H + hh] = y;
+  const float gs = reduce_rows(g, lane), us = reduce_rows(u, lane);
+  if (lane < kF32Rows && i0 + lane < I)
+    hbuf[(static_cast<size_t>(t) * slots + j) * I + i0 + lane] = e >= 0 ? (gs / (1.0f + expf(-gs))) * us : 0.0f;
+}
+
+template <bool kVec>
+__global__ void __launch_bounds__(256)
+k_ffn_f32_down(const float* __restrict__ down, const float* __restrict__ shared_down, const int32_t* idx, const float* w,
+               const float* hbuf, float* __restrict__ out, int T, int H, int I, int E, int k, int n_shared) {
+  const int slots = k + n_shared, groups = (H + kF32Rows - 1) / kF32Rows;
+  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  griddep_launch_dependents();
+  griddep_wait();
+  if (warp >= T * groups) return;
+  const int h0 = (warp % groups) * kF32Rows, t = warp / groups;
+  // the node's experts and weights, a lane per slot (at most kMaxTopK + kMaxShared)
+  int my_e = -1;
+  float my_w = 1.0f;
+  if (lane < slots) {
+    my_e = lane < k ? idx[t * k + lane] : lane - k;
+    if (lane < k) {
+      my_w = w[t * k + lane];
+      if (my_e >= E) my_e = -1;
+    }
+  }
+  float y = 0.f;
+#pragma unroll 2
+  for (int j = 0; j < slots; ++j) {
+    const int e = __shfl_sync(0xffffffffu, my_e, j);
+    if (e < 0) continue;
+    const float* base = (j < k ? down : shared_down) + static_cast<size_t>(e) * H * I;
+    const float* hr = hbuf + (static_cast<size_t>(t) * slots + j) * I;
+    float acc[kF32Rows] = {};
+    if constexpr (kVec) {
+#pragma unroll 4
+      for (int i = 4 * lane; i < I; i += 128) {
+        const float4 hv = *reinterpret_cast<const float4*>(hr + i);
+#pragma unroll
+        for (int r = 0; r < kF32Rows; ++r) {
+          const float4 dv = *reinterpret_cast<const float4*>(base + static_cast<size_t>(min(h0 + r, H - 1)) * I + i);
+          acc[r] = fmaf(dv.x, hv.x, fmaf(dv.y, hv.y, fmaf(dv.z, hv.z, fmaf(dv.w, hv.w, acc[r]))));
+        }
+      }
+    } else {
+      for (int i = lane; i < I; i += 32) {
+        const float hv = hr[i];
+#pragma unroll
+        for (int r = 0; r < kF32Rows; ++r) acc[r] = fmaf(base[static_cast<size_t>(min(h0 + r, H - 1)) * I + i], hv, acc[r]);
+      }
+    }
+    y = fmaf(__shfl_sync(0xffffffffu, my_w, j), reduce_rows(acc, lane), y);
+  }
+  if (lane < kF32Rows && h0 + lane < H) out[static_cast<size_t>(t) * H + h0 + lane] = y;
 }
 
 #endif   // !ACM_FFN_MX
@@ -1738,17 +1803,26 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
 cudaError_t launch_ffn_f32(const float* x, const float* gate_up, const float* down,
                            const float* shared_gate_up, const float* shared_down, int n_shared,
                            const int32_t* idx, const float* w, float* hbuf, float* out, int T, int H,
-                           int I, int E, int k, cudaStream_t s) {
+                           int I, int E, int k, bool pdl, cudaStream_t s) {
   const int slots = k + n_shared;
-  const long long warps1 = static_cast<long long>(T) * slots * I;
-  k_ffn_f32_gate_up<<<static_cast<unsigned>((warps1 * 32 + 255) / 256), 256, 0, s>>>(x, gate_up, shared_gate_up, idx, hbuf,
-                                                                                   T, H, I, E, k, n_shared);
-  cudaError_t err = cudaGetLastError();
+  auto aligned = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  const bool vec = H % 4 == 0 && I % 4 == 0 && aligned(x) && aligned(gate_up) && aligned(down) && aligned(hbuf) &&
+                   (n_shared == 0 || (aligned(shared_gate_up) && aligned(shared_down)));
+  cudaLaunchAttribute attr[1];
+  set_pdl_attr(attr);
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  auto blocks = [](long long warps) { return dim3(static_cast<unsigned>((warps * 32 + 255) / 256)); };
+  cfg.gridDim = blocks(static_cast<long long>(T) * slots * ((I + kF32Rows - 1) / kF32Rows));
+  cudaError_t err = cudaLaunchKernelEx(&cfg, vec ? k_ffn_f32_gate_up<true> : k_ffn_f32_gate_up<false>, x, gate_up, shared_gate_up,
+                                       idx, hbuf, T, H, I, E, k, n_shared);
   if (err != cudaSuccess) return err;
-  const long long warps2 = static_cast<long long>(T) * H;
-  k_ffn_f32_down<<<static_cast<unsigned>((warps2 * 32 + 255) / 256), 256, 0, s>>>(down, shared_down, idx, w, hbuf, out, T,
-                                                                                H, I, E, k, n_shared);
-  return cudaGetLastError();
+  cfg.gridDim = blocks(static_cast<long long>(T) * ((H + kF32Rows - 1) / kF32Rows));
+  return cudaLaunchKernelEx(&cfg, vec ? k_ffn_f32_down<true> : k_ffn_f32_down<false>, down, shared_down, idx, w,
+                            static_cast<const float*>(hbuf), out, T, H, I, E, k, n_shared);
 }
 
 #endif   // !ACM_FFN_MX
@@ -1794,7 +1868,7 @@ extern "C" acm_status acm_expert_ffn_f32_noalloc(const float* x, int T, int hidd
     scratch = g_noalloc_ptr[dev];
   }
   const cudaError_t err = acm::launch_ffn_f32(x, w_gate_up, w_down, nullptr, nullptr, 0, idx, w, scratch, out, T, hidden,
-                                              inter, n_experts, top_k, static_cast<cudaStream_t>(stream));
+                                              inter, n_experts, top_k, false, static_cast<cudaStream_t>(stream));
   return err == cudaSuccess ? ACM_OK : ACM_ERR_CUDA;
 }
 #endif   // !ACM_FFN_MX
