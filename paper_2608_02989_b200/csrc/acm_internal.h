@@ -144,8 +144,8 @@ int split_x_rows(int T, int H, int E);
 int split_x_row_ctas(int E);
 int split_x_ctas(int T, int H);
 cudaError_t launch_split_x(const void* x, int T, int H, const XqArgs& xq, cudaStream_t s);
-cudaError_t launch_select(const SelectArgs& a, int T, int E, int k, cudaStream_t s);
-cudaError_t launch_route(const RouteArgs& a, int T, int E, int k, cudaStream_t s);
+cudaError_t launch_select(const SelectArgs& a, int T, int E, int k, bool pdl, cudaStream_t s);
+cudaError_t launch_route(const RouteArgs& a, int T, int E, int k, bool pdl, cudaStream_t s);
 // The fused calls' stages 1b-3 in ONE launch, a cluster of select_ctas_per_block(widest block) CTAs per block of `bd`
 // (a single block: n_blocks = 1, off = {0, T}): softmax and natural top-k of the logits in ra.logits, selection
 // (unless mask_override, single block only), routes, the FFN kernel's routing inputs.  The per-block outputs of `sa`
@@ -155,9 +155,9 @@ int select_ctas_per_block(int widest);
 cudaError_t select_configure();   // the kernel's function attributes, once per device (when a context is created)
 cudaError_t launch_softmax_select_route(const SelectArgs& sa, const RouteArgs& ra, const BatchDesc& bd,
                                         const uint32_t* mask_override, int E, int k, bool pdl, cudaStream_t s);
-// routes given by the caller -> activated mask, weight table (both cleared first) and cleared `ready`
-cudaError_t launch_routes_to_table(const int32_t* idx, const float* w, uint32_t* act_mask, float* wtab,
-                                   int32_t* ready, int T, int E, int k, cudaStream_t s);
+// routes given by the caller -> activated mask, weight table, cleared `ready` and cleared output
+cudaError_t launch_routes_to_table(const int32_t* idx, const float* w, uint32_t* act_mask, float* wtab, int32_t* ready, int T,
+                                   int E, int k, float* out, size_t out_floats, bool pdl, cudaStream_t s);
 
 // ---- launchers (ffn.cu) -----------------------------------------------------------------
 struct FfnMaps {               // TMA descriptors of one layer (bf16 path)

@@ -766,7 +766,7 @@ acm_status acm_router(acm_ctx* c, int layer, const void* x, int T, float* logits
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // softmax and natural top-k are finished inside the same launch (last CTA of each node tile)
   ACM_CUDA(launch_router_logits(d.dtype, x, L.w_router, L.bias, logits, T, d.hidden, d.n_experts, nullptr, 0,
-                                nullptr, 0, c->ws.status, probs, nat_idx, nullptr, d.top_k, c->ws.tile_done, false, s,
+                                nullptr, 0, c->ws.status, probs, nat_idx, nullptr, d.top_k, c->ws.tile_done, c->pdl, s,
                                 c->trace ? reinterpret_cast<long long*>(c->trace) + 32 * c->sm_count : nullptr));
   c->launches += 1;
   return ACM_OK;
@@ -787,7 +787,7 @@ acm_status acm_select_eligible(acm_ctx* c, const float* probs, const int32_t* na
   a.n_anchor_nodes = n_anchor_nodes; a.resident = params->residency ? resident_mask : nullptr; a.prm = *params;
   a.mask_out = eligible_mask; a.unpruned_out = unpruned_mask; a.count_out = eligible_count;
   a.demand_out = demand; a.stats_out = stats;
-  ACM_CUDA(launch_select(a, T, c->desc.n_experts, c->desc.top_k, static_cast<cudaStream_t>(stream)));
+  ACM_CUDA(launch_select(a, T, c->desc.n_experts, c->desc.top_k, c->pdl, static_cast<cudaStream_t>(stream)));
   c->launches += 1;
   return ACM_OK;
 }
@@ -799,7 +799,7 @@ acm_status acm_route_restricted(acm_ctx* c, const float* logits, const uint32_t*
   RouteArgs a = {};
   a.logits = logits; a.mask = eligible_mask; a.idx_out = idx; a.w_out = w;
   a.weighting = c->desc.weighting; a.routed_scale = c->desc.routed_scale;
-  ACM_CUDA(launch_route(a, T, c->desc.n_experts, c->desc.top_k, static_cast<cudaStream_t>(stream)));
+  ACM_CUDA(launch_route(a, T, c->desc.n_experts, c->desc.top_k, c->pdl, static_cast<cudaStream_t>(stream)));
   c->launches += 1;
   return ACM_OK;
 }
@@ -818,12 +818,12 @@ acm_status acm_expert_ffn(acm_ctx* c, int layer, const void* x, int T, const int
     ACM_CUDA(launch_ffn_f32(static_cast<const float*>(x), static_cast<const float*>(L.gate_up),
                             static_cast<const float*>(L.down), static_cast<const float*>(L.shared_gate_up),
                             static_cast<const float*>(L.shared_down), d.n_shared, idx, w,
-                            static_cast<float*>(c->ws.hbuf), out, T, d.hidden, d.inter, d.n_experts, d.top_k, false, s));
+                            static_cast<float*>(c->ws.hbuf), out, T, d.hidden, d.inter, d.n_experts, d.top_k, c->pdl, s));
     c->launches += 2;
     return ACM_OK;
   }
-  ACM_CUDA(cudaMemsetAsync(out, 0, sizeof(float) * static_cast<size_t>(T) * d.hidden, s));
-  ACM_CUDA(launch_routes_to_table(idx, w, c->ws.act_mask, c->ws.wtab, c->ws.ready, T, d.n_experts, d.top_k, s));
+  ACM_CUDA(launch_routes_to_table(idx, w, c->ws.act_mask, c->ws.wtab, c->ws.ready, T, d.n_experts, d.top_k, out,
+                                  static_cast<size_t>(T) * d.hidden, c->pdl, s));
   c->launches += 1;
   if (L.mx) {
     ACM_CUDA(launch_split_x(x, T, d.hidden, xq_args(c, T), s));

@@ -221,7 +221,8 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
   return false;
 }
 
-// Blocks of 32 hidden states into the FFN kernel's pieces, a thread per block of a node: thread i of n.
+// Blocks of 32 hidden states into the FFN kernel's pieces, a thread per block of a node: thread i of n.  (x may be written
+// while a dependent launch is already resident: never through the read-only path.)
 __device__ __forceinline__ void split_x(const XqArgs& xa, const __nv_bfloat16* x, int T, int H, int i, int n) {
   const int per_node = H / 32;
   for (; i < T * per_node; i += n) {
@@ -229,7 +230,7 @@ __device__ __forceinline__ void split_x(const XqArgs& xa, const __nv_bfloat16* x
     uint32_t w[16];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const uint4 v = *reinterpret_cast<const uint4*>(x + static_cast<size_t>(t) * H + 32 * block + 8 * j);
+      const uint4 v = __ldcg(reinterpret_cast<const uint4*>(x + static_cast<size_t>(t) * H + 32 * block + 8 * j));
       w[4 * j] = v.x; w[4 * j + 1] = v.y; w[4 * j + 2] = v.z; w[4 * j + 3] = v.w;
     }
     MxBlock k;
@@ -824,6 +825,8 @@ __device__ __forceinline__ void publish_routes_local(uint32_t* s_act, int k, int
 
 __global__ void __launch_bounds__(kSelThreads) k_select(SelectArgs a, int T, int E, int k) {
   __shared__ StageSmem sm;
+  griddep_launch_dependents();
+  griddep_wait();
   stage_select<false>(a, sm, T, E, k, nullptr, true);
 }
 
@@ -831,6 +834,8 @@ __global__ void __launch_bounds__(kSelThreads) k_select(SelectArgs a, int T, int
 __global__ void __launch_bounds__(kSelThreads) k_route(RouteArgs a, int T, int E, int k) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int t = blockIdx.x * kNodesPerCta + warp;
+  griddep_launch_dependents();
+  griddep_wait();
   if (t >= T) return;
   float z[4];
   uint32_t mask_w[4];
@@ -1020,20 +1025,42 @@ k_softmax_select_route(SelectArgs sa, RouteArgs ra, BatchDesc bd, const uint32_t
   }
 }
 
-// Routes given by the caller (acm_expert_ffn) -> the FFN kernel's inputs.  One CTA.
+// Routes given by the caller (acm_expert_ffn) -> the FFN kernel's inputs, and the output it accumulates into cleared.  The
+// first four CTAs own a mask word each and gather its 32 experts' rows of the weight table (a thread looks through its
+// node's k choices: nothing is cleared first and scattered into afterwards), the others clear `out`.
+constexpr int kTableCtas = kMaskWords;
 __global__ void __launch_bounds__(512) k_routes_to_table(const int32_t* idx, const float* w, uint32_t* act_mask,
-                                                         float* wtab, int32_t* ready, int T, int E, int k) {
-  for (int i = threadIdx.x; i < kMaxExperts * kWtabStride; i += blockDim.x) wtab[i] = 0.0f;
-  for (int i = threadIdx.x; i < 2 * kMaxSlots; i += blockDim.x) ready[i] = 0;
-  if (threadIdx.x < kMaskWords) act_mask[threadIdx.x] = 0u;
-  __syncthreads();
-  for (int i = threadIdx.x; i < T * k; i += blockDim.x) {
-    const int e = idx[i];
-    if (e >= 0 && e < E) {
-      atomicOr(act_mask + (e >> 5), 1u << (e & 31));
-      wtab[static_cast<size_t>(e) * kWtabStride + i / k] = w[i];
-    }
+                                                         float* wtab, int32_t* ready, int T, int E, int k, float* out,
+                                                         size_t out_floats) {
+  griddep_launch_dependents();
+  griddep_wait();
+  if (blockIdx.x >= kTableCtas) {
+    float4* z4 = reinterpret_cast<float4*>(out);
+    for (size_t i = static_cast<size_t>(blockIdx.x - kTableCtas) * blockDim.x + threadIdx.x; i < out_floats / 4;
+         i += static_cast<size_t>(gridDim.x - kTableCtas) * blockDim.x)
+      z4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    return;
   }
+  __shared__ uint32_t s_word;
+  if (threadIdx.x == 0) s_word = 0u;
+  __syncthreads();
+  const int t = threadIdx.x % kWtabStride, e0 = 32 * blockIdx.x;
+  int mine[kMaxTopK];
+#pragma unroll
+  for (int j = 0; j < kMaxTopK; ++j) mine[j] = (t < T && j < k) ? idx[t * k + j] : -1;
+  for (int el = threadIdx.x / kWtabStride; el < 32; el += blockDim.x / kWtabStride) {
+    const int e = e0 + el;
+    int at = -1;
+#pragma unroll
+    for (int j = 0; j < kMaxTopK; ++j)
+      if (mine[j] == e && e < E) at = j;
+    wtab[static_cast<size_t>(e) * kWtabStride + t] = at >= 0 ? w[t * k + at] : 0.0f;
+    if (__ballot_sync(0xffffffffu, at >= 0) != 0u && (threadIdx.x & 31) == 0) atomicOr(&s_word, 1u << el);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) act_mask[blockIdx.x] = s_word;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < 2 * kMaxSlots; i += blockDim.x) ready[i] = 0;
 }
 
 // The hidden states' pieces for routes given by the caller (acm_expert_ffn).
@@ -1086,16 +1113,12 @@ cudaError_t launch_router_logits(int dtype, const void* x, const void* w_router,
   if ((static_cast<size_t>(H) * elt) % 16 != 0) return cudaErrorInvalidValue;   // rows are copied in 16-byte units
   if (dtype == ACM_F32) {
     auto kern = k_router_logits<float>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (err != cudaSuccess) return err;
     cfg.gridDim = grid; cfg.blockDim = dim3(kRT * kRE * 8); cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<const float*>(x), static_cast<const float*>(w_router), bias,
                               logits, T, H, E, n_chunks, zero_buf, zero_floats, zero_buf2, zero_floats2, status, probs, nat_idx, nat_mask, k,
                               tile_done, dbg, ro, xa);
   } else {
     auto kern = xa.xq ? k_router_logits<__nv_bfloat16, true> : k_router_logits<__nv_bfloat16, false>;
-    cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-    if (err != cudaSuccess) return err;
     cfg.gridDim = grid; cfg.blockDim = dim3(kRT * kRE * (32 / ElemTraits<__nv_bfloat16>::EPT)); cfg.dynamicSmemBytes = smem;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<const __nv_bfloat16*>(x),
                               static_cast<const __nv_bfloat16*>(w_router), bias, logits, T, H, E, n_chunks, zero_buf,
@@ -1103,17 +1126,39 @@ cudaError_t launch_router_logits(int dtype, const void* x, const void* w_router,
   }
 }
 
-cudaError_t launch_select(const SelectArgs& a, int T, int E, int k, cudaStream_t s) {
-  k_select<<<1, kSelThreads, 0, s>>>(a, T, E, k);
-  return cudaGetLastError();
+// The stages' own launches.  `pdl`: their CTAs may become resident while the kernel before them finishes (each waits for it
+// before its first access to global memory), which takes the launch's latency off a caller's chain of stages.
+template <typename... P, typename... A>
+cudaError_t launch_plain(void (*kern)(P...), dim3 grid, dim3 block, bool pdl, cudaStream_t s, A... args) {
+  cudaLaunchAttribute attr[1];
+  set_pdl_attr(attr);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-cudaError_t launch_route(const RouteArgs& a, int T, int E, int k, cudaStream_t s) {
-  k_route<<<(T + kNodesPerCta - 1) / kNodesPerCta, kSelThreads, 0, s>>>(a, T, E, k);
-  return cudaGetLastError();
+cudaError_t launch_select(const SelectArgs& a, int T, int E, int k, bool pdl, cudaStream_t s) {
+  return launch_plain(k_select, dim3(1), dim3(kSelThreads), pdl, s, a, T, E, k);
+}
+
+cudaError_t launch_route(const RouteArgs& a, int T, int E, int k, bool pdl, cudaStream_t s) {
+  return launch_plain(k_route, dim3((T + kNodesPerCta - 1) / kNodesPerCta), dim3(kSelThreads), pdl, s, a, T, E, k);
 }
 
 cudaError_t select_configure() {
+  // (the router kernels' tile of H-element rows may be as large as a CTA's shared memory: see launch_router_logits)
+  for (const void* kern : {reinterpret_cast<const void*>(k_router_logits<float, false>), reinterpret_cast<const void*>(k_router_logits<__nv_bfloat16, false>),
+                           reinterpret_cast<const void*>(k_router_logits<__nv_bfloat16, true>)}) {
+    cudaFuncAttributes fa;
+    cudaError_t err = cudaFuncGetAttributes(&fa, kern);
+    if (err != cudaSuccess) return err;
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448 - static_cast<int>(fa.sharedSizeBytes));
+    if (err != cudaSuccess) return err;
+  }
   return cudaFuncSetAttribute(k_softmax_select_route, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(kFusedSmemRequest));
 }
@@ -1145,10 +1190,10 @@ cudaError_t launch_softmax_select_route(const SelectArgs& sa, const RouteArgs& r
   return cudaLaunchKernelEx(&cfg, k_softmax_select_route, sa, ra, bd, mask_override, E, k);
 }
 
-cudaError_t launch_routes_to_table(const int32_t* idx, const float* w, uint32_t* act_mask, float* wtab,
-                                   int32_t* ready, int T, int E, int k, cudaStream_t s) {
-  k_routes_to_table<<<1, 512, 0, s>>>(idx, w, act_mask, wtab, ready, T, E, k);
-  return cudaGetLastError();
+cudaError_t launch_routes_to_table(const int32_t* idx, const float* w, uint32_t* act_mask, float* wtab, int32_t* ready, int T,
+                                   int E, int k, float* out, size_t out_floats, bool pdl, cudaStream_t s) {
+  return launch_plain(k_routes_to_table, dim3(kTableCtas + 32), dim3(512), pdl, s, idx, w, act_mask, wtab, ready, T, E, k, out,
+                      out_floats);
 }
 
 }  // namespace acm
