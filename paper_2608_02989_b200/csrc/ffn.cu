@@ -777,12 +777,10 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     }
     return good;
   };
-#if ACM_FFN_MX
   // The CTAs walk the K-chunks of their (whole) tiles from different ones on: in step, all of them would fetch the same
   // chunk of the hidden states at the same time, from the same few slices of L2.
   const int k_first = cta % kc1;
   auto k_rot = [&](int kc) { return kc + k_first < kc1 ? kc + k_first : kc + k_first - kc1; };
-#endif
 
   if (warp == 0) {
     // ------------------------------------------------------------------ weight producer
@@ -810,6 +808,9 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #if !ACM_FFN_MX
             const CUtensorMap* gu = pick_map(entry_src(ent), &maps.gate_up, &maps.shared_gate_up, &maps.staged_gate_up);
 #endif
+#if !ACM_FFN_MX
+            int kk = (k0 == 0 && k1 == kc1) ? k_rot(0) : k0;      // the K-chunk of stage kc
+#endif
             for (int kc = k0; kc < k1; ++kc) {
 #if ACM_FFN_MX
               if (!(ok = mbar_wait(smem_u32(&bars->raw_empty[s]), par ^ 1u, quit, kSitePackedFree))) break;
@@ -824,8 +825,9 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
               const uint32_t full = smem_u32(&bars->full[s]);
               const uint32_t sa = smem_u32(stage_base) + s * kStageBytes;
               mbar_expect_tx(full, kABytes + b_bytes);
-              tma_load_5d(sa, gu, full, 0, r0, 0, kc * kAtoms, eidx, pol_w);   // 64 gate + 64 up rows, 2 atoms
-              tma_load_3d(sa + kABytes, &x_map, full, 0, 0, kc * kAtoms, pol_x);
+              tma_load_5d(sa, gu, full, 0, r0, 0, kk * kAtoms, eidx, pol_w);   // 64 gate + 64 up rows, 2 atoms
+              tma_load_3d(sa + kABytes, &x_map, full, 0, 0, kk * kAtoms, pol_x);
+              if (++kk == kc1) kk = 0;
               ++n_armed;
               if (++s == kStages) { s = 0; par ^= 1u; }
 #endif
