@@ -53,7 +53,7 @@ struct Workspace {
   uint32_t* sel_words;  // [kMaxEarlyBlocks][8] the eligible masks as tagged 16-bit pieces (early start of the FFN kernel)
   unsigned long long* root_words;   // [kMaxEarlyBlocks][kMaxExperts] the roots' logits under the call's 32-bit tag (router kernel, see RootArgs)
   unsigned char* xq;    // MXFP4 layers: the hidden states' pieces and scales (mx_act.cuh)
-  int32_t* xq_count;    // CTAs that have stored their part of them, over all calls (never cleared)
+  int32_t* xq_count;    // [2] CTAs that have stored their part of them; calls take the two words in turn
   uint32_t* anc_words;  // [kMaxEarlyBlocks][8] the anchor experts (each root's natural top-k) as tagged 16-bit pieces, published by the router kernel's root CTAs
 };
 
@@ -97,7 +97,8 @@ struct RootArgs {
 // by launch_split_x); each of them adds one to *count when its part is stored.
 struct XqArgs {
   unsigned char* xq;      // null: not wanted
-  int32_t* count;
+  int32_t* count;         // zero when the call starts
+  int32_t* next_count;    // the next call's: cleared here (whoever used it last has completed)
   int n_pad;
   int rows;               // router kernel: rows of CTAs that do it
 };
@@ -199,7 +200,7 @@ struct FfnLaunch {
   const void* mx_gate_up = nullptr;   // MXFP4 layers (launch_ffn_mxfp4): the tiled code + scale tensors
   const void* mx_down = nullptr;
   const void* xq = nullptr;             // MXFP4 layers: the hidden states' pieces (XqArgs), complete once
-  const int32_t* xq_count = nullptr;    // *xq_count has reached xq_target
+  const int32_t* xq_count = nullptr;    // *xq_count has reached xq_target (XqArgs::count)
   int32_t xq_target = 0;
   unsigned long long* trace; // optional [grid][32] device time stamps (acm_stage_timing) or null
 };

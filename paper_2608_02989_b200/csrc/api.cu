@@ -137,7 +137,8 @@ struct acm_ctx {
   std::vector<Layer> layers;
   EncodeTiledFn encode = nullptr;
   int32_t epoch = 0;
-  int32_t xq_target = 0;                 // what ws.xq_count reads once the latest call's hidden-state pieces are stored
+  int32_t xq_target = 0;                 // MXFP4: what ws.xq_count[xq_word] reads once the latest call's hidden-state pieces are stored
+  int xq_word = 0;                       // which of the two count words that call took
   size_t frag_bytes = 0, flag_bytes = 0;   // fragment buffers and arrival counters (zero between launches)
   CUtensorMap h_map[2];
   CUtensorMap h_store_map[2];            // same buffers, one 64-feature tile per TMA store
@@ -395,7 +396,7 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
   if (pdl_ok && c->sm_count > 2 * routing_ctas) p.grid = c->sm_count - routing_ctas;
   c->last_ffn_grid = p.grid;
   if (L.mx) {
-    p.xq = c->ws.xq; p.xq_count = c->ws.xq_count; p.xq_target = c->xq_target;
+    p.xq = c->ws.xq; p.xq_count = c->ws.xq_count + c->xq_word; p.xq_target = c->xq_target;
     p.mx_gate_up = L.has_pool ? L.pool_gate_up : L.mx_gate_up;      // a pool: slot s of the pool tensors
     p.mx_down = L.has_pool ? L.pool_down : L.mx_down;
     ACM_CUDA(launch_ffn_mxfp4(p, maps, x_map, c->h_map[li], c->h_store_map[li], s));
@@ -411,13 +412,15 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
 XqArgs xq_args(acm_ctx* c, int T) {
   XqArgs xa;
   xa.xq = c->ws.xq;
-  xa.count = c->ws.xq_count;
+  xa.count = c->ws.xq_count + (c->xq_word ^ 1);
+  xa.next_count = c->ws.xq_count + c->xq_word;
   xa.n_pad = (T + 15) / 16 * 16;
   xa.rows = split_x_rows(T, c->desc.hidden, c->desc.n_experts);
   return xa;
 }
-void xq_expect(acm_ctx* c, int n_ctas) {
-  c->xq_target = static_cast<int32_t>(static_cast<uint32_t>(c->xq_target) + static_cast<uint32_t>(n_ctas));
+void xq_expect(acm_ctx* c, int n_ctas) {      // (behind the launch)
+  c->xq_target = n_ctas;
+  c->xq_word ^= 1;
 }
 
 // The sequence number of a fused call: its low 16 bits tag the words its kernels publish for one another (0 is

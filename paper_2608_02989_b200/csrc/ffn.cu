@@ -70,6 +70,9 @@ constexpr int kHStageBytes = kMaxNodes * 64 * 2 + (ACM_FFN_MX ? kMxActScaleBytes
 //   (64 clocks at 128 columns, 44 at 32; K = 32 each, so four a stage where bf16 took eight of 75).  What the two-piece
 //   product loses against 64 bits: 6.4e-8 (2-norm) over K = 4096, a serial fp32 sum of the unsplit one: 1.2e-7.
 //   The features are stored in the order the moves leave the weights in (mx_act.cuh).
+// What bounds it: 0.39 us a stage of 64 node columns, 0.30 of them the unpacking groups' chain (waits, shared-memory loads,
+// moves, tensor-memory stores), where HBM would deliver one every 0.20 us.  A layer of 2048 x 768, 64 nodes, 22 experts:
+// 40.3 us; 48.7 with the weights expanded to bf16 by four warps (0.56 us a stage) for eight kind::f16 MMAs.
 constexpr int kThreads = ACM_FFN_MX ? 512 : 256;         // producer, MMA, 4 epilogue warps, helper, publisher (+ 2 x 4 unpacking warps)
 [[maybe_unused]] constexpr int kMxCodeBytes = kTileM * 64;                // 128 rows x 128 four-bit codes
 [[maybe_unused]] constexpr int kMxStageBytes = kMxCodeBytes + kTileM * 4; // + one scale byte per row and 32 K
@@ -263,22 +266,6 @@ __device__ bool flag_wait_ge(const int32_t* p, int target, GiveUp* g, int site) 
     }
   }
 }
-#if ACM_FFN_MX
-// Bounded wait until a running count (it never goes back; it may wrap) has reached `target`.
-__device__ bool count_wait(const int32_t* p, int32_t target, GiveUp* g, int site) {
-  auto reached = [&]() { return static_cast<int32_t>(static_cast<uint32_t>(ld_acquire(p)) - static_cast<uint32_t>(target)) >= 0; };
-  if (reached()) return true;
-  const unsigned long long t0 = global_timer();
-  for (;;) {
-    if (reached()) return true;
-    if (g->flag) return false;
-    if (limit_passed(t0, g->limit_ns)) {
-      give_up(g, site);
-      return false;
-    }
-  }
-}
-#endif
 // Bounded poll of one self-validating word (16 payload bits under a 16-bit tag) written by an earlier kernel
 // of the same stream: returns the payload, or sets `seen` to false when the limit ran out.
 __device__ __forceinline__ uint32_t poll_tagged_word(const uint32_t* word, uint32_t tag, unsigned long long limit_ns, bool& seen) {
@@ -478,8 +465,8 @@ struct FfnArgs {
   const unsigned char* xq_scale;     // [H/64][512] (mx_scale_at)
   unsigned char* hq;                 // activations alike: [slot][I/64][2 n_pad][64]
   unsigned char* hq_scale;           // [slot][I/64][512]
-  const int32_t* xq_count;           // CTAs that have stored their part of the pieces, over all calls of the context
-  int32_t xq_target;                 // ... and what it reads once this call's are complete
+  const int32_t* xq_count;           // CTAs that have stored their part of the pieces
+  int32_t xq_target;                 // ... and how many there are
   int n_raw, n_act;                  // depths of the rings of packed records and activation stages
 #endif
 };
@@ -997,7 +984,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       if (sg.phase == 1) {
         if (lane == 0) {
           if (!x_seen) {
-            ok = count_wait(p.xq_count, p.xq_target, quit, kSiteXPieces);
+            ok = flag_wait_ge(p.xq_count, p.xq_target, quit, kSiteXPieces);
             fence_proxy_async();
             x_seen = true;
           }
@@ -1586,6 +1573,10 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 // 24.9 -> 23.5 us (by then as long as its launches take on the host).
 constexpr int kF32Rows = 4;      // weight rows (of gate and of up; of down) a warp works on at a time
 
+// (four products by themselves before they join the running sum: a quarter of its roundings)
+__device__ __forceinline__ float dot4(const float4& a, const float4& b) {
+  return fmaf(a.x, b.x, a.y * b.y) + fmaf(a.z, b.z, a.w * b.w);
+}
 // Four sums, one per row, over the warp's lanes: lane r < 4 returns that of row r (exchanges of two rows' halves instead of
 // a full reduction per row).
 __device__ __forceinline__ float reduce_rows(const float (&a)[kF32Rows], int lane) {
@@ -1627,8 +1618,8 @@ k_ffn_f32_gate_up(const float* x, const float* __restrict__ gate_up,
 #pragma unroll
         for (int r = 0; r < kF32Rows; ++r) {
           const float4 gv = *reinterpret_cast<const float4*>(g_row[r] + hh), uv = *reinterpret_cast<const float4*>(g_row[r] + to_up + hh);
-          g[r] = fmaf(gv.x, xv.x, fmaf(gv.y, xv.y, fmaf(gv.z, xv.z, fmaf(gv.w, xv.w, g[r]))));
-          u[r] = fmaf(uv.x, xv.x, fmaf(uv.y, xv.y, fmaf(uv.z, xv.z, fmaf(uv.w, xv.w, u[r]))));
+          g[r] += dot4(gv, xv);
+          u[r] += dot4(uv, xv);
         }
       }
     } else {
@@ -1682,7 +1673,7 @@ k_ffn_f32_down(const float* __restrict__ down, const float* __restrict__ shared_
 #pragma unroll
         for (int r = 0; r < kF32Rows; ++r) {
           const float4 dv = *reinterpret_cast<const float4*>(base + static_cast<size_t>(min(h0 + r, H - 1)) * I + i);
-          acc[r] = fmaf(dv.x, hv.x, fmaf(dv.y, hv.y, fmaf(dv.z, hv.z, fmaf(dv.w, hv.w, acc[r]))));
+          acc[r] += dot4(dv, hv);
         }
       }
     } else {

@@ -225,6 +225,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
 // while a dependent launch is already resident: never through the read-only path.)
 __device__ __forceinline__ void split_x(const XqArgs& xa, const __nv_bfloat16* x, int T, int H, int i, int n) {
   const int per_node = H / 32;
+  if (i == 0) *xa.next_count = 0;
   for (; i < T * per_node; i += n) {
     const int t = i / per_node, block = i - t * per_node, half = block >> 1, tb = xa.n_pad + t;
     uint32_t w[16];
