@@ -1043,3 +1043,54 @@ def test_mxfp4_activation_pieces(T, H, I):
         assert torch.isfinite(bad[rest]).all()
         assert float((bad[rest] - alone[rest]).abs().max()) <= 1e-3 * float(alone[rest].double().pow(2).mean().sqrt())
     ctx.close()
+
+
+@pytest.mark.parametrize("T,H,I,E,k,ns", [(1, 32, 4, 5, 1, 0), (9, 96, 66, 13, 3, 1), (40, 160, 132, 40, 8, 2), (64, 256, 3, 16, 2, 0)])
+def test_f32_ffn_rows_and_loads(T, H, I, E, k, ns):
+    """The fp32 FFN kernels take four weight rows a warp (remainders of 1 to 3 rows here) and 16-byte loads where shapes and
+    pointers allow: inter 66 and 3 do not, nor do weights 4 bytes off in the allocation-free call."""
+    g = torch.Generator(device=DEV).manual_seed(T)
+    rnd = lambda *s: torch.randn(*s, generator=g, device=DEV)
+    x, gu, dn = rnd(T, H), 0.1 * rnd(E, 2 * I, H), 0.1 * rnd(E, H, I)
+    sgu, sdn = (0.1 * rnd(ns, 2 * I, H), 0.1 * rnd(ns, H, I)) if ns else (None, None)
+    idx = torch.stack([torch.randperm(E, generator=g, device=DEV)[:k] for _ in range(T)]).to(torch.int32)
+    idx[0, k - 1] = -1
+    w = torch.rand(T, k, generator=g, device=DEV)
+    ctx = acm.Context(H, E, k, I, ns, dtype=acm.F32)
+    ctx.set_layer_weights(0, rnd(E, H), None, gu, dn, sgu, sdn)
+    out = ctx.expert_ffn(0, x, idx, w)
+    assert ctx.device_status() == acm.OK
+    ref = oracle.expert_ffn(x, idx.cpu().numpy(), w.cpu().numpy(), gu, dn, sgu, sdn)
+    rms = float(np.sqrt(np.mean(ref ** 2)))
+    # fp32 products and sums of H and I terms in any order: a few hundred ulp of the largest term at the very most
+    assert float(np.abs(out.double().cpu().numpy() - ref).max()) <= 1e-4 * rms
+    if ns == 0:
+        off = lambda t: torch.cat([t.new_zeros(1), t.flatten()])[1:].view(t.shape)
+        got = acm.expert_ffn_f32_noalloc(off(x), idx, w, off(gu), off(dn), torch.empty(T, H, device=DEV))
+        torch.cuda.synchronize()
+        assert float(np.abs(got.double().cpu().numpy() - ref).max()) <= 1e-4 * rms
+    ctx.close()
+
+
+@pytest.mark.parametrize("T,E,k", [(1, 1, 1), (17, 33, 5), (64, 128, 8)])
+def test_given_routes_reach_the_weight_table(T, E, k):
+    """acm_expert_ffn with routes of the caller's: empty slots, ids outside the layer, nodes without any route, and an output
+    buffer that held something before."""
+    cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, n_nodes=T, n_experts=E, top_k=k, hidden=256, inter=128, zipf_bias=False)
+    ctx = _ctx(cfg)
+    w_, x = wl.layer_weights(cfg, 0, DEV), wl.hidden_states(cfg, 0, DEV)
+    ctx.set_layer_weights(0, w_["w_router"], None, w_["gate_up"], w_["down"])
+    g = torch.Generator().manual_seed(E)
+    idx = torch.stack([torch.randperm(E, generator=g)[:k] for _ in range(T)]).to(torch.int32)
+    w = torch.rand(T, k, generator=g)
+    given = idx.clone()
+    if T > 1:
+        idx[1, :] = -1
+        given[1, :] = torch.tensor([-1, E, 1 << 20, -7, 128][:k] + [-1] * (k - 5), dtype=torch.int32)[:k]
+        idx[T - 1, 0] = given[T - 1, 0] = -1
+    for _ in range(2):
+        out = torch.full((T, 256), 3.0, device=DEV)
+        ctx.expert_ffn(0, x, given.to(DEV), w.to(DEV), out=out)
+        assert ctx.device_status() == acm.OK
+        _ffn_check(out, oracle.expert_ffn(x, idx.numpy(), w.numpy(), w_["gate_up"], w_["down"]), "given routes")
+    ctx.close()
