@@ -1381,6 +1381,8 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
           for (int h = 0; h < n_halves && ok; ++h) {
             const int cb = h * kMaxNodes;                              // first node column of this half
             const int np = min(p.n_pad - cb, kMaxNodes);               // its columns (a multiple of 16)
+            // (all have read the half before out of the exchange buffer before this one is written to it)
+            if (kN > kMaxNodes && h > 0 && !(ok = epi_vote_all(true))) break;
 #if ACM_FFN_MX
             // The tile goes through the exchange buffer, [node][64 gate rows, 64 up rows] with the rows rotated by the
             // node, and a thread then takes up the 32 features of one node, i.e. one scale block, so that the block's
