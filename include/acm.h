@@ -144,9 +144,13 @@ acm_status acm_set_layer_weights(acm_ctx* ctx, int layer, const void* w_router,
 
 /* The same for a layer whose routed experts are stored in MXFP4 (microscaling FP4 -- the storage the
  * paper's offload measurements name for GPT-OSS, Section 4.4): 4-bit E2M1 codes, one E8M0 scale byte
- * (2^(s-127)) per 32 consecutive K elements.  The FFN kernel expands the codes to bf16 on the way to the
- * tensor cores -- every MXFP4 value is a bf16, so the layer computes exactly what a bf16 layer with the
- * dequantised weights computes -- and streams a quarter of the bytes.  The tensors are in the library's
+ * (2^(s-127)) per 32 consecutive K elements.  The layer computes what a bf16 layer with the dequantised
+ * weights computes and streams a quarter of the bytes.  The products are those of the tensor cores' block-scaled
+ * instruction: the codes and scales enter as they are, and every bf16 operand (the hidden states, and the
+ * activations between the two products) as three 8-bit e5m2 pieces under a power-of-two scale per node and 32
+ * consecutive features.  Their sum is the bf16 value exactly if no other of those 32 is more than 2^31 times
+ * larger, and is off by at most 2^-39 of the largest if one is (acm_mxfp4_activation_pieces).  Sums are in fp32.  A hidden
+ * state that is not finite makes its node's output row NaN, and no other row.  The tensors are in the library's
  * tiled layout (one contiguous 8704-byte record per weight tile and pipeline stage):
  *   gate_up_tiles [E][I/64][H/128][8704]: tile t = gate rows 64t..64t+63 then up rows I+64t..I+64t+63,
  *   down_tiles    [E][H/128][I/128][8704]: tile t = rows 128t..128t+127,
@@ -373,6 +377,12 @@ acm_status acm_ffn_plan(int n_experts_streamed, int n_anchor_first, int hidden, 
 /* The same for an MXFP4 layer (inter a multiple of 128): its kernel deals every tile whole. */
 acm_status acm_ffn_plan_mxfp4(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,
                               int32_t* pieces /*host*/, int capacity, int32_t* n_pieces /*host*/, int32_t* n_segments /*host*/);
+
+/* How an MXFP4 layer's kernels take 32 consecutive features of one node, worked out on the host (no GPU is touched):
+ * values [32] are bf16 words; pieces [3][32] receives e5m2 bytes, scales [3] the E8M0 byte of each piece, so that
+ * value i = sum over p of pieces[p][i] * 2^(scales[p] - 127), within the bound given at acm_set_layer_weights_mxfp4.
+ * scales[0] is 255 (NaN) if a value is not finite.  For inspection and for tests of that bound. */
+acm_status acm_mxfp4_activation_pieces(const uint16_t* values /*host*/, uint8_t* pieces /*host*/, uint8_t* scales /*host*/);
 
 /* How far the kernels of a fused call (acm_moe_verify, acm_moe_verify_batch, acm_moe_verify_host) overlap.
  * The stages of Section 3.1-3.4 form a chain, and the expert FFN needs only part of its result to start:

@@ -28,7 +28,7 @@ EXPORTS = [
     "acm_set_slot_pool", "acm_pool_stats", "acm_pool_plan",
     "acm_h2d_bytes", "acm_ffn_timing", "acm_ffn_time_ms", "acm_stage_timing", "acm_stage_times", "acm_launch_count", "acm_device_status", "acm_status_string",
     "acm_set_overlap", "acm_set_wait_limit", "acm_wait_report", "acm_inject_unpublished_wait",
-    "acm_offload_timing", "acm_offload_times", "acm_ffn_plan", "acm_ffn_plan_mxfp4",
+    "acm_offload_timing", "acm_offload_times", "acm_ffn_plan", "acm_ffn_plan_mxfp4", "acm_mxfp4_activation_pieces",
     "acm_expert_ffn_f32_noalloc",
 ]
 NOALLOC_MAX_FLOATS = 1 << 20
@@ -113,6 +113,7 @@ def load_library():
     lib.acm_device_status.argtypes = [c_void_p, c_void_p]
     lib.acm_set_overlap.argtypes = [c_void_p, c_int]
     lib.acm_ffn_plan_mxfp4.argtypes = [c_int] * 5 + [c_void_p, c_int, POINTER(c_int32), POINTER(c_int32)]
+    lib.acm_mxfp4_activation_pieces.argtypes = [c_void_p, c_void_p, c_void_p]
     lib.acm_ffn_plan.argtypes = [c_int] * 5 + [c_void_p, c_int, POINTER(c_int32), POINTER(c_int32)]
     lib.acm_offload_timing.argtypes = [c_void_p, c_int, c_int]
     lib.acm_offload_times.argtypes = [c_void_p, POINTER(ctypes.c_double), POINTER(c_int32)]
@@ -170,6 +171,16 @@ def ffn_plan(n_experts_streamed, hidden, inter, grid, n_anchor_first=0, mxfp4=Fa
             continue
         _check(rc, "acm_ffn_plan")
         return buf[: n.value], nseg.value
+
+
+def mxfp4_activation_pieces(values):
+    """acm_mxfp4_activation_pieces: 32 bf16 values (host) -> (pieces [3, 32] uint8 e5m2, scales [3] uint8 E8M0)."""
+    v = values.detach().cpu().to(torch.bfloat16).contiguous()
+    if v.numel() != 32:
+        raise ValueError("a block has 32 values")
+    pieces, scales = torch.empty(3, 32, dtype=torch.uint8), torch.empty(3, dtype=torch.uint8)
+    _check(load_library().acm_mxfp4_activation_pieces(_p(v), _p(pieces), _p(scales)), "acm_mxfp4_activation_pieces")
+    return pieces, scales
 
 
 def pool_plan(n_experts, slot_expert, last_use, tick, activated):

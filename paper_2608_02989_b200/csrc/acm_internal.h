@@ -93,7 +93,7 @@ struct RootArgs {
   unsigned long long wait_limit_ns;
 };
 
-// MXFP4 layers: the hidden states as e4m3 pieces for the FFN kernel (mx_act.cuh), stored by CTAs of the router kernel (or
+// MXFP4 layers: the hidden states as e5m2 pieces for the FFN kernel (mx_act.cuh), stored by CTAs of the router kernel (or
 // by launch_split_x); each of them adds one to *count when its part is stored.
 struct XqArgs {
   unsigned char* xq;      // null: not wanted

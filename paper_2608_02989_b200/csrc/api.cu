@@ -1493,6 +1493,23 @@ acm_status acm_ffn_plan_mxfp4(int n_experts_streamed, int n_anchor_first, int hi
   return list_plan<true>(n_experts_streamed, n_anchor_first, hidden, inter, grid, pieces, capacity, n_pieces, n_segments);
 }
 
+acm_status acm_mxfp4_activation_pieces(const uint16_t* values, uint8_t* pieces, uint8_t* scales) {
+  if (!values || !pieces || !scales) return ACM_ERR_INVALID;
+  uint32_t w[16];
+  for (int i = 0; i < 16; ++i) w[i] = values[2 * i] | (static_cast<uint32_t>(values[2 * i + 1]) << 16);
+  const int scale = mx_block_scale(w);
+  for (int p = 0; p < kMxPieces; ++p) scales[p] = static_cast<uint8_t>(scale - p * kMxPieceShift);
+  constexpr int order[8] = {0, 4, 1, 5, 2, 6, 3, 7};      // of every eight features (mx_act.cuh)
+  for (int half = 0; half < 2; ++half) {
+    uint32_t k[kMxPieces][4];
+    mx_pieces(w, half, scale, k);
+    for (int p = 0; p < kMxPieces; ++p)
+      for (int i = 0; i < 16; ++i)
+        pieces[32 * p + 16 * half + 8 * (i / 8) + order[i % 8]] = static_cast<uint8_t>(k[p][i / 4] >> (8 * (i % 4)));
+  }
+  return ACM_OK;
+}
+
 acm_status acm_set_overlap(acm_ctx* c, int level) {
   if (!c || level < ACM_OVERLAP_NONE || level > ACM_OVERLAP_ANCHORS) return ACM_ERR_INVALID;
   c->overlap = level;

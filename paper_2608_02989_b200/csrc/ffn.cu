@@ -41,7 +41,7 @@ namespace {
 #define ACM_FFN_MX 0
 #endif
 constexpr int kMaxStages = 3;                            // pipeline stages of the weight ring (see Geo)
-constexpr int kAcc = ACM_FFN_MX ? 3 : 4;                 // TMEM accumulators in flight
+constexpr int kAcc = 4;                                  // TMEM accumulators in flight (power of two)
 constexpr int kBK = 64;                                  // K elements of one 128-byte swizzle atom
 constexpr int kAtoms = 2;                                // atoms per pipeline stage: a stage covers 128 K
 constexpr int kTileM = 128;
@@ -50,10 +50,11 @@ constexpr int kABytes = kAtoms * kAtomABytes;            // 32 KB weight tile, o
 // The epilogue handles node columns kMaxNodes = 64 at a time: one fragment, one activation tile.  A wide tile (a
 // batch of blocks with more than 64 nodes in all, up to kWideNodes = 128 accumulator columns) goes in two halves.
 constexpr int kOutStageBytes = kTileM * kMaxNodes * 4;   // 32 KB: outgoing fragment (also the gate/up exchange buffer)
-// One finished activation tile (64 features x 64 nodes): 8 KB of bf16, or -- the same 8 KB -- two e4m3 pieces per
-// element plus their 512 bytes of scales (MXFP4, see below).
+// One finished activation tile (64 features x 64 nodes): 8 KB of bf16, or three e5m2 pieces per element and 256 bytes of
+// scales (MXFP4, see below).
 constexpr int kHStages = ACM_FFN_MX ? 1 : 2;             // of them in shared memory
-constexpr int kHStageBytes = kMaxNodes * 64 * 2 + (ACM_FFN_MX ? kMxActScaleBytes : 0);
+constexpr int kHPieceBytes = kMaxNodes * 64 * (ACM_FFN_MX ? kMxPieces : 2);
+constexpr int kHStageBytes = kHPieceBytes + (ACM_FFN_MX ? kMxActScaleBytes : 0);
 // ACM_FFN_MX = 1 (set by ffn_mx.cu, which includes this file) builds the same kernel for MXFP4 expert weights on the
 // block-scaled tensor-core instruction (tcgen05.mma kind::mxf8f6f4: 8-bit operands, an E8M0 scale per row and 32 K).
 //   Weights.  A pipeline stage of a tile is one contiguous 8704-byte record (128 rows x 64 bytes of E2M1 codes, 128 x 4
@@ -62,29 +63,25 @@ constexpr int kHStageBytes = kMaxNodes * 64 * 2 + (ACM_FFN_MX ? kMxActScaleBytes
 //   (an e4m3 would take seven), and store them in tensor memory, from where the MMAs take their A operand.  (4-bit
 //   operands as they are would do without the moves, but have to lie in shared memory, 16 bytes for 16 codes: written
 //   there and read again by the MMAs they made shared-memory bandwidth the bound, 670 of 720 clocks a stage.)
-//   Activations.  A bf16 has 8 significand bits, an e4m3 four: x = a + b, a = e4m3(x / s), b = e4m3 of the rest, with
-//   s a power of two per node and 32 K that puts the largest |x| into [128, 256) and b scaled by 2^-4 s.  The split is
-//   exact for every |x| >= 2^-14 of that maximum, and off by at most 2^-22 of the maximum below (an fp32 accumulator
-//   of such products rounds at 2^-24).  The pieces are node columns of their own -- a in columns [0, n_pad), b in
-//   [n_pad, 2 n_pad) of ONE accumulator, added when it is read -- because an instruction costs little more for them
-//   (64 clocks at 128 columns, 44 at 32; K = 32 each, so four a stage where bf16 took eight of 75).  What the two-piece
-//   product loses against 64 bits: 6.4e-8 (2-norm) over K = 4096, a serial fp32 sum of the unsplit one: 1.2e-7.
+//   Activations.  A bf16 has 8 significand bits, an e5m2 three: x is the sum of three of them under one scale per node
+//   and 32 K and its 2^-4 and 2^-8 (mx_act.cuh), exact unless another value of those 32 is more than 2^31 times larger and
+//   then off by at most 2^-39 of that one.  Each piece has MMAs of its own into the same accumulator.  (Two e4m3 pieces as node columns of their
+//   own, one MMA for both, reach down to 2^-13 only.  Weights that are zero wherever a feature is 2^14 times the others then
+//   leave a result with three times the error, 2^20 times the others: 31 % off.)
 //   The features are stored in the order the moves leave the weights in (mx_act.cuh).
-// What bounds it: 0.39 us a stage of 64 node columns, 0.30 of them the unpacking groups' chain (waits, shared-memory loads,
-// moves, tensor-memory stores), where HBM would deliver one every 0.20 us.  A layer of 2048 x 768, 64 nodes, 22 experts:
-// 40.3 us; 48.7 with the weights expanded to bf16 by four warps (0.56 us a stage) for eight kind::f16 MMAs.
 constexpr int kThreads = ACM_FFN_MX ? 512 : 256;         // producer, MMA, 4 epilogue warps, helper, publisher (+ 2 x 4 unpacking warps)
 [[maybe_unused]] constexpr int kMxCodeBytes = kTileM * 64;                // 128 rows x 128 four-bit codes
 [[maybe_unused]] constexpr int kMxStageBytes = kMxCodeBytes + kTileM * 4; // + one scale byte per row and 32 K
 [[maybe_unused]] constexpr int kMxACols = 32;                             // an unpacked stage in tensor memory: 4 weights a column
-[[maybe_unused]] constexpr int kMxScaleCols = 8;                          // its scales: 4 columns the weights', 4 the activations'
-[[maybe_unused]] constexpr int kMxA = 3;                                  // such stages in flight
-static_assert(!ACM_FFN_MX || kAcc * 2 * kMaxNodes + kMxA * (kMxACols + kMxScaleCols) <= 512, "tensor memory: accumulators + unpacked stages");
-// Shared-memory rings of the MXFP4 kernel: activation pieces and packed records.  Both are 1.5 us from request to arrival
-// under load, from L2 and from HBM; they share the space, an activation stage being 256 n_pad bytes: 7 of either beside
-// 64 node columns, 10 and 12 beside 16 (mx_rings).
-[[maybe_unused]] constexpr int kMaxRaw = 12, kMaxAct = 10;
-[[maybe_unused]] constexpr int kMxRingBytes = 181 * 1024;
+[[maybe_unused]] constexpr int kMxScaleCols = 16;                         // its scales: 4 columns the weights', 4 each piece's (2 used)
+// Stages in flight behind the packed records: tensor-memory slots and activation stages, one ring.
+constexpr int kMxA = 5;
+static_assert(!ACM_FFN_MX || kAcc * kMaxNodes + kMxA * (kMxACols + kMxScaleCols) <= 512, "tensor memory: accumulators + unpacked stages");
+// Shared memory of the MXFP4 kernel's rings: kMxA activation stages of 384 n_pad bytes and their scales, and packed records in
+// what they leave (6 beside 64 node columns, 12 beside up to 32: mx_raw_stages).  Either is 1.5 us from request to arrival
+// under load, from L2 and from HBM.
+[[maybe_unused]] constexpr int kMaxRaw = 12;
+[[maybe_unused]] constexpr int kMxRingBytes = 178 * 1024;
 constexpr int kFragBytes = ACM_FFN_MX ? 0 : kTileM * kMaxNodes * 4;   // contributor fragments pre-summed in shared memory (MXFP4: no cut tiles)
 constexpr int kFragFloats = kTileM * kMaxNodes;
 
@@ -124,7 +121,7 @@ enum WaitSite : int {
   kSitePackedStage = 18,    // MXFP4 unpacking warps: the packed weight stage
   kSitePackedFree = 19,     // MXFP4 weight producer: a record slot the unpacking warps have not read
   kSiteActStage = 20,       // MXFP4 unpacking warps: the stage's activations
-  kSiteActSlot = 21,        // MXFP4 activation producer: a stage the MMAs have not released
+  kSiteActSlot = 21,        // MXFP4 activation producer: a ring stage the MMAs have not released
   kSiteXPieces = 22         // MXFP4 activation producer: the hidden states' pieces
 };
 struct GiveUp {
@@ -135,10 +132,12 @@ struct GiveUp {
   int32_t tag;                   // launch number << 8
 };
 
+// stages of the ring that the MMAs take their operands from
+constexpr int kMaxRing = ACM_FFN_MX ? kMxA : kMaxStages;
 template <int kN>
 struct __align__(8) BarriersT {
-  unsigned long long full[kMaxStages];
-  unsigned long long empty[kMaxStages];
+  unsigned long long full[kMaxRing];
+  unsigned long long empty[kMaxRing];
   unsigned long long tfull[kAcc];
   unsigned long long tempty[kAcc];
   unsigned long long drained;
@@ -149,7 +148,7 @@ struct __align__(8) BarriersT {
   unsigned long long hst_full[2], hst_free[2];   // epilogue <-> publisher: activation tile staged / stored
 #if ACM_FFN_MX
   unsigned long long raw[kMaxRaw], raw_empty[kMaxRaw];   // packed records: landed (-> unpacking warps) / read (-> producer)
-  unsigned long long act[kMaxAct], act_empty[kMaxAct];   // activation stages: landed / multiplied (-> activation producer)
+  unsigned long long act[kMaxRing];      // activation stages landed (-> unpacking warps)
 #endif
   volatile uint32_t armed;           // stages whose barrier the weight producer has armed so far
   volatile int32_t n_routed_slots;   // routed experts in this launch's work list (known with the complete list)
@@ -171,12 +170,13 @@ struct Geo {
   static constexpr int kStages = kN > kMaxNodes ? 2 : 3;
   static constexpr int kBBytes = kAtoms * kN * kBK * 2;          // activation chunk of a stage, one TMA copy
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kTmemCols = ACM_FFN_MX ? 512 : kAcc * kN;    // MXFP4: two-piece accumulators, then the scales
+  static constexpr int kTmemCols = ACM_FFN_MX ? 512 : kAcc * kN;    // MXFP4: accumulators, unpacked weights, scales
   static constexpr int kRingBytes = ACM_FFN_MX ? kMxRingBytes : kStages * kStageBytes;
   static constexpr size_t kSmemBytes =
       1024 + static_cast<size_t>(kRingBytes) + kOutStageBytes + kFragBytes + kHStages * kHStageBytes + sizeof(BarriersT<kN>);
   static_assert(kSmemBytes <= 232448, "shared memory: ring + staging buffers + control block exceed 227 KB");
-  static_assert(kStages <= kMaxStages, "barrier arrays");
+  static constexpr int kRing = ACM_FFN_MX ? kMxA : kStages;
+  static_assert(kRing <= kMaxRing, "barrier arrays");
 };
 
 // ---------------------------------------------------------------------------------- PTX helpers
@@ -391,7 +391,7 @@ __device__ __forceinline__ uint64_t umma_smem_desc(uint32_t smem_addr) {
   return d;
 }
 #if ACM_FFN_MX
-// Block-scaled MMA over 32 K: unpacked weights (128 rows, e2m3, in tensor memory: row = lane, four K a column) x e4m3
+// Block-scaled MMA over 32 K: unpacked weights (128 rows, e2m3, in tensor memory: row = lane, four K a column) x e5m2
 // activation pieces (K-major in shared memory), with their E8M0 scales in tensor memory (row or column j: lane j % 32 of
 // every quarter, column j / 32).
 __device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint32_t tmem_a, uint64_t desc_b, uint32_t idesc, uint32_t accumulate,
@@ -401,12 +401,12 @@ __device__ __forceinline__ void umma_mx(uint32_t tmem_d, uint32_t tmem_a, uint64
       "tcgen05.mma.cta_group::1.kind::mxf8f6f4.block_scale.scale_vec::1X [%0], [%1], %2, %3, [%5], [%6], p;\n\t}\n"
       ::"r"(tmem_d), "r"(tmem_a), "l"(desc_b), "r"(idesc), "r"(accumulate), "r"(tmem_sfa), "r"(tmem_sfb) : "memory");
 }
-// Its instruction descriptor: A = E2M3, B = E4M3, E8M0 scales, fp32 accumulator, M = 128, N = n (bits 29, 30 and 4, 5: which
+// Its instruction descriptor: A = E2M3, B = E5M2, E8M0 scales, fp32 accumulator, M = 128, N = n (bits 29, 30 and 4, 5: which
 // byte of the scales' words).
 __device__ __forceinline__ uint32_t umma_mx_idesc(int n) {
-  return (3u << 7) | (static_cast<uint32_t>(n >> 3) << 17) | (1u << 23) | (static_cast<uint32_t>(kTileM >> 7) << 27);
+  return (3u << 7) | (1u << 10) | (static_cast<uint32_t>(n >> 3) << 17) | (1u << 23) | (static_cast<uint32_t>(kTileM >> 7) << 27);
 }
-// Descriptor of an activation half-stage: rows of 64 bytes (64 K e4m3), 64-byte swizzle, groups of 8 rows 512 bytes apart.
+// Descriptor of an activation half-stage: rows of 64 bytes (64 K e5m2), 64-byte swizzle, groups of 8 rows 512 bytes apart.
 __device__ __forceinline__ uint64_t umma_smem_desc_64(uint32_t smem_addr) {
   return static_cast<uint64_t>((smem_addr & 0x3ffffu) >> 4) | (static_cast<uint64_t>(1) << 16) |
          (static_cast<uint64_t>(512 >> 4) << 32) | (static_cast<uint64_t>(1) << 46) | (static_cast<uint64_t>(4) << 61);
@@ -414,6 +414,9 @@ __device__ __forceinline__ uint64_t umma_smem_desc_64(uint32_t smem_addr) {
 // 4 consecutive columns of this thread's lane
 __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
+}
+__device__ __forceinline__ void tmem_st2(uint32_t taddr, uint32_t a, uint32_t b) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1,%2};" ::"r"(taddr), "r"(a), "r"(b) : "memory");
 }
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&v)[32]) {
   asm volatile(
@@ -461,13 +464,13 @@ struct FfnArgs {
 #if ACM_FFN_MX
   const unsigned char* mx_gate_up;   // [E][I/64][H/128][8704]
   const unsigned char* mx_down;      // [E][H/128][I/128][8704]
-  const unsigned char* xq;           // hidden states in pieces: [H/64][2 n_pad][64], 64-byte swizzled
-  const unsigned char* xq_scale;     // [H/64][512] (mx_scale_at)
-  unsigned char* hq;                 // activations alike: [slot][I/64][2 n_pad][64]
-  unsigned char* hq_scale;           // [slot][I/64][512]
+  const unsigned char* xq;           // hidden states in pieces: [H/64][3 n_pad][64], 64-byte swizzled
+  const unsigned char* xq_scale;     // [H/64][256] (mx_scale_at)
+  unsigned char* hq;                 // activations alike: [slot][I/64][3 n_pad][64]
+  unsigned char* hq_scale;           // [slot][I/64][256]
   const int32_t* xq_count;           // CTAs that have stored their part of the pieces
   int32_t xq_target;                 // ... and how many there are
-  int n_raw, n_act;                  // depths of the rings of packed records and activation stages
+  int n_raw;                         // packed records in flight
 #endif
 };
 
@@ -491,7 +494,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUtensorMap x_map,
            const __grid_constant__ CUtensorMap h_map, const __grid_constant__ CUtensorMap hs_map,
            const FfnArgs p) {
-  constexpr int kStages = Geo<kN>::kStages, kAccCols = ACM_FFN_MX ? 2 * kN : kN, kTmemCols = Geo<kN>::kTmemCols;
+  constexpr int kRing = Geo<kN>::kRing, kAccCols = kN, kTmemCols = Geo<kN>::kTmemCols;
 #if !ACM_FFN_MX
   constexpr int kStageBytes = Geo<kN>::kStageBytes;
 #endif
@@ -504,10 +507,10 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   unsigned char* after_ring = smem + static_cast<size_t>(Geo<kN>::kRingBytes);
 #if ACM_FFN_MX
   // the ring area: activation pieces, their scales, packed records
-  const int act_bytes = p.n_pad * 256;
+  const int act_bytes = p.n_pad * (kMxPieces * 128);      // of a stage: two half-stages of 64 K
   unsigned char* act_base = smem;
-  unsigned char* act_scale_base = act_base + p.n_act * act_bytes;
-  unsigned char* raw_base = act_scale_base + p.n_act * 2 * kMxActScaleBytes;
+  unsigned char* act_scale_base = act_base + kMxA * act_bytes;
+  unsigned char* raw_base = act_scale_base + kMxA * 2 * kMxActScaleBytes;
 #endif
   float* ostage = reinterpret_cast<float*>(after_ring);           // outgoing fragment [node][128 rows]
 #if !ACM_FFN_MX
@@ -522,7 +525,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   const int cta = blockIdx.x, G = gridDim.x;
   griddep_launch_dependents();
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kRing; ++s) {
       mbar_init(smem_u32(&bars->full[s]), ACM_FFN_MX ? 4 : 1);   // MXFP4: one arrival per unpacking warp
       mbar_init(smem_u32(&bars->empty[s]), 1);
     }
@@ -531,10 +534,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       mbar_init(smem_u32(&bars->raw[s]), 1);
       mbar_init(smem_u32(&bars->raw_empty[s]), 4);
     }
-    for (int s = 0; s < p.n_act; ++s) {
-      mbar_init(smem_u32(&bars->act[s]), 1);
-      mbar_init(smem_u32(&bars->act_empty[s]), 1);
-    }
+    for (int s = 0; s < kRing; ++s) mbar_init(smem_u32(&bars->act[s]), 1);
 #endif
     for (int b = 0; b < kAcc; ++b) {
       mbar_init(smem_u32(&bars->tfull[b]), 1);
@@ -816,7 +816,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
               tma_load_3d(sa + kABytes, &x_map, full, 0, 0, kk * kAtoms, pol_x);
               if (++kk == kc1) kk = 0;
               ++n_armed;
-              if (++s == kStages) { s = 0; par ^= 1u; }
+              if (++s == kRing) { s = 0; par ^= 1u; }
 #endif
             }
           }
@@ -852,7 +852,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
               mbar_expect_tx(full, kABytes + b_bytes);
               tma_load_4d(sa, dn, full, 0, ht * kTileM, ic * kAtoms, eidx, pol_w);
               bars->armed = ++n_armed;      // the helper warp may now add this stage's activation chunk
-              if (++s == kStages) { s = 0; par ^= 1u; }
+              if (++s == kRing) { s = 0; par ^= 1u; }
               if (++ic == kpe && kc + 1 < k1) {
                 ic = 0;
                 ent = s_entry[++a];
@@ -892,17 +892,15 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     // MXFP4 stage: 370 clocks to issue, 110 this way).
     const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
 #if ACM_FFN_MX
-    const uint32_t idesc = umma_mx_idesc(2 * p.n_pad);
+    const uint32_t idesc = umma_mx_idesc(p.n_pad);
     const uint64_t act_hi = umma_smem_desc_64(0);
-    const uint32_t half_step = static_cast<uint32_t>(act_bytes) >> 5;      // (in 16-byte units) from one half-stage to the other
+    // (in 16-byte units) from one half-stage to the other, from one piece to the next
+    const uint32_t half_step = static_cast<uint32_t>(act_bytes) >> 5, piece_step = static_cast<uint32_t>(p.n_pad) * 4;
     const uint32_t act0 = (smem_u32(act_base) & 0x3ffffu) >> 4;
-    uint32_t act_slot = 0;
-    constexpr uint32_t kRing = kMxA;
 #else
     const uint32_t idesc = umma_idesc(p.n_pad);
     const uint64_t desc_hi = umma_smem_desc(0);
     const uint32_t stage0 = (smem_u32(stage_base) & 0x3ffffu) >> 4;
-    constexpr uint32_t kRing = kStages;
 #endif
     uint32_t s = 0, par = 0, b = 0, bpar = 1;
     bool ok = true;
@@ -922,17 +920,20 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #if ACM_FFN_MX
           const uint32_t ta = tm + kAcc * kAccCols + s * kMxACols;
           const uint32_t sf = tm + kAcc * kAccCols + kMxA * kMxACols + s * kMxScaleCols;
-          const uint64_t db = act_hi | (act0 + act_slot * (static_cast<uint32_t>(act_bytes) >> 4));
+          const uint64_t db = act_hi | (act0 + s * (static_cast<uint32_t>(act_bytes) >> 4));
           if (elect_one()) {
             // 32 K = one scale each (byte kb of the scales' words); two half-stages of 64 K of activations
-            umma_mx(d_tmem, ta, db, idesc, kc > 0 ? 1u : 0u, sf, sf + 4);
-            umma_mx(d_tmem, ta + 8, db + 2, idesc | (1u << 29) | (1u << 4), 1u, sf, sf + 4);
-            umma_mx(d_tmem, ta + 16, db + half_step, idesc | (2u << 29) | (2u << 4), 1u, sf, sf + 4);
-            umma_mx(d_tmem, ta + 24, db + half_step + 2, idesc | (3u << 29) | (3u << 4), 1u, sf, sf + 4);
+#pragma unroll
+            for (int pc = 0; pc < kMxPieces; ++pc) {
+#pragma unroll
+              for (int kb = 0; kb < 4; ++kb)
+                umma_mx(d_tmem, ta + 8 * kb, db + pc * piece_step + (kb >> 1) * half_step + (kb & 1) * 2,
+                        idesc | (static_cast<uint32_t>(kb) << 29) | (static_cast<uint32_t>(kb) << 4), (kc > 0 || pc > 0 || kb > 0) ? 1u : 0u,
+                        sf, sf + 4 + 4 * pc);
+            }
             umma_commit(smem_u32(&bars->empty[s]));
             if (kc + 1 == nk) umma_commit(smem_u32(&bars->tfull[b]));
           }
-          if (++act_slot == static_cast<uint32_t>(p.n_act)) act_slot = 0;
 #else
           // descriptors: only the address field changes from stage to stage and atom to atom
           const uint64_t da0 = desc_hi | (stage0 + s * (kStageBytes >> 4));
@@ -970,12 +971,12 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     const uint64_t pol_x = policy_evict_last();
     uint32_t ai = 0, apar = 0;
     auto fetch = [&](const unsigned char* pieces, const unsigned char* scales) -> bool {
-      if (!mbar_wait(smem_u32(&bars->act_empty[ai]), apar ^ 1u, quit, kSiteActSlot)) return false;
+      if (!mbar_wait(smem_u32(&bars->empty[ai]), apar ^ 1u, quit, kSiteActSlot)) return false;
       const uint32_t full = smem_u32(&bars->act[ai]);
       mbar_expect_tx(full, static_cast<uint32_t>(act_bytes) + 2 * kMxActScaleBytes);
       bulk_load_hint(smem_u32(act_base) + ai * act_bytes, pieces, act_bytes, full, pol_x);
       bulk_load_hint(smem_u32(act_scale_base) + ai * 2 * kMxActScaleBytes, scales, 2 * kMxActScaleBytes, full, pol_x);
-      if (++ai == static_cast<uint32_t>(p.n_act)) { ai = 0; apar ^= 1u; }
+      if (++ai == kRing) { ai = 0; apar ^= 1u; }
       return true;
     };
     for (int si = 0; ok && have_seg(si, true); ++si) {
@@ -1042,7 +1043,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       const int n_exp = sg.a1 - sg.a0;
       if (sg.phase == 1) {
         hidx += bars->plan.range[si].n_stages;
-        hs = hidx % kStages;
+        hs = hidx % kRing;
         if (sg.whole) continue;          // whole tiles: nothing to exchange
         const unsigned ub = cut_begin(sg, cta, p.d_grid), ue = cut_begin(sg, cta + 1, p.d_grid);
         if (ue <= ub) continue;
@@ -1133,7 +1134,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
               tma_load_4d(smem_u32(stage_base) + hs * kStageBytes + kABytes, &h_map, smem_u32(&bars->full[hs]),
                           0, 0, ic * kAtoms, a, pol_x);
               ++hidx;
-              if (++hs == kStages) hs = 0;
+              if (++hs == kRing) hs = 0;
               if (++ic == kpe) { ic = 0; ++a; }
             }
           }
@@ -1194,7 +1195,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #if ACM_FFN_MX
             const size_t tile_at = static_cast<size_t>(a) * tpe + ti;
             bulk_store(p.hq + tile_at * (act_bytes / 2), smem_u32(hstage + hb * kHStageBytes), act_bytes / 2);
-            bulk_store(p.hq_scale + tile_at * kMxActScaleBytes, smem_u32(hstage + hb * kHStageBytes) + kMaxNodes * 128,
+            bulk_store(p.hq_scale + tile_at * kMxActScaleBytes, smem_u32(hstage + hb * kHStageBytes) + kHPieceBytes,
                        kMxActScaleBytes);
 #else
             asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];"
@@ -1214,15 +1215,14 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   } else if (warp >= 8) {
     // ------------------------------------------------------------------ unpacking warps
     // Two groups of four warps take the stages in turn.  Thread r of a group unpacks row r = lane r of tensor memory;
-    // every warp stores the stage's scales, both operands', into its quarter (rows i, i + 32, i + 64, i + 96 in lane i;
-    // copies by tcgen05.cp instead took 260 clocks a stage out of the MMAs' pipe).  A group's next
+    // every warp stores the stage's scales, both operands', into its quarter (rows i, i + 32, i + 64, i + 96 and nodes i,
+    // i + 32 in lane i; copies by tcgen05.cp instead took 260 clocks a stage out of the MMAs' pipe).  A group's next
     // record is loaded while the stage at hand is being stored, and given back behind it.
     const int r = threadIdx.x & 127, group = (warp - 8) >> 2;
     const uint32_t my_lane = static_cast<uint32_t>((warp & 3) * 32) << 16;
     bool ok = true;
     unsigned it = static_cast<unsigned>(group), total = 0;
-    uint32_t ri = static_cast<uint32_t>(group), rpar = 0, ai = static_cast<uint32_t>(group), apar = 0;
-    uint32_t ai_done = static_cast<uint32_t>(group ^ 1);      // of the stage kMxA before the group's next one from stage kMxA on
+    uint32_t ri = static_cast<uint32_t>(group), rpar = 0, s = static_cast<uint32_t>(group), par = 0;
     uint4 q[4];
     uint32_t sa[4];
     auto wait_raw = [&]() -> bool {
@@ -1265,16 +1265,8 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       // (scale bytes above the limit, which no registered tensor holds, count as the limit)
 #pragma unroll
       for (int g = 0; g < 4; ++g) so[g] = __vminu4(sa[g], 0x80808080u);
-      const uint32_t s = it % kMxA, par = (it / kMxA) & 1u;
       if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->empty[s]), par ^ 1u, quit, kSiteStageEmpty)))) break;
       tc_fence_after();
-      if (it >= static_cast<unsigned>(kMxA)) {
-        // the stage before in this slot has been multiplied: so have its activations (a commit of their own would cost
-        // the MMAs' pipe 60 clocks a stage)
-        if (r == 0) mbar_arrive(smem_u32(&bars->act_empty[ai_done]));
-        ai_done += 2u;
-        if (ai_done >= static_cast<uint32_t>(p.n_act)) ai_done -= static_cast<uint32_t>(p.n_act);
-      }
       tmem_st32(tmem_base + my_lane + kAcc * kAccCols + s * kMxACols, o);
       const uint32_t sf = tmem_base + my_lane + kAcc * kAccCols + kMxA * kMxACols + s * kMxScaleCols;
       tmem_st4(sf, so[0], so[1], so[2], so[3]);
@@ -1283,17 +1275,19 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         if (!(ok = wait_raw())) break;
         load_raw();
       }
-      if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->act[ai]), apar, quit, kSiteActStage)))) break;
-      const uint4* S = reinterpret_cast<const uint4*>(act_scale_base + ai * 2 * kMxActScaleBytes) + lane;
-      const uint4 lo = S[0], hi = S[kMxActScaleBytes / 16];      // two half-stages, two bytes of a word each
-      tmem_st4(sf + 4, __byte_perm(lo.x, hi.x, 0x5410), __byte_perm(lo.y, hi.y, 0x5410), __byte_perm(lo.z, hi.z, 0x5410),
-               __byte_perm(lo.w, hi.w, 0x5410));
+      if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->act[s]), par, quit, kSiteActStage)))) break;
+      const uint2* S = reinterpret_cast<const uint2*>(act_scale_base + s * 2 * kMxActScaleBytes) + lane;
+      const uint2 lo = S[0], hi = S[kMxActScaleBytes / 8];      // two half-stages, two bytes of a word each
+      const uint32_t s0 = __byte_perm(lo.x, hi.x, 0x5410), s1 = __byte_perm(lo.y, hi.y, 0x5410);
+#pragma unroll
+      for (int pc = 0; pc < kMxPieces; ++pc)      // (no scale is below 8; that of a block that is not finite has to be NaN once)
+        tmem_st2(sf + 4 + 4 * pc, s0 - pc * (kMxPieceShift * 0x01010101u), s1 - pc * (kMxPieceShift * 0x01010101u));
       tmem_st_wait();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&bars->full[s]));
-      ai += 2u;
-      if (ai >= static_cast<uint32_t>(p.n_act)) { ai -= static_cast<uint32_t>(p.n_act); apar ^= 1u; }
+      s += 2u;
+      if (s >= kRing) { s -= kRing; par ^= 1u; }
       if (fetched) release_raw();
      }
     }
@@ -1312,19 +1306,12 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #endif
     bool ok = true, waited = !early;
 #if ACM_FFN_MX
-    // 32 node columns from column c on (the last 16 only if there are that many): both pieces' sums
+    // 32 node columns from column c on (the last 16 only if there are that many)
     auto load_32 = [&](uint32_t b, int c, int np, float (&v)[32]) {
-      float v2[32];
       const uint32_t at = tmem_base + lane_addr + b * kAccCols + c;
       tmem_ld16(at, v);
-      tmem_ld16(at + np, v2);
-      if (c + 16 < np) {
-        tmem_ld16(at + 16, v + 16);
-        tmem_ld16(at + np + 16, v2 + 16);
-      }
+      if (c + 16 < np) tmem_ld16(at + 16, v + 16);
       tmem_ld_wait();
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] += v2[j];
     };
     auto release_acc = [&](uint32_t b) {
       tc_fence_before();
@@ -1427,13 +1414,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
                   const __nv_bfloat162 pair = __floats2bfloat162_rn(hval[0], hval[1]);
                   h2[i / 2] = *reinterpret_cast<const uint32_t*>(&pair);
                 }
-                MxBlock blk;
-                mx_split_block(h2, blk);
-                const int tb = p.n_pad + t;
-                mx_store_rows(hs, blk, t, tb, half);
-                unsigned char* scales = hs + kMaxNodes * 128 + half;
-                scales[mx_scale_at(t)] = blk.scale_a;
-                scales[mx_scale_at(tb)] = blk.scale_b;
+                mx_store_block(hs, hs + kHPieceBytes, h2, t, p.n_pad, half);
               }
               fence_proxy_async_smem();
               mbar_arrive(smem_u32(&bars->hst_full[0]));
@@ -1696,12 +1677,9 @@ k_ffn_f32_down(const float* __restrict__ down, const float* __restrict__ shared_
 
 #if ACM_FFN_MX
 namespace {
-// Ring depths for a launch of n_pad node columns: as many activation stages as there is room for with a packed record
-// each, then records with what is left (at least 7 of either).
-void mx_rings(int n_pad, int* n_act, int* n_raw) {
-  const int left = kMxRingBytes, act = n_pad * 256 + 2 * kMxActScaleBytes;
-  *n_act = min(kMaxAct, left / (act + kMxStageBytes));
-  *n_raw = min(kMaxRaw, (left - *n_act * act) / kMxStageBytes);
+// Packed records in flight in a launch of n_pad node columns.
+int mx_raw_stages(int n_pad) {
+  return min(kMaxRaw, (kMxRingBytes - kMxA * (n_pad * (kMxPieces * 128) + 2 * kMxActScaleBytes)) / kMxStageBytes);
 }
 }  // namespace
 cudaError_t ffn_mx_configure() {
@@ -1754,10 +1732,10 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
   a.xq = static_cast<const unsigned char*>(L.xq);
   a.xq_scale = a.xq + mx_act_scale_offset(L.H);
   a.xq_count = L.xq_count; a.xq_target = L.xq_target;
-  // (a slot's share of the activation buffer is 256 I bytes: up to 128 I of pieces; the scales lie behind all pieces)
+  // (a slot's share of the activation buffer is 256 I bytes: up to 192 I of pieces; the scales lie behind all pieces)
   a.hq = static_cast<unsigned char*>(L.hbuf);
-  a.hq_scale = a.hq + static_cast<size_t>(kMaxSlots) * 128 * L.I;
-  mx_rings(L.n_pad, &a.n_act, &a.n_raw);
+  a.hq_scale = a.hq + static_cast<size_t>(kMaxSlots) * (kMxPieces * 64) * L.I;
+  a.n_raw = mx_raw_stages(L.n_pad);
 #endif
   void* args[] = {const_cast<FfnMaps*>(&maps), const_cast<CUtensorMap*>(&x_map), const_cast<CUtensorMap*>(&h_map),
                   const_cast<CUtensorMap*>(&hs_map), &a};

@@ -227,19 +227,15 @@ __device__ __forceinline__ void split_x(const XqArgs& xa, const __nv_bfloat16* x
   const int per_node = H / 32;
   if (i == 0) *xa.next_count = 0;
   for (; i < T * per_node; i += n) {
-    const int t = i / per_node, block = i - t * per_node, half = block >> 1, tb = xa.n_pad + t;
+    const int t = i / per_node, block = i - t * per_node, half = block >> 1;
     uint32_t w[16];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const uint4 v = __ldcg(reinterpret_cast<const uint4*>(x + static_cast<size_t>(t) * H + 32 * block + 8 * j));
       w[4 * j] = v.x; w[4 * j + 1] = v.y; w[4 * j + 2] = v.z; w[4 * j + 3] = v.w;
     }
-    MxBlock k;
-    mx_split_block(w, k);
-    mx_store_rows(xa.xq + static_cast<size_t>(half) * (2 * xa.n_pad * 64), k, t, tb, block & 1);
-    unsigned char* sc = xa.xq + mx_act_scale_offset(H) + static_cast<size_t>(half) * kMxActScaleBytes + (block & 1);
-    sc[mx_scale_at(t)] = k.scale_a;
-    sc[mx_scale_at(tb)] = k.scale_b;
+    mx_store_block(xa.xq + static_cast<size_t>(half) * (kMxPieces * xa.n_pad * 64),
+                   xa.xq + mx_act_scale_offset(H) + static_cast<size_t>(half) * kMxActScaleBytes, w, t, xa.n_pad, block & 1);
   }
   __syncthreads();
   if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(xa.count) : "memory");

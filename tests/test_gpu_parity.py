@@ -1004,9 +1004,8 @@ def test_wide_batch_shares_one_pass_over_the_experts(c, sizes):
 
 @pytest.mark.parametrize("T,H,I", [(1, 128, 128), (16, 256, 384), (17, 2048, 128), (48, 1152, 640), (64, 4096, 256)])
 def test_mxfp4_activation_pieces(T, H, I):
-    """The MXFP4 kernel multiplies bf16 activations as two 8-bit pieces each: for ordinary rows, rows of any magnitude and
-    rows with outliers (features 2^11 times the others in the same block of 32 keep all their bits) the output is as close
-    to 64 bits as the bf16 kernel's on the dequantised weights -- in the fused call, whose router kernel stores the pieces,
+    """The MXFP4 kernel multiplies bf16 activations as three 8-bit pieces each: for ordinary rows, rows of any magnitude and
+    rows with outliers 2^11 times the others (what becomes of the others: the test below) the output is as close to 64 bits as the bf16 kernel's on the dequantised weights -- in the fused call, whose router kernel stores the pieces,
     and in acm_expert_ffn, which has a kernel for it.  A row that is not finite stays so, the others do not notice."""
     cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, n_nodes=T, hidden=H, inter=I, n_experts=24, zipf_bias=False)
     ctx = _ctx(cfg, n_layers=2)
@@ -1042,6 +1041,39 @@ def test_mxfp4_activation_pieces(T, H, I):
         rest = [t for t in range(T) if t != T // 2]
         assert torch.isfinite(bad[rest]).all()
         assert float((bad[rest] - alone[rest]).abs().max()) <= 1e-3 * float(alone[rest].double().pow(2).mean().sqrt())
+    ctx.close()
+
+
+@pytest.mark.parametrize("p", [11, 14, 17, 20, 24, 28])
+def test_mxfp4_small_features_beside_large_ones(p):
+    """One feature in 32 is 2^p (or almost 2^(p+1)) times the others and no expert has a weight for it: the output then
+    depends on the small ones alone, which must have kept all their bits -- in the hidden states' pieces that the router
+    kernel stores, and in those of acm_expert_ffn."""
+    T, H, I = 33, 1024, 256
+    cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, n_nodes=T, hidden=H, inter=I, n_experts=24, zipf_bias=False)
+    w = wl.layer_weights_mxfp4(cfg, 0, DEV)
+    w["gate_up_codes"].view(24, 2 * I, H // 32, 32)[..., 5] = 0
+    w["w_router"].view(24, H // 32, 32)[..., 5] = 0
+    gu, dn = (torch.tensor(oracle.dequantize_mxfp4(w[n + "_codes"], w[n + "_scales"])).to(torch.bfloat16).to(DEV) for n in ("gate_up", "down"))
+    x = wl.hidden_states(cfg, 0, DEV)
+    big = torch.tensor([1.0, -1.9921875, -1.0, 1.9921875], device=DEV) * 2.0 ** p
+    x.view(T, H // 32, 32)[..., 5] = big[torch.arange(T * H // 32, device=DEV) % 4].view(T, H // 32)
+    ctx = _ctx(cfg, n_layers=2)
+    ctx.set_layer_weights_mxfp4(0, w["w_router"], None, acm.pack_mxfp4_gate_up(w["gate_up_codes"], w["gate_up_scales"]),
+                                acm.pack_mxfp4_down(w["down_codes"], w["down_scales"]))
+    ctx.set_layer_weights(1, w["w_router"], None, gu, dn)
+    alpha = torch.ones(T, device=DEV)
+    out, idx, wt, _, _ = ctx.moe_verify(0, x, alpha, want=True)
+    bf16 = ctx.moe_verify(1, x, alpha)
+    alone = ctx.expert_ffn(0, x, idx, wt)
+    assert ctx.device_status() == acm.OK
+    ref = oracle.expert_ffn(x, idx.cpu().numpy(), wt.cpu().numpy(), gu, dn)
+    norm = np.sqrt((ref ** 2).sum())
+    off = lambda o: np.sqrt(((o.double().cpu().numpy() - ref) ** 2).sum()) / norm
+    # (both round the activation between the two products to bf16, 1.7e-3 of the output, from sums that differ in their last
+    # bits; over 33 rows the norm of those roundings agrees to a few per cent)
+    for o in (out, alone):
+        assert off(o) <= 1.1 * off(bf16), (p, off(o), off(bf16))
     ctx.close()
 
 

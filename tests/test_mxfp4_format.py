@@ -1,6 +1,7 @@
 """MXFP4 storage (E2M1 codes, one E8M0 scale per 32 elements): the oracle's dequantiser against the format's
 definition, the input quantiser against it, and the library's tiled layout as a pure permutation."""
 import numpy as np
+import pytest
 import torch
 
 import oracle
@@ -95,3 +96,43 @@ def test_tiled_layout_is_a_permutation_of_the_plain_one():
     blk = t[1, 1, 0]
     np.testing.assert_array_equal(_unpack_words(blk[: 128 * 64].reshape(128, 64)), dc.numpy()[1][128:256, 0:128])
     np.testing.assert_array_equal(blk[128 * 64:].reshape(128, 4), ds.numpy()[1][128:256, 0:4])
+
+
+def _block_values(top, exponent, below):
+    """32 bf16 values: the largest `top` / 128 * 2^exponent, then values 2^below of its power of two, of every significand."""
+    return [top / 128 * 2.0 ** exponent] + [s * m / 128 * 2.0 ** (exponent + below) for m, s in zip(range(128, 256), [1, -1] * 64)]
+
+
+def test_activation_pieces_keep_a_bf16_exactly_down_to_2_to_the_minus_31_of_the_block():
+    """What the MXFP4 kernels multiply in the place of a bf16 (three e5m2 pieces): all 128 significands at every distance
+    from the block's largest value, which is a power of two or almost the next one -- and at both ends of the exponents."""
+    for exponent in (0, 5, -40, 127, -100, -126):
+        for top in (128, 171, 255):
+            for below in range(0, -60, -1):
+                if exponent + below - 7 < -133:            # (bf16 has nothing finer)
+                    continue
+                big, rest = _block_values(top, exponent, below)[0], _block_values(top, exponent, below)[1:]
+                rest = [v for v in rest if abs(v) <= big]
+                for at in range(0, len(rest), 31):
+                    vals = torch.tensor(([big] + rest[at:at + 31] + [0.0] * 31)[:32], dtype=torch.float64)
+                    assert torch.equal(vals.to(torch.bfloat16).double(), vals)
+                    pieces, scales = acm.mxfp4_activation_pieces(vals.to(torch.bfloat16))
+                    got = (pieces.view(torch.float8_e5m2).double() * torch.exp2(scales.double() - 127)[:, None]).sum(0)
+                    err = (got - vals).abs()
+                    assert float(err[vals.abs() >= big * 2.0 ** -31].max()) == 0.0, (exponent, top, below)
+                    assert float(err.max()) <= big * 2.0 ** -39
+
+
+def test_activation_pieces_of_special_blocks():
+    zero = torch.zeros(32, dtype=torch.bfloat16)
+    pieces, scales = acm.mxfp4_activation_pieces(zero)
+    assert (pieces.view(torch.float8_e5m2).double() == 0).all() and (scales < 255).all()
+    tiny = torch.arange(32, dtype=torch.float64) * 2.0 ** -133              # bf16 subnormals
+    pieces, scales = acm.mxfp4_activation_pieces(tiny.to(torch.bfloat16))
+    assert torch.equal((pieces.view(torch.float8_e5m2).double() * torch.exp2(scales.double() - 127)[:, None]).sum(0), tiny)
+    for bad in (float("inf"), -float("inf"), float("nan")):
+        x = torch.ones(32, dtype=torch.bfloat16)
+        x[17] = bad
+        assert int(acm.mxfp4_activation_pieces(x)[1][0]) == 255
+    with pytest.raises(ValueError):
+        acm.mxfp4_activation_pieces(torch.ones(31, dtype=torch.bfloat16))
