@@ -883,11 +883,6 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         p.stats->n_staged = n_stg;
         p.stats->n_streamed = bars->n_routed_slots;
       }
-      if (!ok) {
-        // giving up: let copies already in flight land before the CTA exits
-        const unsigned long long t0 = global_timer();
-        while (global_timer() - t0 < 200000ull) {}
-      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
@@ -960,12 +955,6 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         if (++b == kAcc) { b = 0; bpar ^= 1u; }
       }
     }
-    if (!ok) {
-      // giving up: wait (bounded) for the MMAs already issued before TMEM is released
-      if (lane == 0) umma_commit(smem_u32(&bars->drained));
-      const unsigned long long t0 = global_timer();
-      while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
-    }
 #if ACM_FFN_MX
   } else if (warp == 6) {
     // ------------------------------------------------------------------ activation producer
@@ -1025,11 +1014,6 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         }
       }
       ok = __all_sync(0xffffffffu, ok);
-    }
-    if (!ok) {
-      // giving up: let copies already in flight land before the CTA exits
-      const unsigned long long t0 = global_timer();
-      while (global_timer() - t0 < 200000ull) {}
     }
 #else
   } else if (warp == 6) {
@@ -1547,6 +1531,16 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
+    if (__any_sync(0xffffffffu, quit->flag)) {
+      // A role has given up, and any other may have left with work in flight: wait (bounded) for the MMAs before tensor
+      // memory is released -- a commit covers those of the lane that makes it, hence the same election -- and for copies
+      // to land before the CTA's shared memory is.
+      if (elect_one()) umma_commit(smem_u32(&bars->drained));
+      const unsigned long long t0 = global_timer();
+      while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
+      while (global_timer() - t0 < 200000ull) {}
+      __syncwarp();
+    }
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }

@@ -213,6 +213,33 @@ def test_wait_that_runs_out_is_reported_and_the_context_recovers():
     ctx.close()
 
 
+@pytest.mark.parametrize("T", [1, 64])
+def test_a_wait_that_runs_out_on_an_mxfp4_layer(T):
+    """The MXFP4 kernel gives up a wait for words that nobody publishes: every CTA reports it and leaves with its tensor
+    memory released, since correct calls follow -- the fused one, and the expert FFN alone, whose MMAs and copies run
+    through all roles again."""
+    cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, hidden=512, inter=256, n_experts=32, n_nodes=T)
+    w = wl.layer_weights_mxfp4(cfg, 0, DEV)
+    gu, dn = (torch.tensor(oracle.dequantize_mxfp4(w[n + "_codes"], w[n + "_scales"])).to(torch.bfloat16).to(DEV) for n in ("gate_up", "down"))
+    ctx = acm.Context.for_config(cfg, n_layers=1)
+    ctx.set_layer_weights_mxfp4(0, w["w_router"], w["router_bias"], acm.pack_mxfp4_gate_up(w["gate_up_codes"], w["gate_up_scales"]),
+                                acm.pack_mxfp4_down(w["down_codes"], w["down_scales"]))
+    x = wl.hidden_states(cfg, 0, DEV)
+    alpha = torch.ones(T, device=DEV)
+    ctx.set_wait_limit(3_000_000)
+    for _ in range(3):
+        ctx.inject_unpublished_wait(0, x)
+        assert ctx.device_status() == acm.ERR_TIMEOUT
+        assert set(ctx.wait_report()) == {2}
+        out, idx, wt, _, _ = ctx.moe_verify(0, x, alpha, want=True)
+        alone = ctx.expert_ffn(0, x, idx, wt)
+        assert ctx.device_status() == acm.OK and set(ctx.wait_report()) == {0}
+        ref = oracle.expert_ffn(x, idx.cpu().numpy(), wt.cpu().numpy(), gu, dn)
+        for o in (out, alone):
+            assert float(np.abs(o.double().cpu().numpy() - ref).max()) <= 2e-2 * float(np.sqrt(np.mean(ref ** 2)))
+    ctx.close()
+
+
 def test_sequence_tags_coming_round_do_not_revive_old_words():
     """The words the kernels publish for one another carry the call's sequence number in 16 bits.  A batch call
     writes words for eight blocks; 65534 single-block calls later the tags come round, and a second batch call,
