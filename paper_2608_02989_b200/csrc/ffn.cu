@@ -1279,6 +1279,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       if (fetched) release_raw();
      }
     }
+    if (!ok) tmem_st_wait();      // (left between a stage's stores and its wait: tensor memory is released behind this)
 #endif
   } else {
     // ------------------------------------------------------------------ epilogue (128 threads)
