@@ -371,6 +371,17 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}\n" : "=r"(r));
   return r != 0;
 }
+// The end of a CTA in which a role has given up, so that any other may have left with work in flight: waits (bounded) for the
+// MMAs before tensor memory is released -- a commit covers those of the lane that makes it, hence the issuer's election --
+// and for copies to land before the CTA's shared memory is.  By the issuing warp.  (Out of line: in line it put 0.14 us
+// on a launch that never runs it.)
+__device__ __noinline__ void drain_cta(uint32_t drained) {
+  if (elect_one()) umma_commit(drained);
+  const unsigned long long t0 = global_timer();
+  while (!mbar_try_wait(drained, 0) && global_timer() - t0 < 1000000ull) {}
+  while (global_timer() - t0 < 200000ull) {}
+  __syncwarp();
+}
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
@@ -699,7 +710,8 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   const int n_seg_fixed = bars->plan.n_seg;
   auto have_seg = [&](int si, bool wait_for_plan) -> bool {
     if (pre) {
-      if (si == 1 && wait_for_plan && !mbar_wait(smem_u32(&bars->plan_ready), 0u, quit, kSitePlanReady)) return false;
+      if (si == 1 && wait_for_plan && !mbar_wait(smem_u32(&bars->plan_ready), 0u, quit, kSitePlanReady))
+        return false;
       return si < bars->plan.n_seg;
     } else {
       return si < n_seg_fixed;
@@ -1532,16 +1544,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
-    if (__any_sync(0xffffffffu, quit->flag)) {
-      // A role has given up, and any other may have left with work in flight: wait (bounded) for the MMAs before tensor
-      // memory is released -- a commit covers those of the lane that makes it, hence the same election -- and for copies
-      // to land before the CTA's shared memory is.
-      if (elect_one()) umma_commit(smem_u32(&bars->drained));
-      const unsigned long long t0 = global_timer();
-      while (!mbar_try_wait(smem_u32(&bars->drained), 0) && global_timer() - t0 < 1000000ull) {}
-      while (global_timer() - t0 < 200000ull) {}
-      __syncwarp();
-    }
+    if (__any_sync(0xffffffffu, quit->flag)) drain_cta(smem_u32(&bars->drained));
     tc_fence_after();
     tmem_dealloc(tmem_base, kTmemCols);
   }
