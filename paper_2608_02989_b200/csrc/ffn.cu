@@ -238,6 +238,20 @@ __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, GiveU
     }
   }
 }
+// The wait for the rest of the plan.  The threads of a role must agree on its outcome -- one that left alone would strand the
+// others at their next vote -- so it looks at the barrier only, not at the flag, and its limit is eight times that of the
+// two polls behind which the barrier is opened, found or not.
+__device__ __noinline__ bool mbar_wait_plan(uint32_t bar, GiveUp* g) {
+  const unsigned long long t0 = global_timer();
+  for (;;) {
+    for (int i = 0; i < 64; ++i)
+      if (mbar_try_wait(bar, 0u)) return true;
+    if (limit_passed(t0, 8 * g->limit_ns)) {
+      give_up(g, kSitePlanReady);
+      return false;
+    }
+  }
+}
 // One inlined poll for the common case (the phase is already complete), the bounded loop out of line: the
 // single-thread roles pay every instruction of their per-stage loop.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, GiveUp* g, int site) {
@@ -710,7 +724,8 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   const int n_seg_fixed = bars->plan.n_seg;
   auto have_seg = [&](int si, bool wait_for_plan) -> bool {
     if (pre) {
-      if (si == 1 && wait_for_plan && !mbar_wait(smem_u32(&bars->plan_ready), 0u, quit, kSitePlanReady))
+      if (si == 1 && wait_for_plan && !mbar_try_wait(smem_u32(&bars->plan_ready), 0u) &&
+          !mbar_wait_plan(smem_u32(&bars->plan_ready), quit))
         return false;
       return si < bars->plan.n_seg;
     } else {
