@@ -85,3 +85,15 @@ def test_no_silent_fallback_without_a_gpu(lib):
     with pytest.raises(acm.AcmError) as e:
         acm.Context(256, 16, 2, 128)
     assert e.value.code in (acm.ERR_CUDA, acm.ERR_UNSUPPORTED)
+
+
+@pytest.mark.parametrize("missing", ["_current_raw_stream", "_current_device"])
+def test_current_stream_without_torchs_private_functions(monkeypatch, missing):
+    """A torch that lacks either of the two private functions behind the default stream: its public one is asked."""
+    class Stream:
+        cuda_stream = 0x1234
+    monkeypatch.setattr(acm, missing, None)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    assert acm._stream(None) == 0x1234
+    Stream.cuda_stream = 7
+    assert acm._stream(Stream) == 7
