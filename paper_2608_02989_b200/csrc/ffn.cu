@@ -223,31 +223,21 @@ __device__ __noinline__ void give_up(GiveUp* g, int site) {
 }
 // Returns false if the limit ran out (the status is raised once) or the CTA has already given up; callers
 // then skip the rest of their work.
+// The wait for the rest of the plan is each thread's own, and the threads of a role must agree on its outcome -- one that
+// left alone would strand the others at their next vote.  So it looks at the barrier only, not at the flag, and its limit
+// is eight times that of the two polls behind which the barrier is opened, found or not.
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, GiveUp* g, int site) {
-  if (g->flag) return false;
+  const bool for_plan = site == kSitePlanReady;
+  if (g->flag && !for_plan) return false;
   for (int i = 0; i < 1024; ++i)
     if (mbar_try_wait(bar, parity)) return true;
   const unsigned long long t0 = global_timer();
   for (;;) {
     for (int i = 0; i < 64; ++i)
       if (mbar_try_wait(bar, parity)) return true;
-    if (g->flag) return false;
-    if (limit_passed(t0, g->limit_ns)) {
+    if (g->flag && !for_plan) return false;
+    if (limit_passed(t0, for_plan ? 8 * g->limit_ns : g->limit_ns)) {
       give_up(g, site);
-      return false;
-    }
-  }
-}
-// The wait for the rest of the plan.  The threads of a role must agree on its outcome -- one that left alone would strand the
-// others at their next vote -- so it looks at the barrier only, not at the flag, and its limit is eight times that of the
-// two polls behind which the barrier is opened, found or not.
-__device__ __noinline__ bool mbar_wait_plan(uint32_t bar, GiveUp* g) {
-  const unsigned long long t0 = global_timer();
-  for (;;) {
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait(bar, 0u)) return true;
-    if (limit_passed(t0, 8 * g->limit_ns)) {
-      give_up(g, kSitePlanReady);
       return false;
     }
   }
@@ -724,9 +714,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
   const int n_seg_fixed = bars->plan.n_seg;
   auto have_seg = [&](int si, bool wait_for_plan) -> bool {
     if (pre) {
-      if (si == 1 && wait_for_plan && !mbar_try_wait(smem_u32(&bars->plan_ready), 0u) &&
-          !mbar_wait_plan(smem_u32(&bars->plan_ready), quit))
-        return false;
+      if (si == 1 && wait_for_plan && !mbar_wait(smem_u32(&bars->plan_ready), 0u, quit, kSitePlanReady)) return false;
       return si < bars->plan.n_seg;
     } else {
       return si < n_seg_fixed;
