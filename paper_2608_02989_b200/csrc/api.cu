@@ -337,18 +337,21 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
                         bool anchors_first = false, int widest_block = 0) {
   const acm_model_desc& d = c->desc;
   const int n_pad = (T + 15) / 16 * 16;
-  acm_status st = ensure_h_maps(c, n_pad);
-  if (st != ACM_OK) return st;
   CUtensorMap x_map;
-  st = encode_x(c, &x_map, x, T, n_pad);
-  if (st != ACM_OK) return st;
-  FfnMaps maps = L.maps;
-  if (L.has_pool) {
-    maps.staged_gate_up = L.pool_map_gu;
-    maps.staged_down = L.pool_map_dn;
-  } else if (c->stage_gate_up) {
-    maps.staged_gate_up = c->stage_map_gu;
-    maps.staged_down = c->stage_map_dn;
+  FfnMaps maps;
+  if (!L.mx) {      // (the MXFP4 kernel has no tensor copies)
+    acm_status st = ensure_h_maps(c, n_pad);
+    if (st != ACM_OK) return st;
+    st = encode_x(c, &x_map, x, T, n_pad);
+    if (st != ACM_OK) return st;
+    maps = L.maps;
+    if (L.has_pool) {
+      maps.staged_gate_up = L.pool_map_gu;
+      maps.staged_down = L.pool_map_dn;
+    } else if (c->stage_gate_up) {
+      maps.staged_gate_up = c->stage_map_gu;
+      maps.staged_down = c->stage_map_dn;
+    }
   }
   FfnLaunch p;
   p.T = T; p.H = d.hidden; p.I = d.inter; p.n_pad = n_pad;
@@ -399,7 +402,7 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
     p.xq = c->ws.xq; p.xq_count = c->ws.xq_count + c->xq_word; p.xq_target = c->xq_target;
     p.mx_gate_up = L.has_pool ? L.pool_gate_up : L.mx_gate_up;      // a pool: slot s of the pool tensors
     p.mx_down = L.has_pool ? L.pool_down : L.mx_down;
-    ACM_CUDA(launch_ffn_mxfp4(p, maps, x_map, c->h_map[li], c->h_store_map[li], s));
+    ACM_CUDA(launch_ffn_mxfp4(p, s));
   } else {
     ACM_CUDA(launch_ffn_bf16(p, maps, x_map, c->h_map[li], c->h_store_map[li], s));
   }

@@ -145,16 +145,19 @@ struct __align__(8) BarriersT {
   unsigned long long tfull[kAcc];
   unsigned long long tempty[kAcc];
   unsigned long long drained;
+#if !ACM_FFN_MX
   unsigned long long frag_full;      // helper -> epilogue: the pre-summed fragments of the next cut tile (half) are in smem
   unsigned long long frag_free;      // epilogue -> helper: the fragment buffer may be overwritten
   unsigned long long helper;         // completion of the helper warp's bulk copy
   unsigned long long ost_full, ost_free;   // epilogue <-> publisher: outgoing fragment staged / copied out
-  unsigned long long hst_full[2], hst_free[2];   // epilogue <-> publisher: activation tile staged / stored
+#endif
+  unsigned long long hst_full[kHStages], hst_free[kHStages];   // epilogue <-> publisher: activation tile staged / stored
 #if ACM_FFN_MX
   unsigned long long raw[kMaxRaw], raw_empty[kMaxRaw];   // packed records: landed (-> unpacking warps) / read (-> producer)
   unsigned long long act[kMaxRing];      // activation stages landed (-> unpacking warps)
-#endif
+#else
   volatile uint32_t armed;           // stages whose barrier the weight producer has armed so far
+#endif
   volatile int32_t n_routed_slots;   // routed experts in this launch's work list (known with the complete list)
   uint32_t tmem_base;
   GiveUp give_up;
@@ -466,10 +469,11 @@ struct FfnArgs {
   const int32_t* slot_of;
   const float* wtab;
   acm_block_stats* stats;
-  __nv_bfloat16* hbuf;
   int32_t* ready;
+#if !ACM_FFN_MX
   float* frag;
   int32_t* frag_flag;
+#endif
   const uint32_t* sel_flag;
   int32_t sel_epoch;
   int sel_blocks;
@@ -510,9 +514,13 @@ __device__ __forceinline__ const CUtensorMap* pick_map(int src, const CUtensorMa
 // kN = node columns of an accumulator tile (see Geo).
 template <int kN>
 __global__ void __launch_bounds__(kThreads, 1)
+#if ACM_FFN_MX      // (every copy of it is a plain bulk one: no tensor maps)
+ACM_FFN_KERNEL(const FfnArgs p) {
+#else
 ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUtensorMap x_map,
            const __grid_constant__ CUtensorMap h_map, const __grid_constant__ CUtensorMap hs_map,
            const FfnArgs p) {
+#endif
   constexpr int kRing = Geo<kN>::kRing, kAccCols = kN, kTmemCols = Geo<kN>::kTmemCols;
 #if !ACM_FFN_MX
   constexpr int kStageBytes = Geo<kN>::kStageBytes;
@@ -561,12 +569,14 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     }
     mbar_init(smem_u32(&bars->drained), 1);
     mbar_init(smem_u32(&bars->plan_ready), 1);
+#if !ACM_FFN_MX
     mbar_init(smem_u32(&bars->frag_full), 1);
     mbar_init(smem_u32(&bars->frag_free), 128);
     mbar_init(smem_u32(&bars->helper), 1);
     mbar_init(smem_u32(&bars->ost_full), 128);
     mbar_init(smem_u32(&bars->ost_free), 1);
-    for (int b = 0; b < 2; ++b) {
+#endif
+    for (int b = 0; b < kHStages; ++b) {
       mbar_init(smem_u32(&bars->hst_full[b]), 128);
       mbar_init(smem_u32(&bars->hst_free[b]), 1);
     }
@@ -576,17 +586,19 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
     bars->give_up.where = p.wait_diag ? p.wait_diag + blockIdx.x : nullptr;
     bars->give_up.tag = p.launch_tag;
     if (p.wait_diag) p.wait_diag[blockIdx.x] = p.launch_tag;      // "this CTA of that launch has started"
+#if !ACM_FFN_MX
     bars->armed = 0;
+#endif
     fence_barrier_init();
   }
-  if (warp == 0 && lane == 0) {
 #if !ACM_FFN_MX
+  if (warp == 0 && lane == 0) {
     prefetch_tensormap(&maps.gate_up);
     prefetch_tensormap(&maps.down);
     prefetch_tensormap(&x_map);
     prefetch_tensormap(&h_map);
-#endif
   }
+#endif
   if (warp == 1) {
     tmem_alloc(smem_u32(&bars->tmem_base), kTmemCols);
     tmem_relinquish();
@@ -1691,8 +1703,7 @@ cudaError_t ffn_mx_configure() {
   return cudaFuncSetAttribute(ACM_FFN_KERNEL<kMaxNodes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(Geo<kMaxNodes>::kSmemBytes));
 }
-cudaError_t launch_ffn_mxfp4(const FfnLaunch& L, const FfnMaps& maps, const CUtensorMap& x_map,
-                             const CUtensorMap& h_map, const CUtensorMap& hs_map, cudaStream_t s) {
+cudaError_t launch_ffn_mxfp4(const FfnLaunch& L, cudaStream_t s) {
 #else
 
 cudaError_t ffn_configure() {
@@ -1723,8 +1734,7 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
   a.T = L.T; a.H = L.H; a.I = L.I; a.n_pad = L.n_pad;
   a.act_mask = L.act_mask; a.resident = L.resident; a.li = L.li; a.n_shared = L.n_shared; a.slot_of = L.slot_of; a.wtab = L.wtab;
   for (int w = 0; w < 4; ++w) a.only[w] = L.only[w];
-  a.stats = L.stats; a.hbuf = static_cast<__nv_bfloat16*>(L.hbuf);
-  a.ready = L.ready; a.frag = L.frag; a.frag_flag = L.frag_flag;
+  a.stats = L.stats; a.ready = L.ready;
   a.sel_flag = L.sel_flag; a.sel_epoch = L.sel_epoch; a.sel_blocks = L.sel_blocks;
   a.anc_flag = (L.sel_blocks < 1 || L.sel_blocks > kMaxEarlyBlocks || L.li != 0 || L.resident || L.slot_of) ? nullptr : L.anc_flag;
   a.out = L.out; a.status = L.status; a.trace = L.trace;
@@ -1741,9 +1751,12 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
   a.hq = static_cast<unsigned char*>(L.hbuf);
   a.hq_scale = a.hq + static_cast<size_t>(kMaxSlots) * (kMxPieces * 64) * L.I;
   a.n_raw = mx_raw_stages(L.n_pad);
-#endif
+  void* args[] = {&a};
+#else
+  a.frag = L.frag; a.frag_flag = L.frag_flag;
   void* args[] = {const_cast<FfnMaps*>(&maps), const_cast<CUtensorMap*>(&x_map), const_cast<CUtensorMap*>(&h_map),
                   const_cast<CUtensorMap*>(&hs_map), &a};
+#endif
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(L.grid);
   cfg.blockDim = dim3(kThreads);
