@@ -51,7 +51,7 @@ def parse_args():
     ap.add_argument("--budget", type=int, default=22, help="B0 of the fixed-budget selectors")
     ap.add_argument("--mxfp4", action="store_true",
                     help="supplementary: the routed experts stored in MXFP4 (the configuration's weights quantised), "
-                         "expanded to bf16 inside the FFN kernel")
+                         "multiplied on the block-scaled tensor-core instruction")
     ap.add_argument("--zipf", action="store_true",
                     help="supplementary: give the configuration the Zipf(1.1) router bias that C3 has (skewed expert "
                          "popularity), e.g. --config 5 --zipf")

@@ -384,7 +384,10 @@ acm_status acm_ffn_plan_mxfp4(int n_experts_streamed, int n_anchor_first, int hi
  * scales[0] is 255 (NaN) if a value is not finite.  For inspection and for tests of that bound. */
 acm_status acm_mxfp4_activation_pieces(const uint16_t* values /*host*/, uint8_t* pieces /*host*/, uint8_t* scales /*host*/);
 
-/* How far the kernels of a fused call (acm_moe_verify, acm_moe_verify_batch, acm_moe_verify_host) overlap.
+/* How far the kernels of a fused call (acm_moe_verify, acm_moe_verify_batch, acm_moe_verify_host) overlap -- and, from
+ * ACM_OVERLAP_DEPENDENT on, whether the stage calls (acm_router, acm_select_eligible, acm_route_restricted,
+ * acm_expert_ffn) and the kernels of fp32 layers are launched as dependents of the kernel before them in the stream; each
+ * waits for that kernel, whoever launched it, before it touches anything but the router's weights.
  * The stages of Section 3.1-3.4 form a chain, and the expert FFN needs only part of its result to start:
  *   ACM_OVERLAP_NONE       plain stream order.  The FFN kernel is a cooperative launch, so the driver itself
  *                          checks that all its CTAs can be resident together.  The mode to use when anything

@@ -216,10 +216,9 @@ def pool_plan(n_experts, slot_expert, last_use, tick, activated):
 # contiguous copy, so the weights are stored tile by tile: per (expert, tile, stage) 8704 bytes =
 #   128 rows x 64 bytes of codes, then 128 rows x 4 scale bytes (one E8M0 byte per 32 K).
 # Inside each group of 8 consecutive K elements the codes sit in one 32-bit word with the even elements in
-# the low half and the odd ones in the high half (nibble j = element 2j, nibble 4+j = element 2j+1), which
-# is the order the kernel's expansion to bf16 pairs wants; the four 16-byte pieces of a row (32 K each) are
-# stored rotated by the row number (piece p of row r at position p ^ ((r >> 1) & 3)).  These functions only
-# permute bytes.
+# the low half and the odd ones in the high half (nibble j = element 2j, nibble 4+j = element 2j+1); the four
+# 16-byte pieces of a row (32 K each) are stored rotated by the row number (piece p of row r at position
+# p ^ ((r >> 1) & 3)).  These functions only permute bytes.
 MX_STAGE_BYTES = 128 * 64 + 128 * 4
 
 

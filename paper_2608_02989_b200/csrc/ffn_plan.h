@@ -24,9 +24,12 @@
 // others are still in their anchor tile:
 //   fewer rest tiles than CTAs: they are dealt whole, one per CTA, to the idle CTAs first (no exchange at all);
 //   else as above.  The anchors' experts are complete early: their down projection comes first.
-// A launch of the MXFP4 kernel (kUncut) deals every tile whole, behind the anchors to the idle CTAs first: its tiles take
-// a third of the bf16 ones' time, less than the exchange of a cut tile's partial sums (7-9 us, during which the CTA that
-// waits for them finalises nothing else).
+// A launch of the MXFP4 kernel (kUncut) deals every tile whole, behind the anchors to the idle CTAs first.  At hidden 2048 a
+// tile takes 6 us (16 stages), less than the exchange of a cut tile's partial sums (7-9 us, during which the CTA that
+// waits for them finalises nothing else).  At hidden 4096 it takes 12.5 us: a second round of a few tiles then costs more
+// than a cut would, but a layer still less than with the kernel that cut them and expanded the weights to bf16 (4096 x 1536,
+// 64 nodes, 8 / 20 / 100 experts: 72 / 120 / 516 -> 62 / 93 / 424 us; hidden 1024 to 4096, inter 512 to 1536, 8 to 100
+// experts, 1 to 64 nodes: none slower).
 // (Measured and dropped, bf16: every tile whole with the CTAs that get one tile less taking down work early -- the last
 // round's experts then start their down projection too late; the leftover tiles after the whole rounds instead of
 // before them; the leftover tiles cut over the idle CTAs only.)

@@ -745,8 +745,8 @@ def _mx_layer(cfg, layer=0):
 @pytest.mark.parametrize("shape", [dict(inter=256, n_experts=32), dict(), dict(hidden=4096, inter=1536, n_nodes=33)])
 def test_mxfp4_layer_equals_the_bf16_layer_with_the_dequantised_weights(shape):
     """Expert weights in MXFP4: sets and routes as always (the router is bf16); the FFN output against the oracle
-    run on the dequantised weights, and against the library's own bf16 kernel on them, which does the same
-    arithmetic in the same order."""
+    run on the dequantised weights, and against the library's own bf16 kernel on them, which adds the same products
+    in another order."""
     cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, **shape)
     ctx = _ctx(cfg, n_layers=2)
     w = _mx_layer(cfg)
@@ -764,7 +764,8 @@ def test_mxfp4_layer_equals_the_bf16_layer_with_the_dequantised_weights(shape):
         np.testing.assert_array_equal(_u32(mask), _u32(ref_mask))
         ffn = oracle.expert_ffn(x, idx.cpu().numpy(), wt.cpu().numpy(), w["gate_up_deq"], w["down_deq"])
         _ffn_check(out, ffn, "MXFP4 layer")
-        # same tiles, same MMAs, same order of additions inside a tile; split-K partial sums meet in L2 in any order
+        # the same products, summed in fp32 in another order (pieces of the activations, whole tiles); the activation between
+        # the two products then rounds to the other bf16 now and then, 2^-8 of one of inter terms
         rms = float(ref_out.double().pow(2).mean().sqrt())
         assert float((out - ref_out).abs().max()) <= 1e-3 * rms
     ctx.close()
@@ -794,7 +795,7 @@ def test_mxfp4_scale_bytes_up_to_the_limit_and_beyond():
         out, idx, wt, mask, stats = ctx.moe_verify(0, x, alpha.to(DEV), want=True)
         ref_out = ctx.moe_verify(1, x, alpha.to(DEV))
         assert ctx.device_status() == acm.OK
-        # the expansion is exact: the bf16 kernel on the dequantised weights does the same arithmetic
+        # codes and scales enter the products exactly: the bf16 kernel on the dequantised weights adds the same ones
         rms = float(ref_out.double().pow(2).mean().sqrt())
         assert float((out - ref_out).abs().max()) <= 1e-3 * rms
         if len(names) == 1:
