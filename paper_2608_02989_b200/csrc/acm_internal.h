@@ -12,6 +12,19 @@ namespace acm {
 constexpr int kMaxExperts = 128;   // E limit; also the padded length of expert-axis tree sums
 constexpr int kMaxTopK = 8;
 constexpr int kMaxNodes = 64;      // T limit of one verification block; the FFN kernel handles node columns 64 at a time
+// Launches that k_ffn_bf16_small takes, whose CTAs keep the activations they make.  It saves a few microseconds a launch and
+// pays with reductions into the output that grow with the nodes: up to 8 nodes they stay behind the weights, and the smaller an
+// expert, the more nodes the saving is worth.  us a layer, the kernel before -> this one, with 12 / 20 / 40 experts:
+//   30 nodes  1024 x 512 28.3 / 30.9 / 40.6 -> 24.7 / 26.2 / 33.6     1536 x 768 33.1 / 38.4 / 56.5 -> 30.9 / 36.0 / 54.4 (32 nodes)
+//             1664 x 1152 35.3 / 48.8 / 78.5 -> 41.0 / 50.2 / 79.3    2048 x 768 36.5 / 42.7 / 68.2 -> 34.1 / 43.0 / 65.3
+//   16 nodes  2048 x 768 35.9 / 42.7 / 68.1 -> 31.4 / 39.1 / 66.0     1664 x 1152 35.1 / 47.5 / 78.2 -> 34.6 / 45.9 / 76.3
+//             2048 x 1408 43.2 / 61.9 / 111 -> 43.8 / 63.2 / 112      4096 x 1536 81.2 / 124 / 238 -> 82.5 / 125 / 233
+//    8 nodes  2048 x 1408 43.2 / 62.0 / 111 -> 42.3 / 61.7 / 111      4096 x 1536 80.4 / 124 / 236 -> 79.8 / 124 / 232
+constexpr int kSmallNodes = 32;
+inline bool small_block(int T, int hidden, int inter) {
+  const long long expert = static_cast<long long>(hidden) * inter;
+  return T <= (expert <= 1280 * 1024 ? kSmallNodes : expert <= 2048 * 1152 ? 16 : 8);
+}
 constexpr int kWideNodes = 128;    // T limit of a batch of blocks = node columns of one wide FFN accumulator tile
 constexpr int kWtabStride = kWideNodes;   // row length of the combine-weight table [expert][node]
 constexpr int kMaxShared = 4;
@@ -165,6 +178,7 @@ struct FfnMaps {               // TMA descriptors of one layer (bf16 path)
   CUtensorMap gate_up, down;               // routed experts  [E,2I,H] / [E,H,I]
   CUtensorMap shared_gate_up, shared_down; // shared experts (copies of the above if none)
   CUtensorMap staged_gate_up, staged_down; // staging slots   (copies of the above if none)
+  CUtensorMap down_slice, shared_down_slice, staged_down_slice;   // the down tensors in boxes of 256 rows x 64 features (small blocks)
 };
 struct FfnLaunch {
   int T, H, I, n_pad;

@@ -35,7 +35,7 @@ struct Layer {
   int n_slots = 0;
   void* pool_gate_up = nullptr;         // device [n_slots, 2I, H]
   void* pool_down = nullptr;            // device [n_slots, H, I]
-  CUtensorMap pool_map_gu, pool_map_dn;
+  CUtensorMap pool_map_gu, pool_map_dn, pool_map_ds;
   std::vector<int32_t> slot_expert;     // slot -> expert id or -1
   std::vector<int32_t> expert_slot;     // expert id -> slot or -1
   std::vector<uint64_t> last_use;       // slot -> tick of its last use
@@ -146,7 +146,7 @@ struct acm_ctx {
   // staging of non-resident experts
   void* stage_gate_up = nullptr;
   void* stage_down = nullptr;
-  CUtensorMap stage_map_gu, stage_map_dn;
+  CUtensorMap stage_map_gu, stage_map_dn, stage_map_ds;
   int32_t* host_stage_list = nullptr;    // pinned + mapped: [0] = count, [1..] = expert ids
   int32_t* host_stage_list_dev = nullptr;
   int32_t* slot_table_pinned = nullptr;        // pinned ring of expert -> slot tables in flight (kSlotTableRing x kMaxExperts)
@@ -264,6 +264,14 @@ acm_status encode_down(acm_ctx* c, CUtensorMap* m, const void* base, uint64_t n)
   const uint32_t box[4] = {64, 128, 2, 1};
   return encode_view(c, m, base, 4, dims, strides, box);
 }
+// ... in boxes of 256 rows x 1 atom (32 KB), for small blocks.
+acm_status encode_down_slice(acm_ctx* c, CUtensorMap* m, const void* base, uint64_t n) {
+  const uint64_t H = c->desc.hidden, I = c->desc.inter;
+  const uint64_t dims[4] = {64, H, I / 64, n};
+  const uint64_t strides[3] = {I * 2, 128, H * I * 2};
+  const uint32_t box[4] = {64, 256, 1, 1};
+  return encode_view(c, m, base, 4, dims, strides, box);
+}
 // x [T, H] as {k in atom, node, atom of H}; one box = n_pad nodes x 2 atoms.
 acm_status encode_x(acm_ctx* c, CUtensorMap* m, const void* x, int T, int n_pad) {
   const uint64_t H = c->desc.hidden;
@@ -334,13 +342,13 @@ void expert_tensor_bytes(const acm_model_desc& d, bool mx, size_t* gu, size_t* d
 acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li, float* out, cudaStream_t s,
                         const uint32_t* res_dev = nullptr, acm_block_stats* stats_dev = nullptr, bool pdl_ok = false,
                         int32_t early_epoch = 0, const uint32_t* only = nullptr, int n_blocks = 0,
-                        bool anchors_first = false, int widest_block = 0) {
+                        bool anchors_first = false, int widest_block = 0, bool behind_table = false) {
   const acm_model_desc& d = c->desc;
   const int n_pad = (T + 15) / 16 * 16;
   CUtensorMap x_map;
   FfnMaps maps;
   if (!L.mx) {      // (the MXFP4 kernel has no tensor copies)
-    acm_status st = ensure_h_maps(c, n_pad);
+    acm_status st = !small_block(T, d.hidden, d.inter) ? ensure_h_maps(c, n_pad) : ACM_OK;      // (small blocks: no activations in global memory)
     if (st != ACM_OK) return st;
     st = encode_x(c, &x_map, x, T, n_pad);
     if (st != ACM_OK) return st;
@@ -348,9 +356,11 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
     if (L.has_pool) {
       maps.staged_gate_up = L.pool_map_gu;
       maps.staged_down = L.pool_map_dn;
+      maps.staged_down_slice = L.pool_map_ds;
     } else if (c->stage_gate_up) {
       maps.staged_gate_up = c->stage_map_gu;
       maps.staged_down = c->stage_map_dn;
+      maps.staged_down_slice = c->stage_map_ds;
     }
   }
   FfnLaunch p;
@@ -388,7 +398,9 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
     ACM_CUDA(cudaEventRecord(e0, s));
   }
   // dependent launch only straight after the select/route kernel (no event, memset or copy between)
-  p.pdl = pdl_ok && c->pdl && !e0;
+  // ... or, for the kernel whose CTAs do not wait on one another, after the kernel that made the weight table
+  const bool free_ctas = !L.mx && small_block(T, d.hidden, d.inter);
+  p.pdl = (pdl_ok || (behind_table && free_ctas)) && c->pdl && !e0;
   // the anchors' pre-segment pays only when this launch overlaps the selection; a launch ordered after it (one
   // bracketed by events) has the whole set at hand and takes the balanced plan
   if (anchors_first && p.pdl && early_epoch != 0) p.anc_flag = c->ws.anc_words;
@@ -472,6 +484,8 @@ acm_status ensure_staging(acm_ctx* c) {
   acm_status st = encode_gate_up(c, &c->stage_map_gu, c->stage_gate_up, d.n_experts);
   if (st != ACM_OK) return st;
   st = encode_down(c, &c->stage_map_dn, c->stage_down, d.n_experts);
+  if (st != ACM_OK) return st;
+  st = encode_down_slice(c, &c->stage_map_ds, c->stage_down, d.n_experts);
   if (st != ACM_OK) return st;
   return ACM_OK;
 }
@@ -694,16 +708,22 @@ acm_status acm_set_layer_weights(acm_ctx* c, int layer, const void* w_router, co
     if (st != ACM_OK) return st;
     st = encode_down(c, &L.maps.down, w_down, d.n_experts);
     if (st != ACM_OK) return st;
+    st = encode_down_slice(c, &L.maps.down_slice, w_down, d.n_experts);
+    if (st != ACM_OK) return st;
     L.maps.shared_gate_up = L.maps.gate_up;
     L.maps.shared_down = L.maps.down;
+    L.maps.shared_down_slice = L.maps.down_slice;
     if (d.n_shared) {
       st = encode_gate_up(c, &L.maps.shared_gate_up, shared_gate_up, d.n_shared);
       if (st != ACM_OK) return st;
       st = encode_down(c, &L.maps.shared_down, shared_down, d.n_shared);
       if (st != ACM_OK) return st;
+      st = encode_down_slice(c, &L.maps.shared_down_slice, shared_down, d.n_shared);
+      if (st != ACM_OK) return st;
     }
     L.maps.staged_gate_up = L.maps.gate_up;
     L.maps.staged_down = L.maps.down;
+    L.maps.staged_down_slice = L.maps.down_slice;
   }
   L.set = true;
   c->layers[layer] = L;
@@ -836,7 +856,7 @@ acm_status acm_expert_ffn(acm_ctx* c, int layer, const void* x, int T, const int
     xq_expect(c, split_x_ctas(T, d.hidden));
     c->launches += 1;
   }
-  return run_ffn_list(c, L, x, T, 0, out, s);
+  return run_ffn_list(c, L, x, T, 0, out, s, nullptr, nullptr, false, 0, nullptr, 0, false, 0, true);
 }
 
 acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const float* alpha,
@@ -1273,13 +1293,17 @@ acm_status acm_set_slot_pool(acm_ctx* c, int layer, int n_slots, void* pool_gate
     if (st != ACM_OK) return st;
     st = encode_down(c, &L.pool_map_dn, pool_down, n_slots);
     if (st != ACM_OK) return st;
+    st = encode_down_slice(c, &L.pool_map_ds, pool_down, n_slots);
+    if (st != ACM_OK) return st;
   }
   if (!L.gate_up && !L.mx) {          // no full device tensors: every descriptor the kernel is handed must still be valid
     L.maps.gate_up = L.pool_map_gu;
     L.maps.down = L.pool_map_dn;
+    L.maps.down_slice = L.pool_map_ds;
     if (d.n_shared == 0) {
       L.maps.shared_gate_up = L.pool_map_gu;
       L.maps.shared_down = L.pool_map_dn;
+      L.maps.shared_down_slice = L.pool_map_ds;
     }
   }
   const int E = d.n_experts;

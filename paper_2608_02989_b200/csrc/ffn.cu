@@ -25,6 +25,8 @@
 // per expert orders them (a CTA waits for the experts its share of the K range reads).  Every wait is
 // bounded; on expiry the kernel raises a status and drains.
 //
+// Small blocks (bf16, up to 32 node columns): k_ffn_bf16_small below, whose CTAs keep their activation tiles.
+//
 // f32 path: plain FMA kernels (the fp32 toy configuration is a few MFLOP).
 #include <cuda_bf16.h>
 
@@ -116,7 +118,7 @@ enum WaitSite : int {
   kSiteExpertReady = 9,     // helper: finished-tile counters of the experts a down stage reads
   kSiteStageArmed = 10,     // helper: the weight producer has not armed the stage
   kSiteOutStaged = 11,      // publisher: an outgoing fragment from the epilogue
-  kSiteActStaged = 12,      // publisher: a finished activation tile from the epilogue
+  kSiteActStaged = 12,      // publisher (small blocks: MMA issuer): a finished activation tile from the epilogue
   kSiteAccFull = 13,        // epilogue: an accumulator's MMAs
   kSiteOutFree = 14,        // epilogue: the outgoing-fragment buffer
   kSiteFragFull = 15,       // epilogue: the summed fragments of a cut tile
@@ -259,6 +261,11 @@ __device__ __forceinline__ int ld_acquire(const int32_t* p) {
 __device__ __forceinline__ void red_release_add(int32_t* p, int v) {
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
+// *p += v unless w is zero: one predicated reduction, no branch
+__device__ __forceinline__ void red_add_if(float* p, float w, float v) {
+  asm volatile("{\n\t.reg .pred q;\n\tsetp.neu.f32 q, %1, 0f00000000;\n\t@q red.relaxed.gpu.global.add.f32 [%0], %2;\n\t}\n"
+               ::"l"(p), "f"(w), "f"(v) : "memory");
+}
 // Bounded wait until *p >= target (p written by other CTAs with release semantics).
 __device__ bool flag_wait_ge(const int32_t* p, int target, GiveUp* g, int site) {
   if (g->flag) return false;
@@ -316,6 +323,15 @@ __device__ __forceinline__ bool epi_vote_all(bool pred) {
   return r != 0;
 }
 
+// The same over the 128 threads of one of several epilogue teams (named barriers 1, 2).
+__device__ __forceinline__ bool team_vote_all(int team, bool pred) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+      "bar.red.and.pred q, %2, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}\n"
+      : "=r"(r) : "r"(static_cast<uint32_t>(pred)), "r"(1 + team) : "memory");
+  return r != 0;
+}
 __device__ __forceinline__ uint64_t policy_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
@@ -399,7 +415,26 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
+}
+// (the value is there behind tmem_ld_wait)
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, float& v) {
+  uint32_t r;
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
+  v = __uint_as_float(r);
+}
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// ... naming the registers, so that no use of them can move ahead of it
+__device__ __forceinline__ void tmem_ld_wait8(float (&v)[8]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])::"memory");
+}
 
 // Shared-memory matrix descriptor: K-major operand, rows of 128 bytes, 128-byte swizzle, groups of
 // 8 rows 1024 bytes apart.  The tile base is 1024-byte aligned; stepping K by 16 elements adds 32 bytes.
@@ -1566,6 +1601,532 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 }
 
 #if !ACM_FFN_MX
+// ---------------------------------------------------------------------------------- bf16, up to 32 node columns
+// The kernel above sends every activation tile through L2 to whichever CTAs take the down projection's work on that expert:
+// finalise, store, announce, poll, load, about 4 us of a launch in which a small block streams for 11 us.  With few nodes
+// that trip can be left out.  A unit of work here is a gate/up tile (64 features) AND its part of the down projection,
+//   out[:, all H] += w * h[:, these 64 features] W_down[:, these 64 features]^T,
+// by the same CTA: the activation tile goes from the epilogue into shared memory and from there into the MMAs, and no CTA
+// waits for another one.  What that costs is reductions into the output: H per unit and routed node instead of about one
+// output tile a CTA (an expert's combine weight is applied to them, and a node that has none takes no part).  An SM issues a
+// warp's reduction in 5 clocks at best and all of them together reach 5 to 6 TB/s: 2.7 us a unit of 16 nodes, 10.8 of 64,
+// beside 9 to 17 us of its weights (64 nodes of 2048 x 768, 8 / 20 / 80 experts: 44 / 53 / 123 us a layer against 31 / 44 /
+// 122 with the kernel above; small_block has the line).
+//   roles    warp 0 weights and hidden states, warp 1 MMAs, warps 2-9 epilogue (two teams of four: of a gate/up tile each takes
+//            half the columns, of the down phase every other node), warp 10 the list behind the anchors
+//   stages   gate/up: 128 rows x 128 K and the matching hidden states; down: 256 output rows x 64 features (the activations
+//            are there already).  Five of them, where the kernel above has three.
+//   tiles    number i of the list (anchors first, as above) to CTA i mod grid, whole.  HBM serves the CTAs in proportion to
+//            what they have in flight, so one that has less to do than others keeps fewer stages in flight and all end
+//            together: with 21 experts on 2048 x 768 40.4 us instead of 44.2, with 40 experts 63.8 instead of 66.0.
+// What bounds it: HBM, 5.8 to 6.7 TB/s from the roles' start to the last copy.  us a layer, the kernel above -> this one, with
+// 8 / 12 / 20 / 40 experts: 2048 x 768, 1 node 28.0 / 35.8 / 42.1 / 67.3 -> 21.9 / 29.1 / 38.4 / 65.5, 16 nodes 29.2 / 35.9 /
+// 42.7 / 68.1 -> 24.9 / 31.4 / 39.1 / 66.0; 1024 x 512, 1 node 23.7 / 27.6 / 29.7 / 38.2 -> 16.8 / 21.2 / 24.4 / 33.1;
+// 4096 x 1536, 1 node 64.7 / 80.2 / 124 / 234 -> 59.9 / 77.8 / 123 / 229, 16 nodes 66.4 / 81.2 / 124 / 238 -> 68.1 / 82.5 / 125 / 233.
+constexpr int kEpiTeams = 2;                                       // of four epilogue warps
+constexpr int kSmallThreads = 96 + 128 * kEpiTeams;
+constexpr int kHeadStart = 16;                                     // stages of an anchor tile that are through when the rest of the list comes
+template <int kN>
+struct SmallGeo {
+  static constexpr int kRing = 5;
+  static constexpr int kStageBytes = kABytes + kAtoms * kN * kBK * 2;
+  static constexpr int kSlotCols = 128;                            // columns of an accumulator slot, of kAcc
+  static constexpr int kSlotTiles = kSlotCols / kN;                // output tiles of the down phase in a slot
+  static constexpr int kExBytes = kN * 64 * 4;                     // gate/up exchange
+  static constexpr int kHBytes = kN * 64 * 2;                      // an activation tile: [node][64 features] bf16, swizzled
+};
+template <int kN>
+struct __align__(8) SmallBars {
+  unsigned long long full[SmallGeo<kN>::kRing], empty[SmallGeo<kN>::kRing];
+  unsigned long long tfull[kAcc], tempty[kAcc];
+  unsigned long long h_full[2], h_free[2];     // epilogue -> MMAs: an activation tile is in place / MMAs -> epilogue: it has been read
+  unsigned long long drained, plan_ready;
+  volatile int32_t n_slots, n_routed_slots;    // length of the work list, routed experts in it (as far as it is known)
+  uint32_t tmem_base;
+  GiveUp give_up;
+  float wd[kEpiTeams][2][kN];                  // combine weights of this and the next unit's expert
+  float2 list[4 * kEpiTeams][kN];              // per epilogue warp: (weight, node) of the nodes that have one
+  int32_t entry[kMaxSlots];                    // the work list, as above
+  int16_t expert[kMaxSlots];
+  uint32_t words[4 * kMaskWords];              // the mask the launch starts on, in 16-bit pieces (second half: blocks 4..7 of a batch)
+};
+template <int kN>
+constexpr size_t small_smem_bytes() {
+  return 1024 + static_cast<size_t>(SmallGeo<kN>::kRing) * SmallGeo<kN>::kStageBytes + 2 * SmallGeo<kN>::kHBytes + SmallGeo<kN>::kExBytes +
+         sizeof(SmallBars<kN>);
+}
+static_assert(small_smem_bytes<16>() <= 232448 && small_smem_bytes<32>() <= 232448, "shared memory");
+
+template <int kN>
+__global__ void __launch_bounds__(kSmallThreads, 1)
+k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUtensorMap x_map, const FfnArgs p) {
+  using Geom = SmallGeo<kN>;
+  constexpr int kRing = Geom::kRing, kStageBytes = Geom::kStageBytes, kSlotCols = Geom::kSlotCols, kSlotTiles = Geom::kSlotTiles;
+  extern __shared__ unsigned char smem_dyn[];
+  unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+  unsigned char* hstage = smem + kRing * kStageBytes;
+  float* ex = reinterpret_cast<float*>(hstage + 2 * Geom::kHBytes);
+  SmallBars<kN>* bars = reinterpret_cast<SmallBars<kN>*>(hstage + 2 * Geom::kHBytes + Geom::kExBytes);
+  GiveUp* const quit = &bars->give_up;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cta = blockIdx.x, G = gridDim.x;
+  griddep_launch_dependents();
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRing; ++s) {
+      mbar_init(smem_u32(&bars->full[s]), 1);
+      mbar_init(smem_u32(&bars->empty[s]), 1);
+    }
+    for (int b = 0; b < kAcc; ++b) {
+      mbar_init(smem_u32(&bars->tfull[b]), 1);
+      mbar_init(smem_u32(&bars->tempty[b]), 128 * kEpiTeams);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&bars->h_full[b]), 128 * kEpiTeams);
+      mbar_init(smem_u32(&bars->h_free[b]), 1);
+    }
+    mbar_init(smem_u32(&bars->drained), 1);
+    mbar_init(smem_u32(&bars->plan_ready), 1);
+    bars->give_up.flag = 0;
+    bars->give_up.limit_ns = p.wait_limit_ns;
+    bars->give_up.status = p.status;
+    bars->give_up.where = p.wait_diag ? p.wait_diag + blockIdx.x : nullptr;
+    bars->give_up.tag = p.launch_tag;
+    if (p.wait_diag) p.wait_diag[blockIdx.x] = p.launch_tag;      // "this CTA of that launch has started"
+    fence_barrier_init();
+  }
+  if (warp == 0 && lane == 0) {
+    prefetch_tensormap(&maps.gate_up);
+    prefetch_tensormap(&maps.down_slice);
+    prefetch_tensormap(&x_map);
+  }
+  if (warp == 1) {
+    tmem_alloc(smem_u32(&bars->tmem_base), 512);
+    tmem_relinquish();
+  }
+  // (Starts as above: on the anchors' words, on the eligible set's, or behind the kernels before.)
+  const bool early = p.sel_flag != nullptr;
+  const bool pre = p.anc_flag != nullptr && early;
+  if (early) {
+    bool timed_out = false;
+    if (threadIdx.x >= 64 && threadIdx.x < 128) {
+      const int j = threadIdx.x - 64;
+      const uint32_t* words = pre ? p.anc_flag : p.sel_flag;
+      bool seen = true;
+      uint32_t bits = 0u;
+      if (j < 2 * kMaskWords * p.sel_blocks)
+        bits = poll_tagged_word(words + j, static_cast<uint32_t>(p.sel_epoch) & 0xffffu, p.wait_limit_ns, seen);
+      timed_out = !seen;
+      bits |= __shfl_xor_sync(0xffffffffu, bits, 8);
+      bits |= __shfl_xor_sync(0xffffffffu, bits, 16);
+      if (lane < 2 * kMaskWords) bars->words[(j >> 5) * 2 * kMaskWords + lane] = bits;
+    }
+    __syncthreads();
+    if (timed_out) give_up(quit, pre ? kSiteAnchorWords : kSiteEligibleWords);
+  } else {
+    griddep_wait();
+  }
+  uint32_t am[kMaskWords];
+  int n_first = 0;          // routed experts of the list known so far (anchor start: the anchors)
+#pragma unroll
+  for (int wd = 0; wd < kMaskWords; ++wd) {
+    uint32_t act;
+    if (early)
+      act = (bars->words[2 * wd] | bars->words[2 * kMaskWords + 2 * wd]) |
+            ((bars->words[2 * wd + 1] | bars->words[2 * kMaskWords + 2 * wd + 1]) << 16);
+    else
+      act = p.act_mask[wd];
+    const uint32_t res = p.resident ? p.resident[wd] : 0xffffffffu;
+    am[wd] = (p.li == 0 ? act & res : act & ~res) & p.only[wd];
+    n_first += __popc(am[wd]);
+  }
+  const int tpe = p.I / 64, kc1 = p.H / (kBK * kAtoms), h_tiles = p.H / kTileM, n_down = (h_tiles + 1) / 2;
+  const uint32_t b_atom_bytes = static_cast<uint32_t>(p.n_pad) * kBK * 2;
+  int32_t* s_entry = bars->entry;
+  // slots of the experts in m behind slot `base`, in ascending id
+  auto list_experts = [&](const uint32_t (&m)[kMaskWords], int base, int e) {
+    const int wd = e >> 5;
+    const uint32_t mine = wd == 0 ? m[0] : wd == 1 ? m[1] : wd == 2 ? m[2] : m[3];
+    if ((mine >> (e & 31)) & 1u) {
+      int local = __popc(mine & ((1u << (e & 31)) - 1u));
+#pragma unroll
+      for (int v = 0; v < kMaskWords; ++v) local += v < wd ? __popc(m[v]) : 0;
+      s_entry[base + local] = p.slot_of ? make_entry(kSrcStaged, p.slot_of[e])
+                                        : p.li == 0 ? make_entry(kSrcRouted, e) : make_entry(kSrcStaged, local);
+      bars->expert[base + local] = e;
+    }
+  };
+  auto list_shared = [&](int base, int i) {
+    s_entry[base + i] = make_entry(kSrcShared, i);
+    bars->expert[base + i] = -1;
+  };
+  if (threadIdx.x < kMaxExperts) {
+    list_experts(am, 0, threadIdx.x);
+  } else if (p.li == 0 && !pre && static_cast<int>(threadIdx.x) - kMaxExperts < p.n_shared) {
+    list_shared(n_first, threadIdx.x - kMaxExperts);
+  }
+  if (threadIdx.x == 0) {
+    bars->n_slots = n_first + ((p.li == 0 && !pre) ? p.n_shared : 0);
+    bars->n_routed_slots = n_first;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = bars->tmem_base;
+  if (threadIdx.x == 0) ACM_STAMP(0);
+  const int n_first_tiles = pre ? n_first * tpe : bars->n_slots * tpe;
+  // Is there a tile `tile`?  With the anchor start the list behind the anchors comes later.
+  int limit = n_first_tiles;
+  bool more = pre;
+  auto have = [&](int tile) -> bool {
+    if (tile < limit) return true;
+    if (!more) return false;
+    more = false;
+    if (!mbar_wait(smem_u32(&bars->plan_ready), 0u, quit, kSitePlanReady)) return false;
+    limit = bars->n_slots * tpe;
+    return tile < limit;
+  };
+  // The CTAs walk a tile's K-chunks and output rows from different ones on: in step, all would fetch the same hidden states and
+  // add into the same rows at the same time.
+  const int k_first = cta % kc1, j_first = cta % n_down;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------ weights and hidden states
+    if (lane == 0) {
+      const uint64_t pol_w = policy_evict_first(), pol_x = policy_evict_last();
+      uint32_t s = 0, par = 0;
+      bool ok = true;
+      // Stages in flight, as soon as the list is known: in proportion to the stages that this CTA has left, against the one with
+      // the most (of the CTAs with an anchor tile, or of the others).
+      const int tile_stages = kc1 + n_down;
+      auto ring_depth = [&]() -> int {
+        auto left = [&](int c) {
+          const int n = c < limit ? tile_stages * (static_cast<int>(fdiv(static_cast<unsigned>(limit - 1 - c), p.d_grid)) + 1) : 0;
+          return pre && c < n_first_tiles ? n - min(tile_stages - 1, kHeadStart) : n;
+        };
+        const int most = max(left(0), left(min(n_first_tiles, G - 1)));
+        const int d = (2 * kRing * left(cta) + most - 1) / (2 * most);
+        return min(max(d, 2), kRing);
+      };
+      int depth = kRing;
+      bool depth_open = true;
+      if (!pre && cta < limit) depth = ring_depth();
+      for (int tile = cta; ok && have(tile); tile += G) {
+        const int a = static_cast<int>(fdiv(static_cast<unsigned>(tile), p.d_tpe)), ti = tile - a * tpe;
+        const int32_t ent = s_entry[a];
+        const int eidx = entry_idx(ent);
+        const CUtensorMap* gu = pick_map(entry_src(ent), &maps.gate_up, &maps.shared_gate_up, &maps.staged_gate_up);
+        const CUtensorMap* dn = pick_map(entry_src(ent), &maps.down_slice, &maps.shared_down_slice, &maps.staged_down_slice);
+        int kk = k_first;
+        if (pre && depth_open && !more) {
+          depth_open = false;
+          depth = ring_depth();
+        }
+        // (the stage `depth` back has been read: at full depth that is the one whose place this stage takes)
+        auto wait_room = [&]() -> bool {
+          if (more && mbar_try_wait(smem_u32(&bars->plan_ready), 0u)) {
+            more = depth_open = false;
+            limit = bars->n_slots * tpe;
+            depth = ring_depth();
+          }
+          const int back = static_cast<int>(s) - depth;
+          const uint32_t at = back < 0 ? back + kRing : back, at_par = back < 0 ? par ^ 1u : par;
+          return mbar_wait(smem_u32(&bars->empty[at]), at_par, quit, kSiteStageEmpty);
+        };
+        for (int kc = 0; kc < kc1; ++kc) {
+          if (!(ok = wait_room())) break;
+          const uint32_t full = smem_u32(&bars->full[s]);
+          const uint32_t sa = smem_u32(smem) + s * kStageBytes;
+          mbar_expect_tx(full, kABytes + kAtoms * b_atom_bytes);
+          tma_load_5d(sa, gu, full, 0, ti * 64, 0, kk * kAtoms, eidx, pol_w);
+          tma_load_3d(sa + kABytes, &x_map, full, 0, 0, kk * kAtoms, pol_x);
+          if (++kk == kc1) kk = 0;
+          if (++s == kRing) { s = 0; par ^= 1u; }
+        }
+        int jj = j_first;
+        for (int j = 0; ok && j < n_down; ++j) {
+          if (!(ok = wait_room())) break;
+          const uint32_t full = smem_u32(&bars->full[s]);
+          mbar_expect_tx(full, kABytes);
+          tma_load_4d(smem_u32(smem) + s * kStageBytes, dn, full, 0, jj * 2 * kTileM, ti, eidx, pol_w);
+          if (++jj == n_down) jj = 0;
+          if (++s == kRing) { s = 0; par ^= 1u; }
+        }
+      }
+      if (p.stats && p.li == 0 && blockIdx.x == 0) {
+        griddep_wait();
+        int n_all = 0, n_stg = 0;
+#pragma unroll
+        for (int wd = 0; wd < kMaskWords; ++wd) {
+          const uint32_t act = __ldcg(p.act_mask + wd);
+          n_all += __popc(act);
+          n_stg += p.resident ? __popc(act & ~p.resident[wd]) : 0;
+        }
+        p.stats->n_activated = n_all;
+        p.stats->n_staged = n_stg;
+        p.stats->n_streamed = bars->n_routed_slots;
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------ MMA issuer (see above)
+    const uint32_t tm = __shfl_sync(0xffffffffu, tmem_base, 0);
+    const uint32_t idesc = umma_idesc(p.n_pad);
+    const uint64_t desc_hi = umma_smem_desc(0);
+    const uint32_t stage0 = (smem_u32(smem) & 0x3ffffu) >> 4, h0 = (smem_u32(hstage) & 0x3ffffu) >> 4;
+    uint32_t s = 0, par = 0, b = 0, bpar = 1, hb = 0, hpar = 0;
+    bool ok = true;
+    auto vote = [&](bool v) { return __all_sync(0xffffffffu, v); };
+    for (int tile = cta; ok && vote(have(tile)); tile += G) {
+      if (!(ok = vote(mbar_wait(smem_u32(&bars->tempty[b]), bpar, quit, kSiteAccEmpty)))) break;
+      tc_fence_after();
+      for (int kc = 0; kc < kc1; ++kc) {
+        if (!(ok = vote(mbar_wait(smem_u32(&bars->full[s]), par, quit, kSiteStageFull)))) break;
+        tc_fence_after();
+        const uint64_t da0 = desc_hi | (stage0 + s * (kStageBytes >> 4));
+        const uint64_t db0 = da0 + (kABytes >> 4);
+        if (elect_one()) {
+#pragma unroll
+          for (int at = 0; at < kAtoms; ++at) {
+#pragma unroll
+            for (int kk = 0; kk < kBK / 16; ++kk)
+              umma_bf16(tm + b * kSlotCols, da0 + (at * (kAtomABytes >> 4) + 2 * kk), db0 + (at * (b_atom_bytes >> 4) + 2 * kk), idesc,
+                        (kc > 0 || at > 0 || kk > 0) ? 1u : 0u);
+          }
+          umma_commit(smem_u32(&bars->empty[s]));
+          if (kc + 1 == kc1) umma_commit(smem_u32(&bars->tfull[b]));
+        }
+        __syncwarp();
+        if (++s == kRing) { s = 0; par ^= 1u; }
+      }
+      if (!ok) break;
+      if (++b == kAcc) { b = 0; bpar ^= 1u; }
+      if (!(ok = vote(mbar_wait(smem_u32(&bars->h_full[hb]), hpar, quit, kSiteActStaged)))) break;
+      tc_fence_after();
+      const uint64_t dh0 = desc_hi | (h0 + hb * (Geom::kHBytes >> 4));
+      for (int j = 0; j < n_down; ++j) {
+        const int first = (2 * j) % kSlotTiles;      // place of the stage's first output tile in its slot
+        if (first == 0) {
+          if (!(ok = vote(mbar_wait(smem_u32(&bars->tempty[b]), bpar, quit, kSiteAccEmpty)))) break;
+          tc_fence_after();
+        }
+        if (!(ok = vote(mbar_wait(smem_u32(&bars->full[s]), par, quit, kSiteStageFull)))) break;
+        tc_fence_after();
+        const uint64_t da0 = desc_hi | (stage0 + s * (kStageBytes >> 4));
+        const bool last = j + 1 == n_down;
+        const bool slot_done = first + 2 == kSlotTiles || last;
+        // (rows beyond the tensor, in the last stage of an odd number of tiles, arrive as zeros)
+        if (elect_one()) {
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+#pragma unroll
+            for (int kk = 0; kk < kBK / 16; ++kk)
+              umma_bf16(tm + b * kSlotCols + (first + half) * kN, da0 + (half * (kAtomABytes >> 4) + 2 * kk), dh0 + 2 * kk, idesc, kk > 0 ? 1u : 0u);
+          }
+          umma_commit(smem_u32(&bars->empty[s]));
+          if (last) umma_commit(smem_u32(&bars->h_free[hb]));
+          if (slot_done) umma_commit(smem_u32(&bars->tfull[b]));
+        }
+        __syncwarp();
+        if (++s == kRing) { s = 0; par ^= 1u; }
+        if (slot_done && ++b == kAcc) { b = 0; bpar ^= 1u; }
+      }
+      if (++hb == 2) { hb = 0; hpar ^= 1u; }
+    }
+  } else if (warp == 2 + 4 * kEpiTeams) {
+    // ------------------------------------------------------------------ the list behind the anchors
+    if (pre) {
+      bool seen = true;
+      uint32_t half = 0u;
+      const uint32_t tag = static_cast<uint32_t>(p.sel_epoch) & 0xffffu;
+      const int n_words = 2 * kMaskWords * p.sel_blocks;
+#pragma unroll
+      for (int part = 0; part < 2; ++part) {
+        const int j = lane + 32 * part;
+        if (j < n_words) {
+          bool got = true;
+          half |= poll_tagged_word(p.sel_flag + j, tag, p.wait_limit_ns, got);
+          seen = seen && got;
+        }
+      }
+      half |= __shfl_xor_sync(0xffffffffu, half, 8);
+      half |= __shfl_xor_sync(0xffffffffu, half, 16);
+      const bool good = __all_sync(0xffffffffu, seen);
+      uint32_t rest[kMaskWords];
+      int n_rest = 0;
+#pragma unroll
+      for (int wd = 0; wd < kMaskWords; ++wd) {
+        const uint32_t lo = __shfl_sync(0xffffffffu, half, 2 * wd), hi = __shfl_sync(0xffffffffu, half, 2 * wd + 1);
+        rest[wd] = ((lo | (hi << 16)) & p.only[wd]) & ~am[wd];
+        n_rest += __popc(rest[wd]);
+      }
+      if (good) {
+        for (int e = lane; e < kMaxExperts; e += 32) list_experts(rest, n_first, e);
+        if (lane < p.n_shared) list_shared(n_first + n_rest, lane);
+        __syncwarp();
+        if (lane == 0) {
+          bars->n_routed_slots = n_first + n_rest;
+          bars->n_slots = n_first + n_rest + p.n_shared;
+        }
+      } else if (lane == 0) {
+        give_up(quit, kSiteEligibleWords);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&bars->plan_ready));
+    }
+  } else {
+    // ------------------------------------------------------------------ epilogue
+    const int team = (warp - 2) >> 2, quarter = warp & 3, row = quarter * 32 + lane, feat = row & 63;
+    const uint32_t lane_addr = static_cast<uint32_t>(quarter * 32) << 16;
+    uint32_t b = 0, bpar = 0, n_tile = 0;
+    bool ok = true, waited = !early;
+    auto acc_wait = [&]() -> bool { return team_vote_all(team, mbar_wait(smem_u32(&bars->tfull[b]), bpar, quit, kSiteAccFull)); };
+    auto acc_next = [&]() {
+      tc_fence_before();
+      mbar_arrive(smem_u32(&bars->tempty[b]));
+      if (++b == kAcc) { b = 0; bpar ^= 1u; }
+    };
+    for (int tile = cta; ok && have(tile); tile += G, ++n_tile) {
+      const int a = static_cast<int>(fdiv(static_cast<unsigned>(tile), p.d_tpe));
+      const uint32_t hb = n_tile & 1u;
+      const int ex_id = bars->expert[a];
+      auto load_weight = [&]() -> float {
+        return row >= p.T ? 0.0f : ex_id >= 0 ? __ldcg(p.wtab + static_cast<size_t>(ex_id) * kWtabStride + row) : 1.0f;
+      };
+      float wd_mine = 0.0f;
+      const bool ready = waited;
+      if (ready) wd_mine = load_weight();
+      if (!(ok = acc_wait())) break;
+      tc_fence_after();
+      {
+        // a team's share of the columns; the gate thread finishes the first half of them, the up thread the other
+        constexpr int kCols = kN / kEpiTeams, kHalf = kCols / 2;
+        const int c_team = team * kCols;
+        float v[kCols];
+#pragma unroll
+        for (int c = 0; c < kCols; c += 8) tmem_ld8(tmem_base + lane_addr + b * kSlotCols + c_team + c, v + c);
+        tmem_ld_wait();
+        acc_next();
+        if (quarter >= 2) {
+#pragma unroll
+          for (int c = 0; c < kHalf; ++c) ex[(c_team + c) * 64 + feat] = v[c];
+        } else {
+#pragma unroll
+          for (int c = kHalf; c < kCols; ++c) ex[(c_team + c) * 64 + feat] = v[c];
+        }
+        bool h_ok = true;
+        if (n_tile >= 2) h_ok = mbar_wait(smem_u32(&bars->h_free[hb]), ((n_tile >> 1) - 1) & 1u, quit, kSiteActFree);
+        if (!(ok = team_vote_all(team, h_ok))) break;
+        unsigned char* hs = hstage + hb * Geom::kHBytes;
+        const int c0 = c_team + (quarter < 2 ? 0 : kHalf);
+#pragma unroll
+        for (int j = 0; j < kHalf; ++j) {
+          if (c0 + j < p.T) {
+            const float other = ex[(c0 + j) * 64 + feat];
+            const float mine = quarter < 2 ? v[j] : v[kHalf + j];
+            const float g = quarter < 2 ? mine : other, u = quarter < 2 ? other : mine;
+            // u * silu(g), silu(g) = g/2 * (1 + tanh(g/2))
+            const float hg = 0.5f * g;
+            float th;
+            asm("tanh.approx.f32 %0, %1;" : "=f"(th) : "f"(hg));
+            const float q = u * hg;
+            const int t = c0 + j;
+            *reinterpret_cast<__nv_bfloat16*>(hs + t * 128 + (((feat >> 3) ^ (t & 7)) << 4) + ((feat & 7) << 1)) =
+                __float2bfloat16_rn(fmaf(q, th, q));
+          }
+        }
+        fence_proxy_async_smem();
+        mbar_arrive(smem_u32(&bars->h_full[hb]));
+      }
+      if (row == 0 && team == 0) ACM_STAMP(10);
+      // The routing kernel's weights, which only the sums need, and the cleared output.
+      if (!ready) {
+        griddep_wait();
+        waited = true;
+        wd_mine = load_weight();
+      }
+      if (row < kN) bars->wd[team][hb][row] = wd_mine;
+      // Every warp lists the nodes that the expert has a weight for and takes their columns alone out of the accumulators:
+      // eight values at a time, kNodes nodes of all of a slot's tiles; the teams take turns.  (The list is filled up with
+      // weights of zero.)
+      constexpr int kNodes = 8 / kSlotTiles;
+      float2* list = bars->list[warp - 2];
+      int n_list = 0, jj = j_first;
+      for (int j0 = 0; j0 < n_down; j0 += kSlotTiles / 2) {
+        if (!(ok = acc_wait())) break;
+        tc_fence_after();
+        if (j0 == 0) {
+#pragma unroll
+          for (int c = 0; c < kN; c += 32) {
+            const float w = c + lane < kN ? bars->wd[team][hb][c + lane] : 0.0f;
+            const unsigned has = __ballot_sync(0xffffffffu, w != 0.0f);
+            if (w != 0.0f) list[n_list + __popc(has & ((1u << lane) - 1u))] = make_float2(w, __int_as_float(c + lane));
+            n_list += __popc(has);
+          }
+          if (kNodes > 1 && lane < (-n_list & (kNodes - 1))) list[n_list + lane] = make_float2(0.0f, 0.0f);
+          __syncwarp();
+        }
+        float* dst[kSlotTiles / 2];
+        bool whole = j0 + kSlotTiles / 2 <= n_down;
+        int last_at = 2 * n_down;      // (at an odd number of tiles the last stage holds one)
+#pragma unroll
+        for (int st = 0; st < kSlotTiles / 2; ++st) {
+          dst[st] = p.out + jj * 2 * kTileM + row;
+          if (j0 + st < n_down) {
+            if (2 * jj + 1 >= h_tiles) { whole = false; last_at = st; }
+            if (++jj == n_down) jj = 0;
+          }
+        }
+        const uint32_t at = tmem_base + lane_addr + b * kSlotCols;
+        float v[8], nv[8];
+        float2 en[kNodes], ne[kNodes];
+        auto fetch = [&](int q, float2 (&e)[kNodes], float (&x)[8]) {
+#pragma unroll
+          for (int m = 0; m < kNodes; ++m) {
+            e[m] = list[q + m];
+#pragma unroll
+            for (int i = 0; i < kSlotTiles; ++i) tmem_ld1(at + i * kN + __float_as_int(e[m].y), x[m * kSlotTiles + i]);
+          }
+        };
+        if (team * kNodes < n_list) fetch(team * kNodes, ne, nv);
+#pragma unroll 1
+        for (int q = team * kNodes; q < n_list; q += kEpiTeams * kNodes) {
+          tmem_ld_wait8(nv);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) v[i] = nv[i];
+#pragma unroll
+          for (int m = 0; m < kNodes; ++m) en[m] = ne[m];
+          if (q + kEpiTeams * kNodes < n_list) fetch(q + kEpiTeams * kNodes, ne, nv);
+#pragma unroll
+          for (int m = 0; m < kNodes; ++m) {
+            const size_t to = static_cast<size_t>(__float_as_int(en[m].y)) * p.H;
+            if (kNodes == 1 || en[m].x != 0.0f) {
+              if (whole) {
+#pragma unroll
+                for (int i = 0; i < kSlotTiles; ++i) atomicAdd(dst[i / 2] + to + (i & 1) * kTileM, en[m].x * v[m * kSlotTiles + i]);
+              } else {
+#pragma unroll
+                for (int i = 0; i < kSlotTiles; ++i)
+                  if (j0 + i / 2 < n_down && !(i / 2 == last_at && (i & 1))) atomicAdd(dst[i / 2] + to + (i & 1) * kTileM, en[m].x * v[m * kSlotTiles + i]);
+              }
+            }
+          }
+        }
+        acc_next();
+      }
+      if (row == 0 && team == 0) ACM_STAMP(11);
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    if (__any_sync(0xffffffffu, quit->flag)) drain_cta(smem_u32(&bars->drained));
+    tc_fence_after();
+    tmem_dealloc(tmem_base, 512);
+  }
+}
+#endif
+
+#if !ACM_FFN_MX
 // ---------------------------------------------------------------------------------- f32 path
 // A few MFLOP in L2: what counts is the chain of latencies, so both kernels are dependent launches in the fused call (the
 // second one's CTAs are resident before the first is done), a warp has the loads of four rows in flight, and rows are
@@ -1706,10 +2267,20 @@ cudaError_t ffn_mx_configure() {
 cudaError_t launch_ffn_mxfp4(const FfnLaunch& L, cudaStream_t s) {
 #else
 
+namespace {
+const void* small_kernel(int n_pad) {
+  return n_pad <= 16 ? reinterpret_cast<const void*>(k_ffn_bf16_small<16>) : reinterpret_cast<const void*>(k_ffn_bf16_small<32>);
+}
+size_t small_smem(int n_pad) { return n_pad <= 16 ? small_smem_bytes<16>() : small_smem_bytes<32>(); }
+}  // namespace
 cudaError_t ffn_configure() {
   cudaError_t err = cudaFuncSetAttribute(ACM_FFN_KERNEL<kMaxNodes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(Geo<kMaxNodes>::kSmemBytes));
   if (err != cudaSuccess) return err;
+  for (int n : {16, kSmallNodes}) {
+    err = cudaFuncSetAttribute(small_kernel(n), cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(small_smem(n)));
+    if (err != cudaSuccess) return err;
+  }
   return cudaFuncSetAttribute(ACM_FFN_KERNEL<kWideNodes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(Geo<kWideNodes>::kSmemBytes));
 }
@@ -1768,6 +2339,14 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
   if (L.n_pad > kWideNodes) return cudaErrorInvalidValue;
 #endif
   cfg.dynamicSmemBytes = wide ? Geo<kWideNodes>::kSmemBytes : Geo<kMaxNodes>::kSmemBytes;
+#if !ACM_FFN_MX
+  const bool small = small_block(L.T, L.H, L.I);
+  void* small_args[] = {const_cast<FfnMaps*>(&maps), const_cast<CUtensorMap*>(&x_map), &a};
+  if (small) {
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = small_smem(L.n_pad);
+  }
+#endif
   cfg.stream = s;
   // The CTAs wait on one another, so all of them must be resident: one CTA per SM on an otherwise
   // idle GPU is, and a cooperative launch makes the driver check it.  A dependent launch cannot be
@@ -1785,6 +2364,7 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
 #if ACM_FFN_MX
   return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(ACM_FFN_KERNEL<kMaxNodes>), args);
 #else
+  if (small) return cudaLaunchKernelExC(&cfg, small_kernel(L.n_pad), small_args);
   return cudaLaunchKernelExC(&cfg, wide ? reinterpret_cast<const void*>(ACM_FFN_KERNEL<kWideNodes>)
                                         : reinterpret_cast<const void*>(ACM_FFN_KERNEL<kMaxNodes>), args);
 #endif

@@ -221,6 +221,37 @@ def test_expert_ffn_against_oracle(T, H, I, E, k, ns):
     ctx.close()
 
 
+@pytest.mark.parametrize("T,H,I,E,k,ns", [(1, 128, 64, 3, 1, 0), (15, 384, 128, 30, 3, 1), (16, 1152, 320, 9, 4, 2), (17, 640, 192, 40, 8, 0),
+                                          (31, 1408, 576, 20, 6, 1), (32, 4096, 64, 128, 8, 0), (8, 4096, 704, 24, 6, 0)])
+def test_small_blocks_keep_their_activations_on_chip(T, H, I, E, k, ns):
+    """Blocks of up to 32 nodes: both node paddings at their edges, odd numbers of output tiles (H / 128) and of accumulator
+    slots, fewer and more units of work than CTAs, shared experts; routes given by the caller and the fused call."""
+    cfg = wl.scaled(wl.CONFIGS[3], hidden=H, inter=I, n_experts=E, top_k=k, n_shared=ns, n_nodes=T, max_depth=4, zipf_bias=False)
+    w, x = wl.layer_weights(cfg, 5, DEV), wl.hidden_states(cfg, 5, DEV)
+    rng = np.random.default_rng(T)
+    idx = np.array([rng.permutation(E)[:k] for _ in range(T)], dtype=np.int32)
+    wt = rng.uniform(0.05, 1.0, (T, k)).astype(np.float32)
+    if T > 1:
+        idx[T // 2, -1], wt[T - 1, 0] = -1, 0.0        # an empty slot, a route of no weight
+    ctx = _ctx(cfg)
+    _set_weights(ctx, w)
+    guard = torch.full((T + 1, H), 7.0, device=DEV)    # a row behind the output stays as it is
+    ref = oracle.expert_ffn(x, idx, wt.astype(np.float64), w["gate_up"], w["down"], w["shared_gate_up"], w["shared_down"])
+    for _ in range(2):
+        ctx.expert_ffn(0, x, torch.tensor(idx, device=DEV), torch.tensor(wt, device=DEV), out=guard[:T])
+        _ffn_check(guard[:T], ref, f"small {T}x{H}x{I}")
+        assert bool((guard[T] == 7.0).all())
+    alpha = acm.node_weights(wl.tree_depths(cfg), wl.commitment_table(cfg))
+    out, got_idx, got_w, mask, stats = ctx.moe_verify(0, x, alpha.to(DEV), acm.SelectParams(), want=True, out=guard[:T])
+    assert ctx.device_status() == acm.OK and set(ctx.wait_report()) == {0}
+    ref = oracle.moe_verify(x, w["w_router"], w["router_bias"], w["gate_up"], w["down"], alpha.numpy(), k, oracle.SelectParams(),
+                            weighting=cfg.weighting, shared_gate_up=w["shared_gate_up"], shared_down=w["shared_down"])
+    np.testing.assert_array_equal(got_idx.cpu().numpy(), ref["idx"])
+    _ffn_check(out, ref["out"], "small fused call")
+    assert bool((guard[T] == 7.0).all()) and acm.stats_dict(stats)["n_streamed"] == ref["count"]
+    ctx.close()
+
+
 def test_expert_ffn_fp32_toy():
     cfg = wl.CONFIGS[1]
     w = wl.layer_weights(cfg, 0, DEV)
