@@ -167,8 +167,16 @@ cudaError_t launch_route(const RouteArgs& a, int T, int E, int k, bool pdl, cuda
 // null) holds 8 tagged words per block for the eligible set.
 int select_ctas_per_block(int widest);
 cudaError_t select_configure();   // the kernel's function attributes, once per device (when a context is created)
+// `logits` (small fp32 layers, select_makes_logits): the kernel works the logits out itself.
+struct LogitArgs {
+  const float *x, *w_router, *bias;
+  int H;
+  int32_t* status;
+};
+bool select_makes_logits(int H, int E);
 cudaError_t launch_softmax_select_route(const SelectArgs& sa, const RouteArgs& ra, const BatchDesc& bd,
-                                        const uint32_t* mask_override, int E, int k, bool pdl, cudaStream_t s);
+                                        const uint32_t* mask_override, int E, int k, bool pdl, cudaStream_t s,
+                                        const LogitArgs* logits = nullptr);
 // routes given by the caller -> activated mask, weight table, cleared `ready` and cleared output
 cudaError_t launch_routes_to_table(const int32_t* idx, const float* w, uint32_t* act_mask, float* wtab, int32_t* ready, int T,
                                    int E, int k, float* out, size_t out_floats, bool pdl, cudaStream_t s);

@@ -914,11 +914,17 @@ acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const flo
   root.anc_tag = static_cast<uint32_t>(early_epoch) & 0xffffu;
   root.wait_limit_ns = c->wait_limit_ns;
   const XqArgs xa = xq_args(c, T);
-  ACM_CUDA(launch_router_logits(d.dtype, x, L.w_router, L.bias, c->ws.logits, T, d.hidden, E, f32 ? nullptr : out,
-                                f32 ? 0 : static_cast<size_t>(T) * d.hidden, c->ws.wtab, c->ffn_in_floats,
-                                c->ws.status, nullptr, nullptr, nullptr, k, nullptr, c->pdl, s,
-                                c->trace ? reinterpret_cast<long long*>(c->trace) + 32 * c->sm_count : nullptr,
-                                early ? &root : nullptr, L.mx ? &xa : nullptr));
+  // (small fp32 layers: the next kernel makes the logits too)
+  const bool own_logits = f32 && select_makes_logits(d.hidden, E);
+  const LogitArgs la = {static_cast<const float*>(x), static_cast<const float*>(L.w_router), L.bias, d.hidden, c->ws.status};
+  if (!own_logits) {
+    ACM_CUDA(launch_router_logits(d.dtype, x, L.w_router, L.bias, c->ws.logits, T, d.hidden, E, f32 ? nullptr : out,
+                                  f32 ? 0 : static_cast<size_t>(T) * d.hidden, c->ws.wtab, c->ffn_in_floats,
+                                  c->ws.status, nullptr, nullptr, nullptr, k, nullptr, c->pdl, s,
+                                  c->trace ? reinterpret_cast<long long*>(c->trace) + 32 * c->sm_count : nullptr,
+                                  early ? &root : nullptr, L.mx ? &xa : nullptr));
+    c->launches += 1;
+  }
   if (L.mx) xq_expect(c, xa.rows * split_x_row_ctas(E));
   // stages 1b-3: one cluster of CTAs, which also fills the FFN kernel's routing inputs
   SelectArgs sa;
@@ -931,7 +937,10 @@ acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const flo
   RouteArgs ra = {};
   ra.logits = c->ws.logits; ra.mask = c->ws.mask; ra.idx_out = c->ws.idx; ra.w_out = c->ws.w;
   ra.weighting = d.weighting; ra.routed_scale = d.routed_scale;
-  ra.act_mask = c->ws.act_mask; ra.wtab = c->ws.wtab; ra.resident = res_dev;
+  if (!f32) {      // (the fp32 FFN kernels read the routes)
+    ra.act_mask = c->ws.act_mask; ra.wtab = c->ws.wtab;
+  }
+  ra.resident = res_dev;
   ra.host_stage_list = L.has_resident ? c->host_stage_list_dev : nullptr;
   if (early) {
     ra.sel_flag = c->ws.sel_words;
@@ -942,8 +951,8 @@ acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const flo
   one.n_blocks = 1;
   one.off[0] = 0;
   one.off[1] = T;
-  ACM_CUDA(launch_softmax_select_route(sa, ra, one, eligible_mask_override, E, k, c->pdl, s));
-  c->launches += 2;
+  ACM_CUDA(launch_softmax_select_route(sa, ra, one, eligible_mask_override, E, k, c->pdl, s, own_logits ? &la : nullptr));
+  c->launches += 1;
 
   if (f32) {
     ACM_CUDA(launch_ffn_f32(static_cast<const float*>(x), static_cast<const float*>(L.gate_up),

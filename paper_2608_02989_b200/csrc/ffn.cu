@@ -261,11 +261,6 @@ __device__ __forceinline__ int ld_acquire(const int32_t* p) {
 __device__ __forceinline__ void red_release_add(int32_t* p, int v) {
   asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-// *p += v unless w is zero: one predicated reduction, no branch
-__device__ __forceinline__ void red_add_if(float* p, float w, float v) {
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.neu.f32 q, %1, 0f00000000;\n\t@q red.relaxed.gpu.global.add.f32 [%0], %2;\n\t}\n"
-               ::"l"(p), "f"(w), "f"(v) : "memory");
-}
 // Bounded wait until *p >= target (p written by other CTAs with release semantics).
 __device__ bool flag_wait_ge(const int32_t* p, int target, GiveUp* g, int site) {
   if (g->flag) return false;

@@ -1109,6 +1109,34 @@ def test_mxfp4_small_features_beside_large_ones(p):
     ctx.close()
 
 
+@pytest.mark.parametrize("T,H,I,E,k,bias", [(1, 32, 4, 5, 1, True), (17, 96, 66, 31, 5, False), (40, 512, 36, 8, 8, True),
+                                            (64, 128, 64, 32, 8, True), (9, 544, 36, 7, 2, True), (33, 64, 20, 33, 3, False)])
+def test_f32_fused_call_with_its_logits_in_the_selection_kernel(T, H, I, E, k, bias):
+    """fp32 layers: logits made by the selection kernel up to 512 x 8 / 128 x 32 and by the router kernel beyond; sets and routes bit
+    for bit, natural routing, calls back to back, and logits that are not finite."""
+    cfg = wl.scaled(wl.CONFIGS[1], hidden=H, inter=I, n_experts=E, top_k=k, n_nodes=T, level_widths=None, max_depth=4, zipf_bias=bias)
+    w, x, alpha = _block(cfg)
+    ctx = _ctx(cfg)
+    _set_weights(ctx, w)
+    n0 = ctx.launch_count()
+    for natural in (False, True, False):
+        kw = dict(mask_override=torch.tensor(full_mask(E).view(np.int32), device=DEV)) if natural else {}
+        ref = oracle.moe_verify(x, w["w_router"], w["router_bias"], w["gate_up"], w["down"], alpha.numpy(), k, weighting=cfg.weighting,
+                                mask_override=full_mask(E) if natural else None)
+        out, idx, _, mask, stats = ctx.moe_verify(0, x, alpha.to(DEV), None if natural else acm.SelectParams(), want=True, **kw)
+        assert ctx.device_status() == acm.OK
+        np.testing.assert_array_equal(idx.cpu().numpy(), ref["idx"])
+        np.testing.assert_array_equal(_u32(mask), ref["mask"])
+        assert acm.stats_dict(stats)["n_activated"] == len(np.unique(ref["idx"][ref["idx"] >= 0]))
+        assert _ffn_check(out, ref["out"], "fp32 fused") < 1e-4
+    assert ctx.launch_count() - n0 == 3 * (3 if H <= 512 and E <= 32 else 4)
+    bad = x.clone()
+    bad[0, 0] = float("nan")
+    ctx.moe_verify(0, bad, alpha.to(DEV), acm.SelectParams())
+    assert ctx.device_status() == acm.ERR_NONFINITE
+    ctx.close()
+
+
 @pytest.mark.parametrize("T,H,I,E,k,ns", [(1, 32, 4, 5, 1, 0), (9, 96, 66, 13, 3, 1), (40, 160, 132, 40, 8, 2), (64, 256, 3, 16, 2, 0)])
 def test_f32_ffn_rows_and_loads(T, H, I, E, k, ns):
     """The fp32 FFN kernels take four weight rows a warp (remainders of 1 to 3 rows here) and 16-byte loads where shapes and
