@@ -1282,9 +1282,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #pragma unroll
       for (int g = 0; g < 4; ++g) sa[g] = *reinterpret_cast<const uint32_t*>(R + kMxCodeBytes + (lane + 32 * g) * 4);
     };
-    auto release_raw = [&]() {        // (once the loads above have arrived)
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->raw_empty[ri]));
+    auto next_raw = [&]() {
       ri += 2u;
       if (ri >= static_cast<uint32_t>(p.n_raw)) { ri -= static_cast<uint32_t>(p.n_raw); rpar ^= 1u; }
     };
@@ -1295,7 +1293,9 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       if (!fetched) {
         if (!(ok = wait_raw())) break;
         load_raw();
-        release_raw();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&bars->raw_empty[ri]));
+        next_raw();
       }
       uint32_t o[32], so[4];
 #pragma unroll
@@ -1316,11 +1316,14 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       const uint32_t sf = tmem_base + my_lane + kAcc * kAccCols + kMxA * kMxACols + s * kMxScaleCols;
       tmem_st4(sf, so[0], so[1], so[2], so[3]);
       fetched = it + 2 < total;
-      if (fetched) {
-        if (!(ok = wait_raw())) break;
-        load_raw();
+      {      // the next record and this stage's activations: polled side by side, one vote
+        const uint32_t raw_bar = smem_u32(&bars->raw[ri]), act_bar = smem_u32(&bars->act[s]);
+        bool raw_there = !fetched || mbar_try_wait(raw_bar, rpar), act_there = mbar_try_wait(act_bar, par);
+        if (!raw_there) raw_there = mbar_wait_slow(raw_bar, rpar, quit, kSitePackedStage);
+        if (!act_there) act_there = mbar_wait_slow(act_bar, par, quit, kSiteActStage);
+        if (!(ok = __all_sync(0xffffffffu, raw_there && act_there))) break;
       }
-      if (!(ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars->act[s]), par, quit, kSiteActStage)))) break;
+      if (fetched) load_raw();
       const uint2* S = reinterpret_cast<const uint2*>(act_scale_base + s * 2 * kMxActScaleBytes) + lane;
       const uint2 lo = S[0], hi = S[kMxActScaleBytes / 8];      // two half-stages, two bytes of a word each
       const uint32_t s0 = __byte_perm(lo.x, hi.x, 0x5410), s1 = __byte_perm(lo.y, hi.y, 0x5410);
@@ -1329,11 +1332,14 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
         tmem_st2(sf + 4 + 4 * pc, s0 - pc * (kMxPieceShift * 0x01010101u), s1 - pc * (kMxPieceShift * 0x01010101u));
       tmem_st_wait();
       tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bars->full[s]));
+      __syncwarp();                     // (the loads above have arrived, too)
+      if (lane == 0) {
+        mbar_arrive(smem_u32(&bars->full[s]));
+        if (fetched) mbar_arrive(smem_u32(&bars->raw_empty[ri]));
+      }
+      if (fetched) next_raw();
       s += 2u;
       if (s >= kRing) { s -= kRing; par ^= 1u; }
-      if (fetched) release_raw();
      }
     }
     if (!ok) tmem_st_wait();      // (left between a stage's stores and its wait: tensor memory is released behind this)
