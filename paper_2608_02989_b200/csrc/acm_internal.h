@@ -186,7 +186,11 @@ struct FfnMaps {               // TMA descriptors of one layer (bf16 path)
   CUtensorMap gate_up, down;               // routed experts  [E,2I,H] / [E,H,I]
   CUtensorMap shared_gate_up, shared_down; // shared experts (copies of the above if none)
   CUtensorMap staged_gate_up, staged_down; // staging slots   (copies of the above if none)
-  CUtensorMap down_slice, shared_down_slice, staged_down_slice;   // the down tensors in boxes of 256 rows x 64 features (small blocks)
+};
+// The down tensors in boxes of 256 rows x 64 features: what a launch of k_ffn_bf16_small has in the place of `down` and its kin.
+// (Maps of their own beside those would go into every launch's parameters: 0.3 to 0.5 % of the other kernels' layers.)
+struct DownSlices {
+  CUtensorMap routed, shared, staged;
 };
 struct FfnLaunch {
   int T, H, I, n_pad;

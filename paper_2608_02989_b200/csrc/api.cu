@@ -23,6 +23,7 @@ struct Layer {
   const void* shared_gate_up = nullptr;
   const void* shared_down = nullptr;
   FfnMaps maps;
+  DownSlices slices;
   bool set = false;
   bool mx = false;                      // MXFP4 layer (acm_set_layer_weights_mxfp4): expert tensors are tiled codes + scales
   const void* mx_gate_up = nullptr;     // [E][I/64][H/128][8704] (null when the experts only live in a pool)
@@ -356,11 +357,14 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
     if (L.has_pool) {
       maps.staged_gate_up = L.pool_map_gu;
       maps.staged_down = L.pool_map_dn;
-      maps.staged_down_slice = L.pool_map_ds;
     } else if (c->stage_gate_up) {
       maps.staged_gate_up = c->stage_map_gu;
       maps.staged_down = c->stage_map_dn;
-      maps.staged_down_slice = c->stage_map_ds;
+    }
+    if (small_block(T, d.hidden, d.inter)) {
+      maps.down = L.slices.routed;
+      maps.shared_down = L.slices.shared;
+      maps.staged_down = L.has_pool ? L.pool_map_ds : c->stage_gate_up ? c->stage_map_ds : L.slices.staged;
     }
   }
   FfnLaunch p;
@@ -708,22 +712,22 @@ acm_status acm_set_layer_weights(acm_ctx* c, int layer, const void* w_router, co
     if (st != ACM_OK) return st;
     st = encode_down(c, &L.maps.down, w_down, d.n_experts);
     if (st != ACM_OK) return st;
-    st = encode_down_slice(c, &L.maps.down_slice, w_down, d.n_experts);
+    st = encode_down_slice(c, &L.slices.routed, w_down, d.n_experts);
     if (st != ACM_OK) return st;
     L.maps.shared_gate_up = L.maps.gate_up;
     L.maps.shared_down = L.maps.down;
-    L.maps.shared_down_slice = L.maps.down_slice;
+    L.slices.shared = L.slices.routed;
     if (d.n_shared) {
       st = encode_gate_up(c, &L.maps.shared_gate_up, shared_gate_up, d.n_shared);
       if (st != ACM_OK) return st;
       st = encode_down(c, &L.maps.shared_down, shared_down, d.n_shared);
       if (st != ACM_OK) return st;
-      st = encode_down_slice(c, &L.maps.shared_down_slice, shared_down, d.n_shared);
+      st = encode_down_slice(c, &L.slices.shared, shared_down, d.n_shared);
       if (st != ACM_OK) return st;
     }
     L.maps.staged_gate_up = L.maps.gate_up;
     L.maps.staged_down = L.maps.down;
-    L.maps.staged_down_slice = L.maps.down_slice;
+    L.slices.staged = L.slices.routed;
   }
   L.set = true;
   c->layers[layer] = L;
@@ -1308,11 +1312,11 @@ acm_status acm_set_slot_pool(acm_ctx* c, int layer, int n_slots, void* pool_gate
   if (!L.gate_up && !L.mx) {          // no full device tensors: every descriptor the kernel is handed must still be valid
     L.maps.gate_up = L.pool_map_gu;
     L.maps.down = L.pool_map_dn;
-    L.maps.down_slice = L.pool_map_ds;
+    L.slices.routed = L.pool_map_ds;
     if (d.n_shared == 0) {
       L.maps.shared_gate_up = L.pool_map_gu;
       L.maps.shared_down = L.pool_map_dn;
-      L.maps.shared_down_slice = L.pool_map_ds;
+      L.slices.shared = L.pool_map_ds;
     }
   }
   const int E = d.n_experts;

@@ -71,8 +71,10 @@ constexpr int kHStageBytes = kHPieceBytes + (ACM_FFN_MX ? kMxActScaleBytes : 0);
 //   node columns of their own, one MMA for both, are exact down to 2^-13 only.  Weights that are zero wherever a feature is
 //   2^14 times the others then leave a result with three times the error; at 2^20 times it is 31 % off.)
 //   The features are stored in the order the moves leave the weights in (mx_act.cuh).
-// What bounds it: up to 32 node columns 0.39 us a stage, 0.30 of them the unpacking groups' chain (waits, shared-memory loads,
-// moves, tensor-memory stores), where HBM would deliver one every 0.20 us; at 64 columns 0.45 us, what an SM takes in (34 KB).
+// What bounds it: at 64 node columns the MMAs (a launch of 103 us takes 90 with a third of them) and what an SM takes in, 34 KB a
+// stage of 0.45 us.  Up to 32 columns a stage takes 0.35 us where HBM would deliver one every 0.20, and no part of it by itself
+// is the reason: with a third of the MMAs, an eighth of the tensor-memory stores, no activations or 512 bytes a record copied, or
+// three unpacking groups, a launch of 85.7 us takes 82 to 86.
 // A layer of 2048 x 768, 64 nodes, 22 experts: 42.5 us; 49.0 with the weights expanded to bf16 by four warps (0.56 us a
 // stage) for eight kind::f16 MMAs.
 constexpr int kThreads = ACM_FFN_MX ? 512 : 256;         // producer, MMA, 4 epilogue warps, helper, publisher (+ 2 x 4 unpacking warps)
@@ -1697,7 +1699,7 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
   }
   if (warp == 0 && lane == 0) {
     prefetch_tensormap(&maps.gate_up);
-    prefetch_tensormap(&maps.down_slice);
+    prefetch_tensormap(&maps.down);
     prefetch_tensormap(&x_map);
   }
   if (warp == 1) {
@@ -1816,7 +1818,7 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
         const int32_t ent = s_entry[a];
         const int eidx = entry_idx(ent);
         const CUtensorMap* gu = pick_map(entry_src(ent), &maps.gate_up, &maps.shared_gate_up, &maps.staged_gate_up);
-        const CUtensorMap* dn = pick_map(entry_src(ent), &maps.down_slice, &maps.shared_down_slice, &maps.staged_down_slice);
+        const CUtensorMap* dn = pick_map(entry_src(ent), &maps.down, &maps.shared_down, &maps.staged_down);      // (slices: DownSlices)
         int kk = k_first;
         if (pre && depth_open && !more) {
           depth_open = false;
