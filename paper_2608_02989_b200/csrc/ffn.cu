@@ -1618,7 +1618,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 //   roles    warp 0 weights and hidden states, warp 1 MMAs, warps 2-9 epilogue (two teams of four: of a gate/up tile each takes
 //            half the columns, of the down phase every other node), warp 10 the list behind the anchors
 //   stages   gate/up: 128 rows x 128 K and the matching hidden states; down: 256 output rows x 64 features (the activations
-//            are there already).  Five of them, where the kernel above has three.
+//            are there already).  Five of them, or three (small_kernel).
 //   tiles    number i of the list (anchors first, as above) to CTA i mod grid, whole.  HBM serves the CTAs in proportion to
 //            what they have in flight, so one that has less to do than others keeps fewer stages in flight and all end
 //            together: with 21 experts on 2048 x 768 40.4 us instead of 44.2, with 40 experts 63.8 instead of 66.0.
@@ -1629,18 +1629,18 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 constexpr int kEpiTeams = 2;                                       // of four epilogue warps
 constexpr int kSmallThreads = 96 + 128 * kEpiTeams;
 constexpr int kHeadStart = 16;                                     // stages of an anchor tile that are through when the rest of the list comes
-template <int kN>
+template <int kN, int kR>
 struct SmallGeo {
-  static constexpr int kRing = 5;
+  static constexpr int kRing = kR;
   static constexpr int kStageBytes = kABytes + kAtoms * kN * kBK * 2;
   static constexpr int kSlotCols = 128;                            // columns of an accumulator slot, of kAcc
   static constexpr int kSlotTiles = kSlotCols / kN;                // output tiles of the down phase in a slot
   static constexpr int kExBytes = kN * 64 * 4;                     // gate/up exchange
   static constexpr int kHBytes = kN * 64 * 2;                      // an activation tile: [node][64 features] bf16, swizzled
 };
-template <int kN>
+template <int kN, int kR>
 struct __align__(8) SmallBars {
-  unsigned long long full[SmallGeo<kN>::kRing], empty[SmallGeo<kN>::kRing];
+  unsigned long long full[SmallGeo<kN, kR>::kRing], empty[SmallGeo<kN, kR>::kRing];
   unsigned long long tfull[kAcc], tempty[kAcc];
   unsigned long long h_full[2], h_free[2];     // epilogue -> MMAs: an activation tile is in place / MMAs -> epilogue: it has been read
   unsigned long long drained, plan_ready;
@@ -1653,23 +1653,23 @@ struct __align__(8) SmallBars {
   int16_t expert[kMaxSlots];
   uint32_t words[4 * kMaskWords];              // the mask the launch starts on, in 16-bit pieces (second half: blocks 4..7 of a batch)
 };
-template <int kN>
+template <int kN, int kR>
 constexpr size_t small_smem_bytes() {
-  return 1024 + static_cast<size_t>(SmallGeo<kN>::kRing) * SmallGeo<kN>::kStageBytes + 2 * SmallGeo<kN>::kHBytes + SmallGeo<kN>::kExBytes +
-         sizeof(SmallBars<kN>);
+  return 1024 + static_cast<size_t>(SmallGeo<kN, kR>::kRing) * SmallGeo<kN, kR>::kStageBytes + 2 * SmallGeo<kN, kR>::kHBytes + SmallGeo<kN, kR>::kExBytes +
+         sizeof(SmallBars<kN, kR>);
 }
-static_assert(small_smem_bytes<16>() <= 232448 && small_smem_bytes<32>() <= 232448, "shared memory");
+static_assert(small_smem_bytes<16, 5>() <= 232448 && small_smem_bytes<32, 5>() <= 232448, "shared memory");
 
-template <int kN>
+template <int kN, int kR>
 __global__ void __launch_bounds__(kSmallThreads, 1)
 k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUtensorMap x_map, const FfnArgs p) {
-  using Geom = SmallGeo<kN>;
+  using Geom = SmallGeo<kN, kR>;
   constexpr int kRing = Geom::kRing, kStageBytes = Geom::kStageBytes, kSlotCols = Geom::kSlotCols, kSlotTiles = Geom::kSlotTiles;
   extern __shared__ unsigned char smem_dyn[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
   unsigned char* hstage = smem + kRing * kStageBytes;
   float* ex = reinterpret_cast<float*>(hstage + 2 * Geom::kHBytes);
-  SmallBars<kN>* bars = reinterpret_cast<SmallBars<kN>*>(hstage + 2 * Geom::kHBytes + Geom::kExBytes);
+  SmallBars<kN, kR>* bars = reinterpret_cast<SmallBars<kN, kR>*>(hstage + 2 * Geom::kHBytes + Geom::kExBytes);
   GiveUp* const quit = &bars->give_up;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int cta = blockIdx.x, G = gridDim.x;
@@ -2271,17 +2271,29 @@ cudaError_t launch_ffn_mxfp4(const FfnLaunch& L, cudaStream_t s) {
 #else
 
 namespace {
-const void* small_kernel(int n_pad) {
-  return n_pad <= 16 ? reinterpret_cast<const void*>(k_ffn_bf16_small<16>) : reinterpret_cast<const void*>(k_ffn_bf16_small<32>);
+// The small blocks' kernel for a launch.  Up to 1152 hidden features with three stages (120 KB): a CTA of the next call's router
+// kernel then fits beside it and has its weights by the time this launch is done, which such short launches gain more from than
+// from stages in flight.  us a layer, five stages -> three, with 8 / 21 / 40 experts: 1024 x 512, 1 node 17.0 / 24.4 / 33.7 -> 15.4 /
+// 22.8 / 31.6; 1024 x 1408, 16 nodes 29.2 / 40.1 / 63.3 -> 26.1 / 39.1 / 62.0; 1152 x 768, 1 node 18.4 / 30.0 / 44.3 -> 17.0 / 30.5 /
+// 43.5; 1536 x 768, 1 node 19.0 / 35.2 / 51.1 -> 19.0 / 35.9 / 51.7; 2048 x 768, 1 node 21.3 / 39.4 / 64.0 -> 22.3 / 41.8 / 66.4.
+// (Six stages: 22.1 / 40.6 / 67.4 there.  The router kernel's CTAs without their request for 104 KB, so that they fit beside five
+// stages: they pile up on the SMs that are free first, 22.7 / 42.3 / 66.7.)
+struct SmallKernel {
+  const void* fn;
+  size_t smem;
+};
+SmallKernel small_kernel(int n_pad, int hidden) {
+  if (n_pad > 16) return {reinterpret_cast<const void*>(k_ffn_bf16_small<kSmallNodes, 5>), small_smem_bytes<kSmallNodes, 5>()};
+  if (hidden <= 1152) return {reinterpret_cast<const void*>(k_ffn_bf16_small<16, 3>), small_smem_bytes<16, 3>()};
+  return {reinterpret_cast<const void*>(k_ffn_bf16_small<16, 5>), small_smem_bytes<16, 5>()};
 }
-size_t small_smem(int n_pad) { return n_pad <= 16 ? small_smem_bytes<16>() : small_smem_bytes<32>(); }
 }  // namespace
 cudaError_t ffn_configure() {
   cudaError_t err = cudaFuncSetAttribute(ACM_FFN_KERNEL<kMaxNodes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(Geo<kMaxNodes>::kSmemBytes));
   if (err != cudaSuccess) return err;
-  for (int n : {16, kSmallNodes}) {
-    err = cudaFuncSetAttribute(small_kernel(n), cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(small_smem(n)));
+  for (const SmallKernel& k : {small_kernel(16, 128), small_kernel(16, 2048), small_kernel(kSmallNodes, 128)}) {
+    err = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(k.smem));
     if (err != cudaSuccess) return err;
   }
   return cudaFuncSetAttribute(ACM_FFN_KERNEL<kWideNodes>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -2347,7 +2359,7 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
   void* small_args[] = {const_cast<FfnMaps*>(&maps), const_cast<CUtensorMap*>(&x_map), &a};
   if (small) {
     cfg.blockDim = dim3(kSmallThreads);
-    cfg.dynamicSmemBytes = small_smem(L.n_pad);
+    cfg.dynamicSmemBytes = small_kernel(L.n_pad, L.H).smem;
   }
 #endif
   cfg.stream = s;
@@ -2367,7 +2379,7 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
 #if ACM_FFN_MX
   return cudaLaunchKernelExC(&cfg, reinterpret_cast<const void*>(ACM_FFN_KERNEL<kMaxNodes>), args);
 #else
-  if (small) return cudaLaunchKernelExC(&cfg, small_kernel(L.n_pad), small_args);
+  if (small) return cudaLaunchKernelExC(&cfg, small_kernel(L.n_pad, L.H).fn, small_args);
   return cudaLaunchKernelExC(&cfg, wide ? reinterpret_cast<const void*>(ACM_FFN_KERNEL<kWideNodes>)
                                         : reinterpret_cast<const void*>(ACM_FFN_KERNEL<kMaxNodes>), args);
 #endif
