@@ -402,6 +402,9 @@ __device__ __noinline__ void drain_cta(uint32_t drained) {
   while (global_timer() - t0 < 200000ull) {}
   __syncwarp();
 }
+// Loads of this thread's lane from column taddr on.  The registers hold the values only behind tmem_arrived, which therefore names
+// them: arithmetic on a register keeps its place beside volatile statements only if they name it, so behind a wait that names none
+// it could be moved ahead of the wait.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
   uint32_t r[16];
   asm volatile(
@@ -410,27 +413,29 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);      // (a name for the same register)
 }
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v) {
-  uint32_t r[8];
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t* r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr) : "memory");
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
-// (the value is there behind tmem_ld_wait)
-__device__ __forceinline__ void tmem_ld1(uint32_t taddr, float& v) {
-  uint32_t r;
+__device__ __forceinline__ void tmem_ld1(uint32_t taddr, uint32_t& r) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
-  v = __uint_as_float(r);
 }
-__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// ... naming the registers, so that no use of them can move ahead of it
-__device__ __forceinline__ void tmem_ld_wait8(float (&v)[8]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7])::"memory");
+template <int kCount>
+__device__ __forceinline__ void tmem_arrived(float (&v)[kCount]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < kCount; ++i) asm volatile("" : "+f"(v[i]));
+}
+template <int kCount>
+__device__ __forceinline__ void tmem_arrived(uint32_t (&r)[kCount], float (&v)[kCount]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int i = 0; i < kCount; ++i) {
+    asm volatile("" : "+r"(r[i]));
+    v[i] = __uint_as_float(r[i]);
+  }
 }
 
 // Shared-memory matrix descriptor: K-major operand, rows of 128 bytes, 128-byte swizzle, groups of
@@ -1365,7 +1370,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
       const uint32_t at = tmem_base + lane_addr + b * kAccCols + c;
       tmem_ld16(at, v);
       if (c + 16 < np) tmem_ld16(at + 16, v + 16);
-      tmem_ld_wait();
+      tmem_arrived(v);
     };
     auto release_acc = [&](uint32_t b) {
       tc_fence_before();
@@ -1378,7 +1383,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 #pragma unroll
       for (int c = 0; c < kMaxNodes; c += 16)
         if (c < np) tmem_ld16(tmem_base + lane_addr + b * kAccCols + cb + c, v + c);
-      tmem_ld_wait();
+      tmem_arrived(v);
       if (release) {
         tc_fence_before();
         mbar_arrive(smem_u32(&bars->tempty[b]));
@@ -2003,10 +2008,11 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
         // a team's share of the columns; the gate thread finishes the first half of them, the up thread the other
         constexpr int kCols = kN / kEpiTeams, kHalf = kCols / 2;
         const int c_team = team * kCols;
+        uint32_t r[kCols];
         float v[kCols];
 #pragma unroll
-        for (int c = 0; c < kCols; c += 8) tmem_ld8(tmem_base + lane_addr + b * kSlotCols + c_team + c, v + c);
-        tmem_ld_wait();
+        for (int c = 0; c < kCols; c += 8) tmem_ld8(tmem_base + lane_addr + b * kSlotCols + c_team + c, r + c);
+        tmem_arrived(r, v);
         acc_next();
         if (quarter >= 2) {
 #pragma unroll
@@ -2079,9 +2085,10 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
           }
         }
         const uint32_t at = tmem_base + lane_addr + b * kSlotCols;
-        float v[8], nv[8];
+        uint32_t nv[8];
+        float v[8];
         float2 en[kNodes], ne[kNodes];
-        auto fetch = [&](int q, float2 (&e)[kNodes], float (&x)[8]) {
+        auto fetch = [&](int q, float2 (&e)[kNodes], uint32_t (&x)[8]) {
 #pragma unroll
           for (int m = 0; m < kNodes; ++m) {
             e[m] = list[q + m];
@@ -2092,9 +2099,7 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
         if (team * kNodes < n_list) fetch(team * kNodes, ne, nv);
 #pragma unroll 1
         for (int q = team * kNodes; q < n_list; q += kEpiTeams * kNodes) {
-          tmem_ld_wait8(nv);
-#pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] = nv[i];
+          tmem_arrived(nv, v);
 #pragma unroll
           for (int m = 0; m < kNodes; ++m) en[m] = ne[m];
           if (q + kEpiTeams * kNodes < n_list) fetch(q + kEpiTeams * kNodes, ne, nv);
