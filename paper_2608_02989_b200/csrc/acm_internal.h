@@ -173,7 +173,7 @@ struct LogitArgs {
   int H;
   int32_t* status;
 };
-bool select_makes_logits(int H, int E);
+bool select_makes_logits(int T, int H, int E);
 cudaError_t launch_softmax_select_route(const SelectArgs& sa, const RouteArgs& ra, const BatchDesc& bd,
                                         const uint32_t* mask_override, int E, int k, bool pdl, cudaStream_t s,
                                         const LogitArgs* logits = nullptr);

@@ -919,7 +919,7 @@ acm_status acm_moe_verify(acm_ctx* c, int layer, const void* x, int T, const flo
   root.wait_limit_ns = c->wait_limit_ns;
   const XqArgs xa = xq_args(c, T);
   // (small fp32 layers: the next kernel makes the logits too)
-  const bool own_logits = f32 && select_makes_logits(d.hidden, E);
+  const bool own_logits = f32 && select_makes_logits(T, d.hidden, E);
   const LogitArgs la = {static_cast<const float*>(x), static_cast<const float*>(L.w_router), L.bias, d.hidden, c->ws.status};
   if (!own_logits) {
     ACM_CUDA(launch_router_logits(d.dtype, x, L.w_router, L.bias, c->ws.logits, T, d.hidden, E, f32 ? nullptr : out,

@@ -888,9 +888,19 @@ struct FusedSmem {      // (kLogits: the router's rows behind it)
 };
 // kLogits: small fp32 layers.  Their logits are a few hundred instructions a row, so the row's warp works them out itself --
 // lane l takes partial sum l, the same sums in the same order as the router kernel's -- from the router's rows, which the CTA
-// has put into shared memory before it waits for the kernel ahead; the call goes without the router kernel.  us a call, with that
-// kernel -> without, 96 x 5 experts 13.0 -> 11.0, 256 x 16 (the toy layer) 18.8 -> 18.4, 384 x 40 25.4 -> 28.5: hence 4096 weights.
-constexpr int kLogitsMaxHidden = 512, kLogitsMaxExperts = 32, kLogitsMaxWeights = 4096;
+// has put into shared memory before it waits for the kernel ahead; the call goes without the router kernel.  A warp takes its
+// experts four at a time, one four after the other, where the router kernel has warps for all of them: so the number of experts
+// draws the line, and from 13 on the number of nodes, whose warps share an SM's issue slots.  Time of a call without the router
+// kernel against with it, over hidden 32 to 512 (up to 4096 weights; more were not measured), inter 64 and 320:
+//   experts      1, 4, 8 nodes       12 to 64 nodes
+//   up to 8      0.80 to 0.97        0.87 to 0.97
+//   9 to 12      0.88 to 1.00        0.93 to 0.99
+//   13 to 16     0.90 to 0.99        0.95 to 1.02
+//   18, 20       0.92 to 1.03        0.98 to 1.05
+//   24, 28       0.94 to 1.06        1.01 to 1.11
+// 32 experts: 0.99 to 1.18.  us a call of the toy layer (256 x 16, 8 nodes) 18.7 -> 17.8.
+constexpr int kLogitsMaxHidden = 512, kLogitsMaxExperts = 16, kLogitsMaxWeights = 4096;
+constexpr int kLogitsAnyNodesExperts = 12, kLogitsFewNodes = 8;
 static_assert(sizeof(FusedSmem) + kLogitsMaxWeights * sizeof(float) <= kFusedSmemRequest, "shared memory of the selection kernel");
 template <bool kLogits>
 __global__ void __launch_bounds__(32 * kFusedWarps)
@@ -1212,8 +1222,9 @@ cudaError_t select_configure() {
                               static_cast<int>(kFusedSmemRequest));
 }
 
-bool select_makes_logits(int H, int E) {
-  return H <= kLogitsMaxHidden && H % 32 == 0 && E <= kLogitsMaxExperts && E * H <= kLogitsMaxWeights;
+bool select_makes_logits(int T, int H, int E) {
+  return H <= kLogitsMaxHidden && H % 32 == 0 && E * H <= kLogitsMaxWeights &&
+         E <= (T <= kLogitsFewNodes ? kLogitsMaxExperts : kLogitsAnyNodesExperts);
 }
 
 int select_ctas_per_block(int widest) {
@@ -1223,10 +1234,10 @@ int select_ctas_per_block(int widest) {
 
 cudaError_t launch_softmax_select_route(const SelectArgs& sa, const RouteArgs& ra, const BatchDesc& bd,
                                         const uint32_t* mask_override, int E, int k, bool pdl, cudaStream_t s, const LogitArgs* logits) {
-  if (logits && !select_makes_logits(logits->H, E)) return cudaErrorInvalidValue;
   int widest = 1;
   for (int b = 0; b < bd.n_blocks; ++b) widest = bd.off[b + 1] - bd.off[b] > widest ? bd.off[b + 1] - bd.off[b] : widest;
   if (widest > kFusedMaxCtas * kFusedWarps) return cudaErrorInvalidValue;      // a warp per row
+  if (logits && !select_makes_logits(widest, logits->H, E)) return cudaErrorInvalidValue;
   const int C = select_ctas_per_block(widest);
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;

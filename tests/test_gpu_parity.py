@@ -1110,10 +1110,14 @@ def test_mxfp4_small_features_beside_large_ones(p):
 
 
 @pytest.mark.parametrize("T,H,I,E,k,bias", [(1, 32, 4, 5, 1, True), (17, 96, 66, 31, 5, False), (40, 512, 36, 8, 8, True),
-                                            (64, 128, 64, 32, 8, True), (9, 544, 36, 7, 2, True), (33, 64, 20, 33, 3, False)])
+                                            (64, 128, 64, 32, 8, True), (9, 544, 36, 7, 2, True), (33, 64, 20, 33, 3, False),
+                                            (64, 320, 20, 12, 3, True), (8, 256, 36, 16, 5, True), (9, 256, 36, 16, 5, True),
+                                            (9, 288, 20, 13, 2, False), (3, 224, 20, 17, 4, True), (8, 288, 36, 15, 4, False),
+                                            (5, 512, 36, 9, 2, True), (64, 384, 20, 12, 8, False)])
 def test_f32_fused_call_with_its_logits_in_the_selection_kernel(T, H, I, E, k, bias):
-    """fp32 layers: logits made by the selection kernel up to 512 x 8 / 128 x 32 and by the router kernel beyond; sets and routes bit
-    for bit, natural routing, calls back to back, and logits that are not finite."""
+    """fp32 layers: logits made by the selection kernel up to 4096 router weights of up to 12 experts, 16 with up to 8 nodes, and by
+    the router kernel beyond (either side of each limit); sets and routes bit for bit, natural routing, calls back to back, and
+    logits that are not finite."""
     cfg = wl.scaled(wl.CONFIGS[1], hidden=H, inter=I, n_experts=E, top_k=k, n_nodes=T, level_widths=None, max_depth=4, zipf_bias=bias)
     w, x, alpha = _block(cfg)
     ctx = _ctx(cfg)
@@ -1129,7 +1133,8 @@ def test_f32_fused_call_with_its_logits_in_the_selection_kernel(T, H, I, E, k, b
         np.testing.assert_array_equal(_u32(mask), ref["mask"])
         assert acm.stats_dict(stats)["n_activated"] == len(np.unique(ref["idx"][ref["idx"] >= 0]))
         assert _ffn_check(out, ref["out"], "fp32 fused") < 1e-4
-    assert ctx.launch_count() - n0 == 3 * (3 if H <= 512 and E <= 32 else 4)
+    own = H <= 512 and E * H <= 4096 and E <= (16 if T <= 8 else 12)
+    assert ctx.launch_count() - n0 == 3 * (3 if own else 4)
     bad = x.clone()
     bad[0, 0] = float("nan")
     ctx.moe_verify(0, bad, alpha.to(DEV), acm.SelectParams())
