@@ -364,7 +364,7 @@ acm_status acm_expert_ffn_f32_noalloc(const float* x, int T, int hidden, int int
  * n_experts_streamed experts of a bf16 layer (hidden, inter) on `grid` CTAs deals its weight tiles, for inspection
  * and for tests of the plan's coverage.  n_anchor_first > 0 lists the plan of a launch that starts on that many
  * anchor experts (Eq. 5) before the rest of the set is known (their tiles, one per CTA, are segment 0).
- * (Launches of few nodes -- up to 8, 16 or 32 by the expert's size -- have no such plan: tile i of the list goes to CTA
+ * (Launches of few nodes -- up to 2 to 32 by hidden, inter and whether there are shared experts -- have no such plan: tile i of the list goes to CTA
  * i mod grid, whole, together with its part of the down projection.)
  * pieces [capacity][8] (host) receives, in each
  * CTA's execution order: CTA, segment, phase (1 = gate/up: 64 gate + 64 up rows x hidden; 2 = down: 128 output

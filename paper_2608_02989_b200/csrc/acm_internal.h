@@ -12,19 +12,35 @@ namespace acm {
 constexpr int kMaxExperts = 128;   // E limit; also the padded length of expert-axis tree sums
 constexpr int kMaxTopK = 8;
 constexpr int kMaxNodes = 64;      // T limit of one verification block; the FFN kernel handles node columns 64 at a time
-// Launches that k_ffn_bf16_small takes, whose CTAs keep the activations they make.  It saves a few microseconds a launch and
-// pays with reductions into the output that grow with the nodes: up to 8 nodes they stay behind the weights, and the smaller an
-// expert, the more nodes the saving is worth.  us a layer, the kernel before -> this one, with 12 / 20 / 40 experts:
-//   30 nodes  1024 x 512 28.3 / 30.9 / 40.6 -> 24.7 / 26.2 / 33.6     1536 x 768 33.1 / 38.4 / 56.5 -> 30.9 / 36.0 / 54.4 (32 nodes)
-//             1664 x 1152 35.3 / 48.8 / 78.5 -> 41.0 / 50.2 / 79.3    2048 x 768 36.5 / 42.7 / 68.2 -> 34.1 / 43.0 / 65.3
-//   16 nodes  2048 x 768 35.9 / 42.7 / 68.1 -> 31.4 / 39.1 / 66.0     1664 x 1152 35.1 / 47.5 / 78.2 -> 34.6 / 45.9 / 76.3
-//             2048 x 1408 43.2 / 61.9 / 111 -> 43.8 / 63.2 / 112      4096 x 1536 81.2 / 124 / 238 -> 82.5 / 125 / 233
-//    8 nodes  2048 x 1408 43.2 / 62.0 / 111 -> 42.3 / 61.7 / 111      4096 x 1536 80.4 / 124 / 236 -> 79.8 / 124 / 232
+// Launches that k_ffn_bf16_small takes, whose CTAs keep the activations they make: up to how many nodes, by the layer's shape.  It
+// saves a few microseconds a launch.  It pays with reductions into the output, which grow with the nodes, and with whole units: an
+// expert has inter / 64 of them, and where their number is a little above a whole number of rounds over the CTAs, the few CTAs
+// that have one more hold up the launch by its stages (hidden / 85) and its sums, which k_ffn_bf16 cuts.  That costs most with many
+// nodes, with shared experts (whose units are the list's last and have every node) and with experts of many units.  Where an
+// output lies in L2 moves a launch of this kernel by another 2 to 3 %.
+// Time of a layer against k_ffn_bf16's, mean / highest over sets of 4 to 64 experts that so many nodes can make, by hidden and inter:
+//   1 node    inter 512 to 896: 0.72 to 0.87 / 0.88; 1024 to 1536: 0.74 to 0.95 / 1.06
+//   2 nodes   512 to 960: 0.77 to 0.92 / 0.98; 1024 to 1536: 0.79 to 0.97 / 1.03
+//   8 nodes   up to 768: 0.80 to 0.95 / 1.01; 832 to 960, hidden to 2048: 0.82 to 0.94 / 1.01, beyond: 0.93 to 0.97 / 1.04;
+//             1024 to 1536, hidden to 1536: 0.83 to 0.97 / 1.01, 1792 and 2048: 0.95 to 1.00 / 1.05, beyond: 0.95 to 1.00 / 1.06
+//   16 nodes  hidden to 1152: 0.78 to 0.93 / 1.00; hidden to 2048, up to 896: 0.85 to 0.95 / 1.00, 960 and more: 0.96 to 1.04 / 1.14;
+//             hidden beyond 2048, 512: 0.89 to 0.94 / 1.01, 768 and more: 0.95 to 1.02 / 1.06
+//   24 nodes  hidden 1024: 0.84 to 0.92 / 1.00; 1152 to 2048, up to 768: 0.87 to 0.93 / 0.99, 896: 0.95 / 1.01
+//   32 nodes  hidden 1024, up to 768: 0.85 to 0.89 / 0.98, 1024: 0.93 / 1.00 (768 x 1024: 0.92 / 1.04); 1152 to 1536, up to 768: 0.89
+//             to 0.96 / 1.01, 896: 0.98 / 1.09; 1792: 0.93 to 0.96 / 1.04
+//   with shared experts: 8 nodes as above, inter 832 to 1408 beyond hidden 1536 0.97 to 1.02 / 1.07; 16 nodes, hidden to 2048, up to
+//             768: 0.86 to 0.97 / 1.03, 896: 0.97 to 1.00 / 1.05, 1024 and more: 1.01 to 1.06 / 1.13; 32 nodes, hidden 1024: 0.88 to
+//             0.97 / 1.05, beyond: 0.95 to 1.07 / 1.21
 constexpr int kSmallNodes = 32;
-inline bool small_block(int T, int hidden, int inter) {
-  const long long expert = static_cast<long long>(hidden) * inter;
-  return T <= (expert <= 1280 * 1024 ? kSmallNodes : expert <= 2048 * 1152 ? 16 : 8);
+inline int small_block_nodes(int hidden, int inter, int n_shared) {
+  const bool shared = n_shared > 0;
+  if (hidden <= 1024 && inter <= 1024) return inter <= 768 ? kSmallNodes : 24;
+  if (!shared && hidden <= 2048 && inter <= 768 && hidden * inter <= 1280 * 1024) return hidden <= 1536 ? kSmallNodes : 24;
+  if (hidden <= 1152 || (hidden <= 2048 && inter <= (shared ? 768 : 896)) || (inter <= 512 && !shared)) return 16;
+  if (inter <= 768 || hidden <= 1536 || (hidden <= 2048 && inter <= 960)) return 8;
+  return 2;
 }
+inline bool small_block(int T, int hidden, int inter, int n_shared) { return T <= small_block_nodes(hidden, inter, n_shared); }
 constexpr int kWideNodes = 128;    // T limit of a batch of blocks = node columns of one wide FFN accumulator tile
 constexpr int kWtabStride = kWideNodes;   // row length of the combine-weight table [expert][node]
 constexpr int kMaxShared = 4;

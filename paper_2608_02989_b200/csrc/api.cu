@@ -349,7 +349,7 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
   CUtensorMap x_map;
   FfnMaps maps;
   if (!L.mx) {      // (the MXFP4 kernel has no tensor copies)
-    acm_status st = !small_block(T, d.hidden, d.inter) ? ensure_h_maps(c, n_pad) : ACM_OK;      // (small blocks: no activations in global memory)
+    acm_status st = !small_block(T, d.hidden, d.inter, d.n_shared) ? ensure_h_maps(c, n_pad) : ACM_OK;      // (small blocks: no activations in global memory)
     if (st != ACM_OK) return st;
     st = encode_x(c, &x_map, x, T, n_pad);
     if (st != ACM_OK) return st;
@@ -361,7 +361,7 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
       maps.staged_gate_up = c->stage_map_gu;
       maps.staged_down = c->stage_map_dn;
     }
-    if (small_block(T, d.hidden, d.inter)) {
+    if (small_block(T, d.hidden, d.inter, d.n_shared)) {
       maps.down = L.slices.routed;
       maps.shared_down = L.slices.shared;
       maps.staged_down = L.has_pool ? L.pool_map_ds : c->stage_gate_up ? c->stage_map_ds : L.slices.staged;
@@ -403,7 +403,7 @@ acm_status run_ffn_list(acm_ctx* c, const Layer& L, const void* x, int T, int li
   }
   // dependent launch only straight after the select/route kernel (no event, memset or copy between)
   // ... or, for the kernel whose CTAs do not wait on one another, after the kernel that made the weight table
-  const bool free_ctas = !L.mx && small_block(T, d.hidden, d.inter);
+  const bool free_ctas = !L.mx && small_block(T, d.hidden, d.inter, d.n_shared);
   p.pdl = (pdl_ok || (behind_table && free_ctas)) && c->pdl && !e0;
   // the anchors' pre-segment pays only when this launch overlaps the selection; a launch ordered after it (one
   // bracketed by events) has the whole set at hand and takes the balanced plan

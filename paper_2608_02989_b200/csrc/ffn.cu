@@ -1619,7 +1619,7 @@ ACM_FFN_KERNEL(const __grid_constant__ FfnMaps maps, const __grid_constant__ CUt
 // output tile a CTA (an expert's combine weight is applied to them, and a node that has none takes no part).  An SM issues a
 // warp's reduction in 5 clocks at best and all of them together reach 5 to 6 TB/s: 2.7 us a unit of 16 nodes, 10.8 of 64,
 // beside 9 to 17 us of its weights (64 nodes of 2048 x 768, 8 / 20 / 80 experts: 44 / 53 / 123 us a layer against 31 / 44 /
-// 122 with the kernel above; small_block has the line).
+// 122 with the kernel above; small_block_nodes has the line).
 //   roles    warp 0 weights and hidden states, warp 1 MMAs, warps 2-9 epilogue (two teams of four: of a gate/up tile each takes
 //            half the columns, of the down phase every other node), warp 10 the list behind the anchors
 //   stages   gate/up: 128 rows x 128 K and the matching hidden states; down: 256 output rows x 64 features (the activations
@@ -2360,7 +2360,7 @@ cudaError_t launch_ffn_bf16(const FfnLaunch& L, const FfnMaps& maps, const CUten
 #endif
   cfg.dynamicSmemBytes = wide ? Geo<kWideNodes>::kSmemBytes : Geo<kMaxNodes>::kSmemBytes;
 #if !ACM_FFN_MX
-  const bool small = small_block(L.T, L.H, L.I);
+  const bool small = small_block(L.T, L.H, L.I, L.n_shared);
   void* small_args[] = {const_cast<FfnMaps*>(&maps), const_cast<CUtensorMap*>(&x_map), &a};
   if (small) {
     cfg.blockDim = dim3(kSmallThreads);

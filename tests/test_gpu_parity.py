@@ -222,7 +222,9 @@ def test_expert_ffn_against_oracle(T, H, I, E, k, ns):
 
 
 @pytest.mark.parametrize("T,H,I,E,k,ns", [(1, 128, 64, 3, 1, 0), (15, 384, 128, 30, 3, 1), (16, 1152, 320, 9, 4, 2), (17, 640, 192, 40, 8, 0),
-                                          (31, 1408, 576, 20, 6, 1), (32, 4096, 64, 128, 8, 0), (8, 4096, 704, 24, 6, 0)])
+                                          (31, 1408, 576, 20, 6, 1), (32, 4096, 64, 128, 8, 0), (8, 4096, 704, 24, 6, 0),
+                                          (31, 1408, 576, 20, 6, 0), (32, 1024, 768, 10, 4, 2), (24, 1920, 640, 30, 5, 0),
+                                          (16, 1280, 896, 12, 3, 0), (2, 4096, 1024, 20, 8, 1)])
 def test_small_blocks_keep_their_activations_on_chip(T, H, I, E, k, ns):
     """Blocks of up to 32 nodes: both node paddings at their edges, odd numbers of output tiles (H / 128) and of accumulator
     slots, fewer and more units of work than CTAs, shared experts; routes given by the caller and the fused call."""
@@ -249,6 +251,44 @@ def test_small_blocks_keep_their_activations_on_chip(T, H, I, E, k, ns):
     np.testing.assert_array_equal(got_idx.cpu().numpy(), ref["idx"])
     _ffn_check(out, ref["out"], "small fused call")
     assert bool((guard[T] == 7.0).all()) and acm.stats_dict(stats)["n_streamed"] == ref["count"]
+    ctx.close()
+
+
+@pytest.mark.parametrize("T,H,I,ns", [(3, 2048, 1024, 0), (9, 2048, 1408, 2), (16, 4096, 1536, 0), (16, 2304, 832, 0), (17, 2048, 768, 0),
+                                      (25, 2048, 512, 0), (33, 1024, 256, 0)])
+def test_few_nodes_of_experts_beyond_the_small_kernels_line(T, H, I, ns):
+    """k_ffn_bf16 at 16, 32 and 48 node columns with few nodes, just beyond the line: routes given by the caller, the fused call at every
+    overlap level, the same nodes in a batch, and a budget that makes most eligible experts ones that no node chose."""
+    E, k = 20, 4
+    cfg = wl.scaled(wl.CONFIGS[3], hidden=H, inter=I, n_experts=E, top_k=k, n_shared=ns, n_nodes=T, max_depth=4, zipf_bias=False)
+    ctx = _ctx(cfg)
+    w, x, alpha = _block(cfg, 2)
+    _set_weights(ctx, w)
+    shared = (w["shared_gate_up"], w["shared_down"])
+    rng = np.random.default_rng(T)
+    idx = np.array([rng.permutation(E)[:k] for _ in range(T)], dtype=np.int32)
+    wt = rng.uniform(0.05, 1.0, (T, k)).astype(np.float32)
+    idx[T // 2, -1] = -1
+    ref = oracle.expert_ffn(x, idx, wt.astype(np.float64), w["gate_up"], w["down"], *shared)
+    for _ in range(2):
+        _ffn_check(ctx.expert_ffn(0, x, torch.tensor(idx, device=DEV), torch.tensor(wt, device=DEV)), ref, "given routes")
+    params = dict(fixed_budget=E - 1)
+    ref = oracle.moe_verify(x, w["w_router"], w["router_bias"], w["gate_up"], w["down"], alpha.numpy(), k, oracle.SelectParams(**params),
+                            weighting=cfg.weighting, shared_gate_up=shared[0], shared_down=shared[1])
+    for level in (acm.OVERLAP_ANCHORS, acm.OVERLAP_ELIGIBLE, acm.OVERLAP_DEPENDENT, acm.OVERLAP_NONE):
+        ctx.set_overlap(level)
+        out, got, _, _, stats = ctx.moe_verify(0, x, alpha.to(DEV), acm.SelectParams(**params), want=True)
+        np.testing.assert_array_equal(got.cpu().numpy(), ref["idx"])
+        _ffn_check(out, ref["out"], f"overlap {level}")
+        assert acm.stats_dict(stats)["n_eligible_pruned"] == ref["count"]
+    ctx.set_overlap(acm.OVERLAP_ANCHORS)
+    offsets = [0, 1, T // 2 + 1, T]
+    refs = [oracle.moe_verify(x[a:b], w["w_router"], w["router_bias"], w["gate_up"], w["down"], alpha.numpy()[a:b], k, oracle.SelectParams(),
+                              weighting=cfg.weighting, shared_gate_up=shared[0], shared_down=shared[1]) for a, b in zip(offsets, offsets[1:])]
+    out, got, _, _, _, _ = ctx.moe_verify_batch(0, x, offsets, alpha.to(DEV), acm.SelectParams(), want=True)
+    assert ctx.device_status() == acm.OK
+    np.testing.assert_array_equal(got.cpu().numpy(), np.concatenate([r["idx"] for r in refs]))
+    _ffn_check(out, np.concatenate([r["out"] for r in refs]), "batch")
     ctx.close()
 
 
