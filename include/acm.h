@@ -364,8 +364,7 @@ acm_status acm_expert_ffn_f32_noalloc(const float* x, int T, int hidden, int int
  * n_experts_streamed experts of a bf16 layer (hidden, inter) on `grid` CTAs deals its weight tiles, for inspection
  * and for tests of the plan's coverage.  n_anchor_first > 0 lists the plan of a launch that starts on that many
  * anchor experts (Eq. 5) before the rest of the set is known (their tiles, one per CTA, are segment 0).
- * (Launches of few nodes -- up to 2 to 32 by hidden, inter and whether there are shared experts -- have no such plan: tile i of the list goes to CTA
- * i mod grid, whole, together with its part of the down projection.)
+ * (Launches of few nodes are dealt differently: acm_ffn_plan_block.)
  * pieces [capacity][8] (host) receives, in each
  * CTA's execution order: CTA, segment, phase (1 = gate/up: 64 gate + 64 up rows x hidden; 2 = down: 128 output
  * rows), for gate/up whether the tile is given whole (1) or cut along K (0) (down: 0), the tile (gate/up: slot *
@@ -375,6 +374,17 @@ acm_status acm_expert_ffn_f32_noalloc(const float* x, int T, int hidden, int int
  * small (*n_pieces then tells how many there are). */
 acm_status acm_ffn_plan(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,
                         int32_t* pieces /*host*/, int capacity, int32_t* n_pieces /*host*/, int32_t* n_segments /*host*/);
+
+/* The same for a launch over n_nodes nodes (1..128; a batch: of all its blocks together) of a layer with n_shared shared
+ * experts (they are counted in n_experts_streamed too).  Where the layer's launches take the plan above at that many
+ * nodes, it is what acm_ffn_plan lists.  A launch of few nodes -- the line depends on hidden, inter and whether there are
+ * shared experts, and is never above 32 -- deals units instead: a gate/up tile together with the part of the down
+ * projection that its 64 features have, unit i of the list (the anchors' first) to CTA i mod grid, whole.  `pieces`
+ * then receives every pipeline stage: CTA, segment (1 = units that are known only with the rest of the set), phase 1 = a
+ * gate/up stage or 3 = a down stage, the constant 1 or the number of 128-row output tiles (1 or 2), the unit (slot *
+ * inter/64 + sub-tile), the first and one-past-last K-chunk of 128 K or output tile, and the expert slot. */
+acm_status acm_ffn_plan_block(int n_nodes, int n_shared, int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,
+                              int32_t* pieces /*host*/, int capacity, int32_t* n_pieces /*host*/, int32_t* n_segments /*host*/);
 
 /* The same for an MXFP4 layer (inter a multiple of 128): its kernel deals every tile whole. */
 acm_status acm_ffn_plan_mxfp4(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,

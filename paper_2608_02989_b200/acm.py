@@ -28,7 +28,7 @@ EXPORTS = [
     "acm_set_slot_pool", "acm_pool_stats", "acm_pool_plan",
     "acm_h2d_bytes", "acm_ffn_timing", "acm_ffn_time_ms", "acm_stage_timing", "acm_stage_times", "acm_launch_count", "acm_device_status", "acm_status_string",
     "acm_set_overlap", "acm_set_wait_limit", "acm_wait_report", "acm_inject_unpublished_wait",
-    "acm_offload_timing", "acm_offload_times", "acm_ffn_plan", "acm_ffn_plan_mxfp4", "acm_mxfp4_activation_pieces",
+    "acm_offload_timing", "acm_offload_times", "acm_ffn_plan", "acm_ffn_plan_block", "acm_ffn_plan_mxfp4", "acm_mxfp4_activation_pieces",
     "acm_expert_ffn_f32_noalloc",
 ]
 NOALLOC_MAX_FLOATS = 1 << 20
@@ -114,6 +114,7 @@ def load_library():
     lib.acm_set_overlap.argtypes = [c_void_p, c_int]
     lib.acm_ffn_plan_mxfp4.argtypes = [c_int] * 5 + [c_void_p, c_int, POINTER(c_int32), POINTER(c_int32)]
     lib.acm_mxfp4_activation_pieces.argtypes = [c_void_p, c_void_p, c_void_p]
+    lib.acm_ffn_plan_block.argtypes = [c_int] * 7 + [c_void_p, c_int, POINTER(c_int32), POINTER(c_int32)]
     lib.acm_ffn_plan.argtypes = [c_int] * 5 + [c_void_p, c_int, POINTER(c_int32), POINTER(c_int32)]
     lib.acm_offload_timing.argtypes = [c_void_p, c_int, c_int]
     lib.acm_offload_times.argtypes = [c_void_p, POINTER(ctypes.c_double), POINTER(c_int32)]
@@ -164,16 +165,22 @@ def node_weights(depth, p_table, beta=0.5, width_norm=True) -> torch.Tensor:
     return alpha
 
 
-def ffn_plan(n_experts_streamed, hidden, inter, grid, n_anchor_first=0, mxfp4=False):
-    """acm_ffn_plan (acm_ffn_plan_mxfp4) on the host -> (pieces [n, 8] int32 numpy array, number of segments); see include/acm.h."""
+def ffn_plan(n_experts_streamed, hidden, inter, grid, n_anchor_first=0, mxfp4=False, n_nodes=None, n_shared=0):
+    """acm_ffn_plan (acm_ffn_plan_mxfp4; acm_ffn_plan_block if n_nodes is given) on the host -> (pieces [n, 8] int32 numpy array,
+    number of segments); see include/acm.h."""
+    if mxfp4 and n_nodes is not None:
+        raise ValueError("an MXFP4 layer's plan does not depend on the number of nodes")
     import numpy as np
     cap = 1 << 16
     while True:
         buf = np.zeros((cap, 8), dtype=np.int32)
         n, nseg = c_int32(0), c_int32(0)
         lib = load_library()
-        rc = (lib.acm_ffn_plan_mxfp4 if mxfp4 else lib.acm_ffn_plan)(n_experts_streamed, n_anchor_first, hidden, inter, grid,
-                                         buf.ctypes.data_as(c_void_p), cap, byref(n), byref(nseg))
+        args = (n_experts_streamed, n_anchor_first, hidden, inter, grid, buf.ctypes.data_as(c_void_p), cap, byref(n), byref(nseg))
+        if n_nodes is not None:
+            rc = lib.acm_ffn_plan_block(n_nodes, n_shared, *args)
+        else:
+            rc = (lib.acm_ffn_plan_mxfp4 if mxfp4 else lib.acm_ffn_plan)(*args)
         if rc == ERR_NOMEM:
             cap = n.value
             continue

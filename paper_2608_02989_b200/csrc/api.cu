@@ -497,6 +497,35 @@ acm_status ensure_staging(acm_ctx* c) {
 }  // namespace
 
 namespace {
+// The stages of a launch of the small blocks' kernel, in each CTA's execution order.
+acm_status list_small_walk(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid, int32_t* pieces, int capacity,
+                           int32_t* n_pieces, int32_t* n_segments) {
+  if (!pieces || !n_pieces || !n_segments || capacity < 0) return ACM_ERR_INVALID;
+  if (n_experts_streamed < 1 || n_experts_streamed > kMaxSlots || n_anchor_first < 0 || n_anchor_first > n_experts_streamed ||
+      hidden < 128 || hidden % 128 != 0 || inter < 64 || inter % 64 != 0 || grid < 1 || grid > 1024)
+    return ACM_ERR_INVALID;
+  int n = 0;
+  auto add = [&](int cta, int seg, int phase, int flag, int tile, int a, int b, int aux) {
+    if (n < capacity) {
+      int32_t* q = pieces + static_cast<size_t>(8) * n;
+      q[0] = cta; q[1] = seg; q[2] = phase; q[3] = flag; q[4] = tile; q[5] = a; q[6] = b; q[7] = aux;
+    }
+    ++n;
+  };
+  for (int cta = 0; cta < grid; ++cta) {
+    const acm::plan::SmallWalk w(hidden, inter, cta);
+    for (int unit = cta; unit < n_experts_streamed * w.tpe; unit += grid) {
+      const int slot = unit / w.tpe, seg = n_anchor_first > 0 && slot >= n_anchor_first ? 1 : 0;
+      for (int i = 0, k = w.k_first; i < w.kc1; ++i, k = w.next_k(k)) add(cta, seg, 1, 1, unit, k, k + 1, slot);
+      for (int i = 0, j = w.j_first; i < w.n_down; ++i, j = w.next_j(j))
+        add(cta, seg, 3, w.out_tiles(j), unit, w.first_tile(j), w.first_tile(j) + w.out_tiles(j), slot);
+    }
+  }
+  *n_pieces = n;
+  *n_segments = n_anchor_first > 0 && n_anchor_first < n_experts_streamed ? 2 : 1;
+  return n <= capacity ? ACM_OK : ACM_ERR_NOMEM;
+}
+
 template <bool kUncut>
 acm_status list_plan(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid, int32_t* pieces,
                      int capacity, int32_t* n_pieces, int32_t* n_segments) {
@@ -1524,6 +1553,14 @@ acm_status acm_launch_count(acm_ctx* c, uint64_t* launches_out) {
 
 acm_status acm_ffn_plan(int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid, int32_t* pieces,
                         int capacity, int32_t* n_pieces, int32_t* n_segments) {
+  return list_plan<false>(n_experts_streamed, n_anchor_first, hidden, inter, grid, pieces, capacity, n_pieces, n_segments);
+}
+
+acm_status acm_ffn_plan_block(int n_nodes, int n_shared, int n_experts_streamed, int n_anchor_first, int hidden, int inter, int grid,
+                              int32_t* pieces, int capacity, int32_t* n_pieces, int32_t* n_segments) {
+  if (n_nodes < 1 || n_nodes > kWideNodes || n_shared < 0 || n_shared > kMaxShared) return ACM_ERR_INVALID;
+  if (small_block(n_nodes, hidden, inter, n_shared))
+    return list_small_walk(n_experts_streamed, n_anchor_first, hidden, inter, grid, pieces, capacity, n_pieces, n_segments);
   return list_plan<false>(n_experts_streamed, n_anchor_first, hidden, inter, grid, pieces, capacity, n_pieces, n_segments);
 }
 

@@ -100,6 +100,7 @@ using plan::Segment;
 using plan::SegRange;
 using plan::Plan;
 using plan::Sched;
+using plan::SmallWalk;
 using plan::make_range;
 using plan::cut_begin;
 using plan::plan_lane;
@@ -1747,7 +1748,9 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
     am[wd] = (p.li == 0 ? act & res : act & ~res) & p.only[wd];
     n_first += __popc(am[wd]);
   }
-  const int tpe = p.I / 64, kc1 = p.H / (kBK * kAtoms), h_tiles = p.H / kTileM, n_down = (h_tiles + 1) / 2;
+  static_assert(kBK * kAtoms == 128 && kTileM == 128, "SmallWalk");
+  const SmallWalk walk(p.H, p.I, cta);
+  const int tpe = walk.tpe, kc1 = walk.kc1, n_down = walk.n_down;
   const uint32_t b_atom_bytes = static_cast<uint32_t>(p.n_pad) * kBK * 2;
   int32_t* s_entry = bars->entry;
   // slots of the experts in m behind slot `base`, in ascending id
@@ -1793,9 +1796,6 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
     limit = bars->n_slots * tpe;
     return tile < limit;
   };
-  // The CTAs walk a tile's K-chunks and output rows from different ones on: in step, all would fetch the same hidden states and
-  // add into the same rows at the same time.
-  const int k_first = cta % kc1, j_first = cta % n_down;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ weights and hidden states
@@ -1824,7 +1824,7 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
         const int eidx = entry_idx(ent);
         const CUtensorMap* gu = pick_map(entry_src(ent), &maps.gate_up, &maps.shared_gate_up, &maps.staged_gate_up);
         const CUtensorMap* dn = pick_map(entry_src(ent), &maps.down, &maps.shared_down, &maps.staged_down);      // (slices: DownSlices)
-        int kk = k_first;
+        int kk = walk.k_first;
         if (pre && depth_open && !more) {
           depth_open = false;
           depth = ring_depth();
@@ -1847,16 +1847,16 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
           mbar_expect_tx(full, kABytes + kAtoms * b_atom_bytes);
           tma_load_5d(sa, gu, full, 0, ti * 64, 0, kk * kAtoms, eidx, pol_w);
           tma_load_3d(sa + kABytes, &x_map, full, 0, 0, kk * kAtoms, pol_x);
-          if (++kk == kc1) kk = 0;
+          kk = walk.next_k(kk);
           if (++s == kRing) { s = 0; par ^= 1u; }
         }
-        int jj = j_first;
+        int jj = walk.j_first;
         for (int j = 0; ok && j < n_down; ++j) {
           if (!(ok = wait_room())) break;
           const uint32_t full = smem_u32(&bars->full[s]);
           mbar_expect_tx(full, kABytes);
-          tma_load_4d(smem_u32(smem) + s * kStageBytes, dn, full, 0, jj * 2 * kTileM, ti, eidx, pol_w);
-          if (++jj == n_down) jj = 0;
+          tma_load_4d(smem_u32(smem) + s * kStageBytes, dn, full, 0, walk.first_tile(jj) * kTileM, ti, eidx, pol_w);
+          jj = walk.next_j(jj);
           if (++s == kRing) { s = 0; par ^= 1u; }
         }
       }
@@ -2058,7 +2058,7 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
       // weights of zero.)
       constexpr int kNodes = 8 / kSlotTiles;
       float2* list = bars->list[warp - 2];
-      int n_list = 0, jj = j_first;
+      int n_list = 0, jj = walk.j_first;
       for (int j0 = 0; j0 < n_down; j0 += kSlotTiles / 2) {
         if (!(ok = acc_wait())) break;
         tc_fence_after();
@@ -2078,10 +2078,10 @@ k_ffn_bf16_small(const __grid_constant__ FfnMaps maps, const __grid_constant__ C
         int last_at = 2 * n_down;      // (at an odd number of tiles the last stage holds one)
 #pragma unroll
         for (int st = 0; st < kSlotTiles / 2; ++st) {
-          dst[st] = p.out + jj * 2 * kTileM + row;
+          dst[st] = p.out + walk.first_tile(jj) * kTileM + row;
           if (j0 + st < n_down) {
-            if (2 * jj + 1 >= h_tiles) { whole = false; last_at = st; }
-            if (++jj == n_down) jj = 0;
+            if (walk.out_tiles(jj) == 1) { whole = false; last_at = st; }
+            jj = walk.next_j(jj);
           }
         }
         const uint32_t at = tmem_base + lane_addr + b * kSlotCols;

@@ -30,6 +30,7 @@
 // than a cut would, but a layer still less than with the kernel that cut them and expanded the weights to bf16 (4096 x 1536,
 // 64 nodes, 8 / 20 / 100 experts: 72 / 120 / 516 -> 62 / 93 / 424 us; hidden 1024 to 4096, inter 512 to 1536, 8 to 100
 // experts, 1 to 64 nodes: none slower).
+// A launch of the small blocks' kernel has no such plan: see SmallWalk.
 // (Measured and dropped, bf16: every tile whole with the CTAs that get one tile less taking down work early -- the last
 // round's experts then start their down projection too late; the leftover tiles after the whole rounds instead of
 // before them; the leftover tiles cut over the idle CTAs only.)
@@ -205,6 +206,21 @@ ACM_PLAN_FN void plan_lane(Plan& pl, int lane, int cta, int n_act, int tpe, int 
 #endif
   if (lane == 0) pl.n_seg = base + n;
 }
+
+// A launch of the small blocks' kernel: unit i of the work list -- a gate/up tile and its 64 features' part of the down projection,
+// numbered as the tiles above, the anchors' first -- goes to CTA i mod G, whole.  Its pipeline stages are kc1 gate/up stages (128 K
+// each) and then n_down down stages (two output tiles each, the last one of an odd number of tiles one).  The CTAs begin with
+// different ones: in step, all would fetch the same hidden states and add into the same rows at the same time.
+struct SmallWalk {
+  int tpe, kc1, h_tiles, n_down;
+  int k_first, j_first;      // the gate/up and the down stage that this CTA takes first, of every unit
+  ACM_PLAN_FN SmallWalk(int hidden, int inter, int cta)
+      : tpe(inter / 64), kc1(hidden / 128), h_tiles(hidden / 128), n_down((h_tiles + 1) / 2), k_first(cta % kc1), j_first(cta % n_down) {}
+  ACM_PLAN_FN int next_k(int k) const { return k + 1 == kc1 ? 0 : k + 1; }
+  ACM_PLAN_FN int next_j(int j) const { return j + 1 == n_down ? 0 : j + 1; }
+  ACM_PLAN_FN int first_tile(int j) const { return 2 * j; }                          // output tiles of down stage j
+  ACM_PLAN_FN int out_tiles(int j) const { return 2 * j + 1 < h_tiles ? 2 : 1; }
+};
 
 }  // namespace plan
 }  // namespace acm

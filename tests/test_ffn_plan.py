@@ -131,3 +131,48 @@ def test_mxfp4_plan_streams_every_stage_once_and_cuts_no_tile(H, I):
                     if len(set(dn[:, 7].tolist())) == 2 and len(rest):
                         rounds = -(-len(rest) // G)
                         assert dn[:, 7].max() * tpe <= n_pre * tpe + (rounds - 1) * G
+
+
+@pytest.mark.parametrize("H,I", [(128, 64), (256, 320), (384, 128), (1152, 512), (2048, 768), (4096, 128)])
+def test_small_launches_stream_every_stage_once_by_the_cta_that_made_the_activations(H, I):
+    """acm_ffn_plan_block at few nodes: units dealt i mod grid, each with all its gate/up stages before its down stages and in
+    the same CTA; every K-chunk and every output tile of every unit exactly once (odd numbers of output tiles, grids larger and
+    smaller than the list, anchor starts); neighbouring CTAs begin with different stages."""
+    tpe, kc1, h_tiles = I // 64, H // 128, H // 128
+    for G in (148, 147, 133, 7):
+        for n_act in (1, 2, 8, 13, 31, 132):
+            for n_pre in sorted({0, 1, min(n_act, 8), n_act}):
+                pieces, n_seg = acm.ffn_plan(n_act, H, I, G, n_pre, n_nodes=2)
+                assert n_seg == (2 if 0 < n_pre < n_act else 1)
+                gu, dn = np.zeros((n_act * tpe, kc1), dtype=np.int32), np.zeros((n_act * tpe, h_tiles), dtype=np.int32)
+                first, last = {}, {}
+                for cta, seg, phase, flag, unit, a, b, slot in pieces.tolist():
+                    assert cta == unit % G and slot == unit // tpe and seg == int(0 < n_pre <= slot)
+                    assert last.get(cta, -1) <= unit                # a CTA's units one after the other
+                    last[cta] = unit
+                    if phase == 1:
+                        assert flag == 1 and b == a + 1 and not dn[unit].any()
+                        first.setdefault(cta, a)
+                        gu[unit, a] += 1
+                    else:
+                        assert phase == 3 and flag == b - a and gu[unit].all() and a % 2 == 0
+                        dn[unit, a:b] += 1
+                assert (gu == 1).all() and (dn == 1).all()
+                assert all(first[c] == c % kc1 for c in first)
+
+
+@pytest.mark.parametrize("H,I,ns,limit", [(1024, 768, 0, 32), (1024, 768, 2, 32), (1024, 1024, 1, 24), (1024, 1536, 0, 16), (1536, 768, 0, 32),
+                                          (1536, 768, 1, 16), (2048, 640, 0, 24), (2048, 768, 0, 16), (2048, 832, 1, 8), (2048, 1024, 0, 2),
+                                          (1536, 1408, 0, 8), (4096, 512, 0, 16), (4096, 512, 1, 8), (4096, 768, 0, 8), (4096, 1536, 0, 2)])
+def test_the_plan_by_node_count_is_the_one_the_launch_takes(H, I, ns, limit):
+    """Up to the layer's line the stages of whole units (phase 3 among them), beyond it exactly what acm_ffn_plan lists."""
+    whole, n_seg = acm.ffn_plan(21, H, I, 140, 4)
+    for T in (1, limit, limit + 1, 33, 64, 128):
+        got, seg = acm.ffn_plan(21, H, I, 140, 4, n_nodes=T, n_shared=ns)
+        if T <= limit:
+            assert (got[:, 2] == 3).any() and seg == 2
+        else:
+            assert seg == n_seg and np.array_equal(got, whole)
+    for T, bad in ((0, 0), (129, 0), (8, -1), (8, 5)):
+        with pytest.raises(acm.AcmError):
+            acm.ffn_plan(21, H, I, 140, n_nodes=T, n_shared=bad)
