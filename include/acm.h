@@ -198,7 +198,11 @@ acm_status acm_route_restricted(acm_ctx* ctx, const float* logits, const uint32_
                                 int T, int32_t* idx, float* w, acm_stream stream);
 
 /* Stage 4 alone: y_t = sum_j w[t,j] * down_e( silu(gate_e x_t) * up_e x_t ), e = idx[t,j]
- * (+ shared experts with weight 1).  x [T,H], idx/w [T,k] -> out [T,H] float (overwritten). */
+ * (+ shared experts with weight 1).  x [T,H], idx/w [T,k] -> out [T,H] float (overwritten).
+ * Expert weights are taken to be finite.  One that is not makes the rows of the nodes that are routed to its expert
+ * non-finite; whether it reaches other nodes' rows too is not specified, here and in the fused calls (most launches give an
+ * expert's node columns a weight of zero where a node is not routed to it, and zero times infinity is NaN; launches of few
+ * nodes leave such nodes out).  No later call is affected. */
 acm_status acm_expert_ffn(acm_ctx* ctx, int layer, const void* x, int T, const int32_t* idx,
                           const float* w, float* out, acm_stream stream);
 

@@ -1231,3 +1231,30 @@ def test_given_routes_reach_the_weight_table(T, E, k):
         assert ctx.device_status() == acm.OK
         _ffn_check(out, oracle.expert_ffn(x, idx.numpy(), w.numpy(), w_["gate_up"], w_["down"]), "given routes")
     ctx.close()
+
+
+@pytest.mark.parametrize("T,H,I", [(8, 256, 128), (16, 2048, 128), (64, 256, 192)])
+def test_a_weight_that_is_not_finite_stays_in_its_call(T, H, I):
+    """Both sides of the line between the small blocks' kernel and the other one: an infinite value in one expert's tensors makes the
+    rows of the nodes routed to it non-finite, and the next call, on a layer without it, finds a clean workspace."""
+    cfg = wl.scaled(wl.CONFIGS[3], hidden=H, inter=I, n_experts=12, top_k=3, n_nodes=T, max_depth=4, zipf_bias=False)
+    ctx = _ctx(cfg, n_layers=2)
+    w, x = wl.layer_weights(cfg, 3, DEV), wl.hidden_states(cfg, 3, DEV)
+    _set_weights(ctx, w, 0)
+    every = torch.tensor(full_mask(12).view(np.int32), device=DEV)
+    clean, idx, wt, _, _ = ctx.moe_verify(0, x, None, None, mask_override=every, want=True)
+    ref = oracle.expert_ffn(x, idx.cpu().numpy(), wt.cpu().numpy(), w["gate_up"], w["down"])
+    _ffn_check(clean, ref, "before")
+    e = int(idx[0, 0])
+    routed = (idx == e).any(1).cpu()
+    for name, at in (("down", (e, 5, 7)), ("gate_up", (e, 3, 11))):
+        bad = {n: w[n].clone() for n in ("gate_up", "down")}
+        bad[name][at] = float("inf")
+        torch.cuda.synchronize()
+        ctx.set_layer_weights(1, w["w_router"], w["router_bias"], bad["gate_up"], bad["down"])
+        for o in (ctx.moe_verify(1, x, None, None, mask_override=every), ctx.expert_ffn(1, x, idx, wt)):
+            assert not torch.isfinite(o).all(1).cpu()[routed].any(), name
+        assert ctx.device_status() == acm.OK
+        _ffn_check(ctx.moe_verify(0, x, None, None, mask_override=every), ref, "fused call after")
+        _ffn_check(ctx.expert_ffn(0, x, idx, wt), ref, "FFN alone after")
+    ctx.close()
