@@ -292,6 +292,29 @@ def test_few_nodes_of_experts_beyond_the_small_kernels_line(T, H, I, ns):
     ctx.close()
 
 
+@pytest.mark.parametrize("T,H,I,ns", [(1, 1024, 192, 0), (16, 2048, 192, 1), (31, 1152, 128, 0)])
+def test_small_blocks_at_every_overlap_level(T, H, I, ns):
+    """The small blocks' kernel in its three instantiations: cooperative in plain order, dependent, started on the eligible set and on
+    the anchors; most of the eligible experts chosen by no node."""
+    E, k = 40, 4
+    cfg = wl.scaled(wl.CONFIGS[3], hidden=H, inter=I, n_experts=E, top_k=k, n_shared=ns, n_nodes=T, max_depth=4)
+    ctx = _ctx(cfg)
+    w, x, alpha = _block(cfg, 1)
+    _set_weights(ctx, w)
+    ref = oracle.moe_verify(x, w["w_router"], w["router_bias"], w["gate_up"], w["down"], alpha.numpy(), k, oracle.SelectParams(fixed_budget=33),
+                            weighting=cfg.weighting, shared_gate_up=w["shared_gate_up"], shared_down=w["shared_down"])
+    for level in (acm.OVERLAP_NONE, acm.OVERLAP_DEPENDENT, acm.OVERLAP_ELIGIBLE, acm.OVERLAP_ANCHORS, acm.OVERLAP_NONE):
+        ctx.set_overlap(level)
+        for _ in range(2):
+            out, got, _, mask, stats = ctx.moe_verify(0, x, alpha.to(DEV), acm.SelectParams(fixed_budget=33), want=True)
+            assert ctx.device_status() == acm.OK
+            np.testing.assert_array_equal(_u32(mask), ref["mask"])
+            np.testing.assert_array_equal(got.cpu().numpy(), ref["idx"])
+            _ffn_check(out, ref["out"], f"overlap {level}")
+            assert acm.stats_dict(stats)["n_activated"] == len(set(ref["idx"].ravel()) - {-1})
+    ctx.close()
+
+
 def test_expert_ffn_fp32_toy():
     cfg = wl.CONFIGS[1]
     w = wl.layer_weights(cfg, 0, DEV)

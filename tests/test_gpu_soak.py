@@ -240,6 +240,32 @@ def test_a_wait_that_runs_out_on_an_mxfp4_layer(T):
     ctx.close()
 
 
+@pytest.mark.parametrize("T,H,I,ns", [(1, 512, 256, 0), (16, 1152, 192, 2), (8, 1280, 256, 0), (16, 2048, 128, 2), (17, 512, 128, 0), (32, 1024, 192, 2)])
+def test_a_wait_that_runs_out_in_the_small_blocks_kernel(T, H, I, ns):
+    """The same for k_ffn_bf16_small, in each of its instantiations (three stages, five, 32 node columns): every CTA reports the
+    wait and leaves; with shared experts the roles have work when the flag goes up.  The fused call and the expert FFN alone that
+    follow are correct, so tensor memory and the barriers' state were left in order."""
+    cfg = wl.scaled(wl.CONFIGS[3], n_layers=1, hidden=H, inter=I, n_experts=32, n_shared=ns, n_nodes=T, max_depth=4)
+    w, x, alpha = wl.layer_weights(cfg, 0, DEV), wl.hidden_states(cfg, 0, DEV), torch.ones(T, device=DEV)
+    ctx = acm.Context.for_config(cfg, n_layers=1)
+    ctx.set_layer_weights(0, w["w_router"], w["router_bias"], w["gate_up"], w["down"], w["shared_gate_up"], w["shared_down"])
+    ctx.set_wait_limit(3_000_000)
+    for _ in range(3):
+        t0 = time.perf_counter()
+        ctx.inject_unpublished_wait(0, x)
+        assert ctx.device_status() == acm.ERR_TIMEOUT
+        assert time.perf_counter() - t0 < 0.5
+        report = ctx.wait_report()
+        assert len(report) == torch.cuda.get_device_properties(0).multi_processor_count and set(report) == {2}, report
+        out, idx, wt, _, _ = ctx.moe_verify(0, x, alpha, want=True)
+        alone = ctx.expert_ffn(0, x, idx, wt)
+        assert ctx.device_status() == acm.OK and set(ctx.wait_report()) == {0}
+        ref = oracle.expert_ffn(x, idx.cpu().numpy(), wt.cpu().numpy(), w["gate_up"], w["down"], w["shared_gate_up"], w["shared_down"])
+        for o in (out, alone):
+            assert float(np.abs(o.double().cpu().numpy() - ref).max()) <= 2e-2 * float(np.sqrt(np.mean(ref ** 2)))
+    ctx.close()
+
+
 def test_sequence_tags_coming_round_do_not_revive_old_words():
     """The words the kernels publish for one another carry the call's sequence number in 16 bits.  A batch call
     writes words for eight blocks; 65534 single-block calls later the tags come round, and a second batch call,
