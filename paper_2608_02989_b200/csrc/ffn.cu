@@ -2278,9 +2278,10 @@ cudaError_t launch_ffn_mxfp4(const FfnLaunch& L, cudaStream_t s) {
 namespace {
 // The small blocks' kernel for a launch.  Up to 1152 hidden features with three stages (120 KB): a CTA of the next call's router
 // kernel then fits beside it and has its weights by the time this launch is done, which such short launches gain more from than
-// from stages in flight.  us a layer, five stages -> three, with 8 / 21 / 40 experts: 1024 x 512, 1 node 17.0 / 24.4 / 33.7 -> 15.4 /
-// 22.8 / 31.6; 1024 x 1408, 16 nodes 29.2 / 40.1 / 63.3 -> 26.1 / 39.1 / 62.0; 1152 x 768, 1 node 18.4 / 30.0 / 44.3 -> 17.0 / 30.5 /
-// 43.5; 1536 x 768, 1 node 19.0 / 35.2 / 51.1 -> 19.0 / 35.9 / 51.7; 2048 x 768, 1 node 21.3 / 39.4 / 64.0 -> 22.3 / 41.8 / 66.4.
+// from stages in flight.  Three stages against five, mean / highest over 13 sets of 4 to 40 experts, 1 to 16 nodes, inter 512 to 1408:
+// hidden 768 0.92 to 0.98 / 1.02, 1024 0.91 to 0.99 / 1.05, 1152 0.92 to 0.99 / 1.04; beyond the line 1280 0.93 to 0.99 / 1.05, 1536
+// 0.96 to 1.00 / 1.06.  us a layer, five -> three, with 8 / 21 / 40 experts: 1024 x 512, 1 node 17.0 / 24.4 / 33.7 -> 15.4 / 22.8 / 31.6;
+// 1024 x 1408, 16 nodes 29.2 / 40.1 / 63.3 -> 26.1 / 39.1 / 62.0; 2048 x 768, 1 node 21.3 / 39.4 / 64.0 -> 22.3 / 41.8 / 66.4.
 // (Six stages: 22.1 / 40.6 / 67.4 there.  The router kernel's CTAs without their request for 104 KB, so that they fit beside five
 // stages: they pile up on the SMs that are free first, 22.7 / 42.3 / 66.7.)
 struct SmallKernel {
